@@ -573,8 +573,8 @@ void ctx_trim(awpm_ctx *c)
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
                       &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom,    &c->gckey,
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,    &c->gtdead,
-                      &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_cmax,
-                      &c->wt_rmax, &c->wt_stage, &c->mroot,    &c->mrpar,    &c->mfront,
+                      &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_max,
+                      &c->wt_scale, &c->wt_stage, &c->mroot,   &c->mrpar,    &c->mfront,
                       &c->mnext,   &c->mroff,    &c->mtend,    &c->mtouch,
                       &c->mstage,  &c->mcolof,   &c->mtiles,   &c->rowsig,   &c->trowptr,
                       &c->rs_k0,   &c->rs_k1,    &c->rs_v0,    &c->rs_v1,    &c->rs_hist,
@@ -661,7 +661,7 @@ void teardown_ctx(awpm_ctx *c)
                       &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom,    &c->gckey,
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,
                       &c->gtdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
-                      &c->wt_cmax, &c->wt_rmax,  &c->wt_stage,
+                      &c->wt_max,  &c->wt_scale, &c->wt_stage,
                       &c->mroot,   &c->mrpar,    &c->mfront,   &c->mnext,    &c->mroff,
                       &c->mtend,   &c->mtouch,   &c->mstage,   &c->mcolof,
                       &c->mtiles,  &c->rowsig,   &c->trowptr,  &c->rs_k0,    &c->rs_k1,
@@ -1623,8 +1623,10 @@ int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t 
     if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!rowidx || !values || !weight_out)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
-    AWPM_TRY(ensure(c, c->wt_cmax, sizeof(double) * n));
-    AWPM_TRY(ensure(c, c->wt_rmax, sizeof(unsigned long long) * n));
+    AWPM_TRY(ensure(c, c->wt_max, sizeof(unsigned long long) * n));
+    AWPM_TRY(ensure(c, c->wt_scale, sizeof(Scale) * n));
+    AWPM_TRY(ensure(c, c->tile_col, sizeof(int32_t) * ((size_t)ntiles + 1)));
+    AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
     double *dout = weight_out;
     if (l_out != 1) {
@@ -1641,8 +1643,10 @@ int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t 
     AWPM_TRY(stage_in(c, c->s_rowidx, rowidx, (size_t)nnz, l_rowidx, &wk.rowidx));
     AWPM_TRY(stage_in(c, c->s_w, values, (size_t)nnz, l_a, &wk.wt_a));
     wk.wt_out = dout;
-    wk.wt_cmax = (double *)c->wt_cmax.p;
-    wk.wt_rmax = (unsigned long long *)c->wt_rmax.p;
+    wk.wt_max = (unsigned long long *)c->wt_max.p;
+    wk.wt_scale = (Scale *)c->wt_scale.p;
+    wk.tile_col = (int32_t *)c->tile_col.p;
+    wk.starts = (uint32_t *)c->starts.p;
     wk.wt_mode = mode;
     wk.ctl = (Ctl *)c->ctl.p;
     CUDA_TRY(cudaMemcpyAsync(c->d_work.p, c->h_work, sizeof(Work), cudaMemcpyHostToDevice,

@@ -122,7 +122,7 @@ struct awpm_ctx {
     awpm::DevBuf gckey, gcpos, grkey, grcol, gtdead;  // greedy matching records
     awpm::DevBuf gmate;                       // greedy start of awpm_improve_ctx
     awpm::DevBuf psel, pslive, pstaken, psused;  // greedy (Pettie-Sanders) selection
-    awpm::DevBuf wt_cmax, wt_rmax, wt_stage;     // weights from matrix values
+    awpm::DevBuf wt_max, wt_scale, wt_stage;     // weights from matrix values
     awpm::DevBuf mroot, mrpar, mfront, mnext, mroff, mtend, mtouch, mstage,
         mcolof, mtiles;  // maximum matching
     awpm::DevBuf rowsig, trowptr, rs_k0, rs_k1, rs_v0, rs_v1, rs_hist, rs_sums;  // row marking

@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "awpm.h"
+#include "awpm_fixed.h"
 
 namespace awpm {
 
@@ -180,12 +181,13 @@ struct Work {
     uint32_t *pslive;
     uint32_t *pstaken;
     uint32_t *psused;
-    // weights from matrix values: values, output, column maxima, row maxima
-    // (bit patterns of positive doubles), mode (0 scaled magnitude, 1 its log)
+    // weights from matrix values: values, output, the columns' and then the
+    // rows' maxima (bit patterns of positive doubles), the same with their
+    // reciprocals, mode (0 scaled magnitude, 1 its log)
     const double *wt_a;
     double *wt_out;
-    double *wt_cmax;
-    unsigned long long *wt_rmax;
+    unsigned long long *wt_max;
+    Scale *wt_scale;
     int32_t wt_mode;
     int32_t wt_pad;
     // maximum cardinality matching: tree of a column, column that reached a
@@ -270,6 +272,8 @@ void launch_greedy_select_begin(const Work *d, const Shape &sh, bool graph,
 void launch_greedy_select_round(const Work *d, const Shape &sh, bool graph,
                                 cudaGraphConditionalHandle h, Sink &k);
 void launch_greedy_select_end_and_flip(const Work *d, const Shape &sh, Sink &k);
+// The column-pointer check with the start marks (k_check_mark).
+void launch_check_mark(const Work *d, const Shape &sh, Sink &k);
 // Weights from matrix values (equilibration, Options A / B).
 void launch_weights(const Work *d, const Shape &sh, Sink &k);
 // Maximum cardinality matching: load and check the starting matching; start

@@ -1,0 +1,78 @@
+"""Weights from matrix values at the edges of the entry-parallel kernels
+(needs a GPU): empty columns, columns longer than a tile, sizes around tile
+ends, values and quotients outside the normal numbers."""
+import numpy as np
+import pytest
+
+from paper_1801_09809_gb300 import awpm
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_09809_gb300 import build
+    build.build()
+    c = awpm.awpm_create(device=0)
+    yield c
+    awpm.awpm_destroy(c)
+
+
+def matrix(degrees, seed, span):
+    """Random rows, `degrees[j]` per column; values 10^U(-span, min(span, 308))."""
+    rng = np.random.default_rng(seed)
+    n = len(degrees)
+    colptr = np.zeros(n + 1, np.int32)
+    np.cumsum(degrees, out=colptr[1:])
+    rows = [np.sort(rng.choice(n, d, replace=False)) for d in degrees]
+    rowidx = np.concatenate(rows).astype(np.int32) if rows else np.zeros(0, np.int32)
+    a = 10.0 ** rng.uniform(-span, min(span, 308), rowidx.size) * rng.choice([-1.0, 1.0], rowidx.size)
+    a[a == 0.0] = 5e-324
+    return n, colptr, rowidx, a
+
+
+def reference(n, colptr, rowidx, a, mode):
+    col = np.repeat(np.arange(n), np.diff(colptr))
+    with np.errstate(all="ignore"):
+        cm = np.zeros(n)
+        np.maximum.at(cm, col, np.abs(a))
+        v = np.abs(a) / cm[col]
+        rm = np.zeros(n)
+        np.maximum.at(rm, rowidx, v)
+        x = v / rm[rowidx]
+        return np.log(x) if mode else x
+
+
+CASES = {
+    "empty_columns": [0, 0, 3, 0, 31, 32, 33, 0, 1, 0, 0, 64, 65, 0, 0, 1] + [0, 1, 2] * 40,
+    "hub": [200] + [1] * 199,
+    "one_tile": [4] * 8,
+    "one_past": [4] * 8 + [1],
+    "one": [1],
+    "all_but_one_empty": [0] * 50 + [37] + [0] * 49,
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("span", [2, 300, 323])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_edges(ctx, name, span, mode):
+    import torch
+    n, colptr, rowidx, a = matrix(CASES[name], 7 + span, span)
+    want = reference(n, colptr, rowidx, a, mode)
+    for in_place in (False, True):
+        cp, ri, av = (torch.from_numpy(x).cuda() for x in (colptr, rowidx, a))
+        out = av if in_place else torch.empty_like(av)
+        awpm.awpm_weights(ctx, n, cp, ri, av, mode, out)
+        got = out.cpu().numpy()
+        if mode == 0:
+            assert np.array_equal(got, want, equal_nan=True)
+        else:
+            # numpy's logarithm is within an ulp of the exact value, the
+            # library's within one too
+            fine = np.isfinite(want)
+            assert np.array_equal(got[~fine], want[~fine], equal_nan=True)
+            assert np.all(np.abs(got[fine] - want[fine]) <= 2 * np.spacing(np.abs(want[fine])))
