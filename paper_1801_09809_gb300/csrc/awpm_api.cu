@@ -140,6 +140,21 @@ bool bloom_enabled()
     return on;
 }
 
+// Tiles from which a solve's later passes are incremental (the environment
+// variable AWPM_INC overrides it, a tuning knob: 0 never, 1 always; results
+// are the same either way).
+constexpr int32_t kIncTiles = 98304;
+int32_t inc_min_tiles()
+{
+    static const int32_t least = [] {
+        const char *v = getenv("AWPM_INC");
+        if (v && (v[0] == '0' || v[0] == '1') && v[1] == 0)
+            return v[0] == '0' ? 0x7fffffff : 0;
+        return kIncTiles;
+    }();
+    return least;
+}
+
 int code_of(unsigned err)
 {
     return awpm_code_of_bits(err);
@@ -174,6 +189,59 @@ Shape shape_of(const awpm_ctx *c, bool batch, int lookup, bool wide, int32_t nti
     return sh;
 }
 
+// Append one pass to `sb` (the search, the selection and the flip, which
+// decides whether another pass runs: handle h).  The greedy selection's rounds
+// are a WHILE node nested in it.
+int add_pass(const Work *d, const Shape &sh, bool first, cudaGraphConditionalHandle h, Sink &sb)
+{
+    cudaError_t e;
+    if (first || !sh.inc)
+        launch_search(d, sh, sb);
+    else
+        launch_search_inc(d, sh, sb);
+    if (sh.select == AWPM_SELECT_GREEDY) {
+        cudaGraphConditionalHandle h2;
+        cudaGraphNodeParams cp2 = {cudaGraphNodeTypeConditional};
+        cudaGraphNode_t n_inner;
+        if ((e = cudaGraphConditionalHandleCreate(&h2, sb.graph, 0, 0)) != cudaSuccess) {
+            note_cuda_error(e, "inner conditional handle", __LINE__);
+            return AWPM_ERR_CUDA;
+        }
+        launch_greedy_select_begin(d, sh, true, h2, sb);
+        cp2.conditional.handle = h2;
+        cp2.conditional.type = cudaGraphCondTypeWhile;
+        cp2.conditional.size = 1;
+        if (sb.err != cudaSuccess ||
+            (e = cudaGraphAddNode(&n_inner, sb.graph, &sb.last, nullptr, 1, &cp2)) !=
+                cudaSuccess) {
+            note_cuda_error(sb.err != cudaSuccess ? sb.err : e, "inner conditional node",
+                            __LINE__);
+            return AWPM_ERR_CUDA;
+        }
+        Sink sr;
+        sr.graph = cp2.conditional.phGraph_out[0];
+        launch_greedy_select_round(d, sh, true, h2, sr);
+        if (sr.err != cudaSuccess) {
+            note_cuda_error(sr.err, "selection round nodes", __LINE__);
+            return AWPM_ERR_CUDA;
+        }
+        sb.last = n_inner;
+        launch_greedy_select_end_and_flip(d, sh, sb);
+    } else if (!sh.batch) {
+        // the flip's last block ends the pass (no control kernel)
+        launch_select_flip_control_graph(d, sh, h, sb);
+    } else {
+        launch_select_and_flip(d, sh, sb);
+    }
+    if (sh.batch || sh.select == AWPM_SELECT_GREEDY)
+        launch_control(d, sh, true, h, sb);
+    if (sb.err != cudaSuccess) {
+        note_cuda_error(sb.err, "pass nodes", __LINE__);
+        return AWPM_ERR_CUDA;
+    }
+    return AWPM_OK;
+}
+
 int ilog2(int64_t x)
 {
     int l = 0;
@@ -185,7 +253,8 @@ int ilog2(int64_t x)
 }
 
 // The solve graph of one launch shape: initialisation, WHILE{pass}, final
-// sum, assembled node by node (no stream capture).
+// sum, assembled node by node (no stream capture).  With incremental passes
+// the first pass, whose search is another kernel, stands before the WHILE.
 int build_graph(awpm_ctx *c, const Shape &sh, cudaGraphExec_t *out)
 {
     const Work *d = (const Work *)c->d_work.p;
@@ -223,58 +292,22 @@ int build_graph(awpm_ctx *c, const Shape &sh, cudaGraphExec_t *out)
     cp.conditional.handle = h;
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
+    if (sh.inc) {
+        Sink s1;
+        s1.graph = top;
+        s1.last = n_init;
+        if ((rc = add_pass(d, sh, true, h, s1)) != AWPM_OK)
+            goto done;
+        n_init = s1.last;
+    }
     if ((e = cudaGraphAddNode(&n_cond, top, &n_init, nullptr, 1, &cp)) != cudaSuccess) {
         note_cuda_error(e, "conditional node", __LINE__);
         rc = AWPM_ERR_CUDA;
         goto done;
     }
     sb.graph = cp.conditional.phGraph_out[0];
-    launch_search(d, sh, sb);
-    if (sh.select == AWPM_SELECT_GREEDY) {
-        // the selection's rounds: a WHILE node nested in the pass body
-        cudaGraphConditionalHandle h2;
-        cudaGraphNodeParams cp2 = {cudaGraphNodeTypeConditional};
-        cudaGraphNode_t n_inner;
-        if ((e = cudaGraphConditionalHandleCreate(&h2, sb.graph, 0, 0)) != cudaSuccess) {
-            note_cuda_error(e, "inner conditional handle", __LINE__);
-            rc = AWPM_ERR_CUDA;
-            goto done;
-        }
-        launch_greedy_select_begin(d, sh, true, h2, sb);
-        cp2.conditional.handle = h2;
-        cp2.conditional.type = cudaGraphCondTypeWhile;
-        cp2.conditional.size = 1;
-        if (sb.err != cudaSuccess ||
-            (e = cudaGraphAddNode(&n_inner, sb.graph, &sb.last, nullptr, 1, &cp2)) !=
-                cudaSuccess) {
-            note_cuda_error(sb.err != cudaSuccess ? sb.err : e, "inner conditional node",
-                            __LINE__);
-            rc = AWPM_ERR_CUDA;
-            goto done;
-        }
-        Sink sr;
-        sr.graph = cp2.conditional.phGraph_out[0];
-        launch_greedy_select_round(d, sh, true, h2, sr);
-        if (sr.err != cudaSuccess) {
-            note_cuda_error(sr.err, "selection round nodes", __LINE__);
-            rc = AWPM_ERR_CUDA;
-            goto done;
-        }
-        sb.last = n_inner;
-        launch_greedy_select_end_and_flip(d, sh, sb);
-    } else if (!sh.batch) {
-        // the flip's last block ends the pass (no control kernel)
-        launch_select_flip_control_graph(d, sh, h, sb);
-    } else {
-        launch_select_and_flip(d, sh, sb);
-    }
-    if (sh.batch || sh.select == AWPM_SELECT_GREEDY)
-        launch_control(d, sh, true, h, sb);
-    if (sb.err != cudaSuccess) {
-        note_cuda_error(sb.err, "pass body nodes", __LINE__);
-        rc = AWPM_ERR_CUDA;
+    if ((rc = add_pass(d, sh, false, h, sb)) != AWPM_OK)
         goto done;
-    }
     if ((e = cudaGraphAddChildGraphNode(&n_final, top, &n_cond, 1, g_final)) != cudaSuccess ||
         (e = cudaGraphInstantiate(out, top, 0)) != cudaSuccess) {
         note_cuda_error(e, "graph instantiation", __LINE__);
@@ -486,7 +519,10 @@ int run_timed(awpm_ctx *c, const Shape &sh, int max_passes, int *passes_enqueued
         NvtxRange pass_range("pass");
         AWPM_TRY(ensure_timing_events(c, (size_t)t + 1));
         CUDA_TRY(cudaEventRecord(c->tev[2 * t], s));
-        launch_search(d, sh, k);
+        if (t > 0 && sh.inc)
+            launch_search_inc(d, sh, k);
+        else
+            launch_search(d, sh, k);
         CUDA_TRY(cudaEventRecord(c->tev[2 * t + 1], s));
         if (sh.select == AWPM_SELECT_GREEDY) {
             // the selection's rounds, driven from the host by the count of
@@ -540,6 +576,37 @@ std::map<int, awpm_ctx *> g_default;
 
 namespace awpm {
 
+// Layout of the incremental passes' buffer (byte offsets, each 256-byte
+// aligned): entry bits twice, old rows, and two sets of bitmaps.
+struct IncLayout {
+    size_t found, pos, mc_old, small[2], large[2], full[2], posi[2], mark[2], bytes;
+    int32_t map_bits;  // of the large folded bitmap (0: none)
+    IncLayout(int32_t n, int32_t ntiles)
+    {
+        size_t at = 0;
+        auto take = [&at](size_t b) {
+            const size_t o = at;
+            at += (b + 255) / 256 * 256;
+            return o;
+        };
+        map_bits = 0;
+        if (n > kMapSmallBits)
+            for (map_bits = kMapSmallBits; map_bits < n && map_bits < kMapLargeBits;)
+                map_bits *= 2;
+        found = take(4 * ((size_t)ntiles + 1));
+        pos = take(4 * ((size_t)ntiles + 1));
+        mc_old = take(4 * (size_t)n);
+        for (int x = 0; x < 2; ++x) {
+            small[x] = take(kMapSmallBits / 8);
+            large[x] = take((size_t)map_bits / 8);
+            full[x] = take(4 * ((size_t)n / 32 + 2));
+            posi[x] = take(4 * ((size_t)n / 32 + 2));
+            mark[x] = take(4 * ((size_t)ntiles / 32 + 1));
+        }
+        bytes = at;
+    }
+};
+
 size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, int select)
 {
     const size_t N = (size_t)n, Z = (size_t)nnz, T = Z / kTile + 1;
@@ -556,6 +623,7 @@ size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, in
         b += 4 * (N + 1) + 12 * Z + 8 * N;
     if (select == AWPM_SELECT_GREEDY)  // selection records and three bitmaps
         b += sizeof(Sel) * N + 3 * 4 * (N / 32 + 1);
+    b += IncLayout(n, (int32_t)T).bytes;
     return b + b / 8;
 }
 
@@ -571,7 +639,7 @@ void ctx_trim(awpm_ctx *c)
                       &c->wpart,   &c->htab,     &c->b_noff,   &c->b_colmat, &c->b_tilemat,
                       &c->b_tlist, &c->b_i32,    &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
-                      &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom,    &c->gckey,
+                      &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,    &c->gckey,
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,    &c->gtdead,
                       &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_max,
                       &c->wt_scale, &c->wt_stage, &c->mroot,   &c->mrpar,    &c->mfront,
@@ -602,6 +670,7 @@ int setup_ctx(awpm_ctx *c, const awpm_options *opt)
     c->device = dev;
     CUDA_TRY(cudaSetDevice(dev));
     CUDA_TRY(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev));
+    CUDA_TRY(search_inc_setup());
     c->search_wide = default_search_wide();
     for (int b = 0; b < 2; ++b)
         for (int p = 0; p < 2; ++p) {
@@ -639,10 +708,11 @@ void teardown_ctx(awpm_ctx *c)
             for (int p = 0; p < 2; ++p)
                 for (int v = 0; v < 2; ++v)
                     for (int q = 0; q < 2; ++q)
-                        if (c->g_exec[b][h][p][v][q]) {
-                            cudaGraphExecDestroy(c->g_exec[b][h][p][v][q]);
-                            c->g_exec[b][h][p][v][q] = nullptr;
-                        }
+                        for (cudaGraphExec_t &g : c->g_exec[b][h][p][v][q])
+                            if (g) {
+                                cudaGraphExecDestroy(g);
+                                g = nullptr;
+                            }
     for (int v = 0; v < 2; ++v) {
         if (c->g_greedy[v]) {
             cudaGraphExecDestroy(c->g_greedy[v]);
@@ -658,7 +728,7 @@ void teardown_ctx(awpm_ctx *c)
                       &c->ctl,     &c->wpart,    &c->htab,     &c->b_noff,   &c->b_colmat,
                       &c->b_tilemat, &c->b_tlist, &c->b_i32,  &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
-                      &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom,    &c->gckey,
+                      &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,    &c->gckey,
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,
                       &c->gtdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
                       &c->wt_max,  &c->wt_scale, &c->wt_stage,
@@ -802,12 +872,33 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
         AWPM_TRY(ensure(c, c->psused, sizeof(uint32_t) * ((size_t)n / 32 + 1)));
     }
 
+    // Passes after the first search only what the last flips affect, in single
+    // solves (a batched solve's passes walk the running matrices' tiles) of at
+    // least kIncTiles tiles: below that a whole search is so short that the
+    // incremental form's kernel (its bitmaps, one block per SM) costs more.
+    // Whole searches against incremental passes, ms per solve: 27-point stencil
+    // 0.87 / 0.95 at 0.5 M entries, 1.43 / 1.27 at 2.1 M, 2.16 / 1.79 at 4.2 M,
+    // 14.8 / 6.8 at 23 M; 5-point stencil 0.40 / 0.43 at 2.1 M, 0.66 / 0.65 at
+    // 4.2 M; banded 0.66 / 0.73 and 1.02 / 1.03; R-MAT 0.24 / 0.25 and 0.40 /
+    // 0.39.  Where the budget or the device has no room for them, every pass
+    // searches all.
+    Shape sh = shape_of(c, count > 0, lookup, wide, ntiles);
+    const IncLayout il(n, ntiles);
+    if (count == 0 && !r.search_only && max_passes > 1 && ntiles >= inc_min_tiles()) {
+        const bool injected = c->fail_after == 0;
+        const int rc = ensure(c, c->incbuf, il.bytes);
+        if (rc == AWPM_ERR_OOM && injected)
+            return rc;
+        sh.inc = rc == AWPM_OK;
+        sh.large = sh.inc && il.map_bits > 0;
+    }
+
     // the solve graph of this launch shape, built once (before the timed span)
-    const Shape sh = shape_of(c, count > 0, lookup, wide, ntiles);
     cudaGraphExec_t gexec = nullptr;
     if (!r.search_only && !timed) {
         cudaGraphExec_t &g = c->g_exec[count > 0 ? 1 : 0][lookup_slot(lookup)]
-                                      [wide ? 1 : 0][sh.search_waves - 1][sh.select];
+                                      [wide ? 1 : 0][sh.search_waves - 1][sh.select]
+                                      [sh.large ? 2 : sh.inc ? 1 : 0];
         if (!g)
             AWPM_TRY(build_graph(c, sh, &g));
         gexec = g;
@@ -855,10 +946,18 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
     wk.dsel = (Sel *)c->dsel.p;
     {
         // solves with Step D's selection (single or batched) leave the
-        // records empty: every pass's flip clears the records of its winners
+        // Step-C records empty: every pass's flip clears the records of its
+        // winners (incremental passes: the last one, which has none); the
+        // Step-D records they leave are of older epochs
         const bool keeps_clean = !r.search_only && !ps;
-        wk.rec_clean = keeps_clean && (int64_t)n <= c->rec_clean ? 1 : 0;
-        pd.rec_clean_after = keeps_clean ? std::max<int64_t>(n, c->rec_clean) : 0;
+        wk.rec_clean = keeps_clean && (int64_t)n <= c->rec_clean &&
+                               c->sel_epoch + max_passes < 0x7fffffff
+                           ? 1
+                           : 0;
+        pd.rec_clean_after = keeps_clean ? std::max<int64_t>(n, wk.rec_clean ? c->rec_clean : 0) : 0;
+        pd.rec_clean_capped = sh.inc ? 0 : pd.rec_clean_after;
+        pd.epoch0 = wk.rec_clean ? c->sel_epoch : 0;
+        wk.epoch0 = (int32_t)pd.epoch0;
         c->rec_clean = 0;
     }
     wk.winbits = (uint32_t *)c->winbits.p;
@@ -867,6 +966,21 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
     wk.starts = (uint32_t *)c->starts.p;
     wk.ctl = (Ctl *)c->ctl.p;
     wk.wpart = (double *)c->wpart.p;
+    if (sh.inc) {
+        unsigned char *p = (unsigned char *)c->incbuf.p;
+        wk.inc = 1;
+        wk.map_bits = il.map_bits;
+        wk.foundbits = (uint32_t *)(p + il.found);
+        wk.posbits = (uint32_t *)(p + il.pos);
+        wk.mc_old = (int32_t *)(p + il.mc_old);
+        for (int x = 0; x < 2; ++x) {
+            wk.map_small[x] = (uint32_t *)(p + il.small[x]);
+            wk.map_large[x] = (uint32_t *)(p + il.large[x]);
+            wk.colfull[x] = (uint32_t *)(p + il.full[x]);
+            wk.colpos[x] = (uint32_t *)(p + il.posi[x]);
+            wk.tilemark[x] = (uint32_t *)(p + il.mark[x]);
+        }
+    }
     if (count > 0) {
         BatchWork &bw = wk.bw;
         bw.count = count;
@@ -987,7 +1101,8 @@ int ctx_finish(awpm_ctx *c, awpm_stats *st, awpm_stats *per_matrix)
     const int rc = code_of(h.err);
     if (rc != AWPM_OK)
         return rc;
-    c->rec_clean = pd.rec_clean_after;
+    c->rec_clean = h.converged ? pd.rec_clean_after : pd.rec_clean_capped;
+    c->sel_epoch = pd.epoch0 + h.iterations;
     double ms_search = 0.0;
     if (pd.timed) {
         for (int t = 0; t < h.iterations && t < pd.passes_enqueued; ++t) {

@@ -72,7 +72,11 @@ struct Pending {
     bool active = false;
     int32_t n = 0, nnz = 0, count = 0, lookup = 0;
     bool search_only = false, timed = false, trivial = false;
-    int64_t rec_clean_after = 0;  // the context's rec_clean once the solve ends without error
+    // the context's rec_clean once the solve ends without error: after a
+    // solve stopped by max_iters (rec_clean_capped) the incremental passes may
+    // leave records behind
+    int64_t rec_clean_after = 0, rec_clean_capped = 0;
+    int64_t epoch0 = 0;
     int passes_enqueued = 0;
     std::vector<int32_t> n_off;  // host copy of the batch offsets
     int tune_cfg = -1;           // autotuner trial of this solve, or -1
@@ -114,11 +118,14 @@ struct awpm_ctx {
     // while a solve is in flight, after an error, and when the buffers are
     // reallocated or released.
     int64_t rec_clean = 0;
+    // the last epoch used in dsel while rec_clean holds
+    int64_t sel_epoch = 0;
     int search_bps[2][3][2] = {};  // [batch][lookup slot][wide]
     bool search_wide = true;      // default when the lookup is given explicitly
     // per-solve device workspace
     awpm::DevBuf mc, mr, wm, rr, rsig, colsig, best, dsel, tile_col, starts, ctl, wpart, htab;
     awpm::DevBuf winbits, wkey, bloom;
+    awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
     awpm::DevBuf gckey, gcpos, grkey, grcol, gtdead;  // greedy matching records
     awpm::DevBuf gmate;                       // greedy start of awpm_improve_ctx
     awpm::DevBuf psel, pslive, pstaken, psused;  // greedy (Pettie-Sanders) selection
@@ -139,7 +146,8 @@ struct awpm_ctx {
     std::vector<cudaEvent_t> tev;     // timing pairs of the timed loop
     std::vector<cudaEvent_t> flagev;  // ring of the timed loop
     // one instantiated graph per [batch][lookup slot][wide][search waves - 1][select]
-    cudaGraphExec_t g_exec[2][3][2][2][2] = {};
+    // [passes after the first: whole searches, incremental, incremental large]
+    cudaGraphExec_t g_exec[2][3][2][2][2][3] = {};
     cudaGraphExec_t g_greedy[2] = {};  // greedy matching, [search waves - 1] of the shape
     cudaGraphExec_t g_mcm[2] = {};     // maximum matching, [search waves - 1] of the shape
     std::map<uint64_t, awpm::TuneEntry> tune;  // autotuner state per problem class

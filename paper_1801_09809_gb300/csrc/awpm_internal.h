@@ -77,11 +77,13 @@ struct alignas(16) Off {
     int32_t pad;
 };
 
-// Step-D selection at a key column k (Algorithm 6): best gain and its root j.
+// Step-D selection at a key column k (Algorithm 6): best gain and its root j,
+// and the pass that wrote it (Work::epoch0 + passes run + 1): a record of
+// another pass counts as empty, so none has to be cleared.
 struct alignas(16) Sel {
     double g;
     int32_t j;
-    int32_t pad;
+    int32_t epoch;
 };
 
 // Device-resident control block of one solve.
@@ -106,6 +108,11 @@ struct Ctl {
     unsigned long long candidates;   // Step A requests (i > m_j)
     unsigned long long found;        // closing edge present
     unsigned long long positive;     // closing edge present and g > 0
+    // incremental passes: this pass's changes of the three counts (signed),
+    // the counts of the last pass, and the cycles it flipped
+    unsigned long long d_candidates, d_found, d_positive;
+    unsigned long long cur_candidates, cur_found, cur_positive;
+    unsigned long long last_flips;
     double weight_in;
     double weight_out;
 };
@@ -135,6 +142,14 @@ struct BatchWork {
 // Tile whose nonzeros all belong to one matrix.
 constexpr int32_t kTileSingle = (int32_t)0x80000000;
 
+// Rows whose mate the last pass changed, as folded bitmaps: bit r mod 2^17 of
+// the small one, bit r mod 2^k of the large one (2^k >= n, at most 2^20; only
+// kept for n > 2^17, and then searched instead of the small one after a pass
+// of more than kSmallFlips flips).
+constexpr int kMapSmallBits = 1 << 17;
+constexpr int kMapLargeBits = 1 << 20;
+constexpr unsigned kSmallFlips = 1024;
+
 // Descriptor of one solve.  It lives in device memory and every kernel reads
 // it from there, so launch configurations do not depend on the problem and
 // one instantiated CUDA graph serves every problem of a context: a new
@@ -146,6 +161,10 @@ struct Work {
     int32_t max_passes;
     int32_t lookup;     // AWPM_LOOKUP_BSEARCH, _HASH or _ROWMARK
     int32_t rec_clean;  // the Step-C and Step-D records of columns [0, n) are all empty
+    int32_t inc;        // passes after the first search only what the last flips affect
+    int32_t epoch0;     // Step-D records of this solve's passes: epochs epoch0 + 1, ...
+    int32_t map_bits;   // bits of the large folded bitmap (0: none kept)
+    int32_t inc_pad;
     const int32_t *colptr;
     const int32_t *rowidx;
     const double *w;
@@ -161,7 +180,20 @@ struct Work {
     Rec *best;          // Step-C records
     Sel *dsel;          // Step-D selections
     uint32_t *winbits;  // bit j: column j holds a Step-C winner this pass
-    int32_t *wkey;      // key column of winner j (set by Step D), -1 if dropped
+    int32_t *wkey;      // key column k of winner j (set by Step D), ~k if dropped
+    // incremental passes: per entry, a bit each for "closing entry found" and
+    // "positive gain" at its last evaluation; per column whose mate changed
+    // the row matched to it before; two sets (of alternate passes) of bitmaps:
+    // changed rows (folded), columns to search whole, columns to search by
+    // their entries of positive gain, tiles of either
+    uint32_t *foundbits;
+    uint32_t *posbits;
+    int32_t *mc_old;
+    uint32_t *map_small[2];
+    uint32_t *map_large[2];
+    uint32_t *colfull[2];
+    uint32_t *colpos[2];
+    uint32_t *tilemark[2];
     int32_t *tile_col;  // column holding the first nonzero of each tile
     uint32_t *starts;   // bit p set when a column starts at nonzero p
     Ctl *ctl;
@@ -237,6 +269,8 @@ struct Shape {
     int search_waves;   // size class: 2 when there are at least 64 tiles per resident
                         // search warp, else 1 (keys the cached graphs; Step D's grid)
     int select;         // AWPM_SELECT_STEP_D or AWPM_SELECT_GREEDY
+    bool inc = false;   // passes after the first are incremental
+    bool large = false; // n > kMapSmallBits: the incremental search's large form
 };
 
 constexpr int kWsumBlocks = 1024;
@@ -251,13 +285,17 @@ struct Sink {
     cudaGraph_t graph = nullptr;
     cudaGraphNode_t last = nullptr;
     cudaError_t err = cudaSuccess;
-    void launch(const void *func, unsigned grid, unsigned block, void **args);
+    void launch(const void *func, unsigned grid, unsigned block, void **args, unsigned smem = 0);
 };
 
 // Launch sequences; `d` is the device copy of the Work.
 void launch_init(const Work *d, const Shape &sh, Sink &k);
 void launch_weight_sum(const Work *d, const Shape &sh, bool out, Sink &k);
 void launch_search(const Work *d, const Shape &sh, Sink &k);
+// The search of a pass after the first with Shape::inc.
+void launch_search_inc(const Work *d, const Shape &sh, Sink &k);
+// Allow the incremental search kernels their shared memory (once per device).
+cudaError_t search_inc_setup();
 void launch_select_and_flip(const Work *d, const Shape &sh, Sink &k);
 // Graph form for single problems with Step D: the selection and the flip,
 // whose last block also ends the pass (no separate control kernel).

@@ -231,16 +231,37 @@ __device__ __forceinline__ bool sel_better(double g, int32_t j, double cg, int32
     return a > b || (a == b && j < cj);
 }
 
-// Maximum of (g, lowest root j) into a Step-D selection.
+// A Step-D selection read in one piece: its gain is only meaningful together
+// with its epoch.
+__device__ __forceinline__ Sel ld_sel(const Sel *addr)
+{
+    unsigned long long a, b;
+    asm volatile("{\n\t"
+                 ".reg .b128 t;\n\t"
+                 "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+                 "mov.b128 {%0, %1}, t;\n\t"
+                 "}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(addr)
+                 : "memory");
+    Sel s;
+    s.g = __longlong_as_double((long long)a);
+    s.j = (int32_t)(uint32_t)b;
+    s.epoch = (int32_t)(uint32_t)(b >> 32);
+    return s;
+}
+
+// Maximum of (g, lowest root j) into a Step-D selection (a record of another
+// epoch counts as empty).
 __device__ void sel_combine(Sel *addr, Sel mine, Ctl *ctl)
 {
-    Sel cur = *addr;
+    Sel cur = ld_sel(addr);
     for (int it = 0; it < kCasRetryCap; ++it) {
-        if (!sel_better(mine.g, mine.j, cur.g, cur.j))
+        if (cur.epoch == mine.epoch && !sel_better(mine.g, mine.j, cur.g, cur.j))
             return;
         Sel old = atomicCAS(addr, cur, mine);
         if (__double_as_longlong(old.g) == __double_as_longlong(cur.g) && old.j == cur.j &&
-            old.pad == cur.pad)
+            old.epoch == cur.epoch)
             return;
         cur = old;
     }
@@ -322,6 +343,21 @@ __device__ __forceinline__ int32_t coop_find(const int32_t *__restrict__ rowidx,
 // Initialisation and validation (before the loop of Algorithm 2)
 // ---------------------------------------------------------------------------
 
+// Clear one set of the incremental passes' bitmaps.
+__device__ __forceinline__ void inc_clear(const Work &w, int set)
+{
+    for (int64_t x = gtid(); x < kMapSmallBits / 32; x += gstride())
+        w.map_small[set][x] = 0u;
+    for (int64_t x = gtid(); x < w.map_bits / 32; x += gstride())
+        w.map_large[set][x] = 0u;
+    for (int64_t x = gtid(); x < w.n / 32 + 2; x += gstride()) {
+        w.colfull[set][x] = 0u;
+        w.colpos[set][x] = 0u;
+    }
+    for (int64_t x = gtid(); x < w.ntiles / 32 + 1; x += gstride())
+        w.tilemark[set][x] = 0u;
+}
+
 // Clear everything a solve expects to start at zero (or empty).
 __global__ void k_reset(const Work *__restrict__ W)
 {
@@ -340,6 +376,7 @@ __global__ void k_reset(const Work *__restrict__ W)
         c->candidates = 0ull;
         c->found = 0ull;
         c->positive = 0ull;
+        c->d_candidates = c->d_found = c->d_positive = 0ull;
         c->weight_in = 0.0;
         c->weight_out = 0.0;
         if (w.bw.count > 0) {
@@ -368,6 +405,14 @@ __global__ void k_reset(const Work *__restrict__ W)
     if (w.bloom)
         for (int64_t x = gtid(); x <= (int64_t)w.nnz / 4; x += gstride())
             w.bloom[x] = 0u;
+    if (w.inc) {
+        for (int64_t x = gtid(); x < w.ntiles; x += gstride()) {
+            w.foundbits[x] = 0u;
+            w.posbits[x] = 0u;
+        }
+        inc_clear(w, 0);
+        inc_clear(w, 1);
+    }
     if (w.rowsig)
         for (int64_t x = gtid(); x < w.n; x += gstride())
             w.rowsig[x] = 0ull;
@@ -1201,27 +1246,30 @@ struct LookupQueue {
 // a closing entry found gives the gain in the fixed order
 // ((w_ij + w_q) - w(i, m_i)) - w(m_j, j), and a positive gain goes into the
 // root's Step-C record (maximum gain, then lowest position; Algorithm 5).
-// Called by the whole warp.
-template <int kLookup, typename Queue>
-__device__ __forceinline__ void resolve_lookups(
-    const Queue &qu, int head, int k, int lane, const int32_t *__restrict__ rowidx,
-    const double *__restrict__ wv, const double *__restrict__ wm,
-    const unsigned long long *__restrict__ htab, const uint32_t *__restrict__ bloom,
-    const int32_t *__restrict__ trowptr, const int32_t *__restrict__ tpos,
-    const RowRange *__restrict__ rrange, int32_t nnz, int32_t nrows, Rec *__restrict__ best,
-    uint32_t *winbits,
-    Ctl *ctl, uint32_t &n_found, uint32_t &n_pos)
+// With foundbits, the outcome is also kept per entry (for the incremental
+// passes).  Called by the whole warp.
+//
+// Returns bit 0: closing entry found, bit 1: positive gain.
+template <int kLookup>
+__device__ __forceinline__ unsigned resolve_inline(const Work *__restrict__ W, const int2 *qim,
+                                                 const int2 *qjp, int head, int k)
 {
+    const Work &w = *W;
+    const int lane = threadIdx.x & 31;
+    const int32_t *__restrict__ rowidx = w.rowidx;
+    const int32_t nnz = w.nnz;
+    [[maybe_unused]] const int32_t nrows = w.n;
+    Ctl *ctl = w.ctl;
     const int x = (head + lane) & (kQueue - 1);
     const bool act = lane < k;
-    const int2 im = act ? qu.im[x] : make_int2(0, 0);
+    const int2 im = act ? qim[x] : make_int2(0, 0);
     const int32_t mj = im.y;
     // column m_i's rows rowidx[lo, lo + len) and w(i, m_i), from the row
     // record of i
     int32_t lo = 0, len = 0;
     double wmi = 0.0;
     if (act && AWPM_IN(ctl, im.x, nrows)) {
-        const RowRange rg = ld_range(rrange + im.x);
+        const RowRange rg = ld_range(w.rrange + im.x);
         lo = rg.s;
         len = rg.e - rg.s;
         wmi = rg.w;
@@ -1234,7 +1282,7 @@ __device__ __forceinline__ void resolve_lookups(
         const int32_t hsize = 2 * len;
         int32_t pos = hsize > 0 ? slot_start(mj, hbase, hsize) : 0;
         for (int32_t left = hsize; left > 0; --left) {
-            const unsigned long long v = __ldg(htab + pos);
+            const unsigned long long v = __ldg(w.htab + pos);
             if ((int32_t)(uint32_t)v == mj) {
                 q = (int32_t)(v >> 32);
                 break;
@@ -1248,8 +1296,8 @@ __device__ __forceinline__ void resolve_lookups(
         // column m_i's positions are [a, b); row m_j's entries tpos[lo, lo + len)
         const int32_t a = lo, b = lo + len;
         if (act) {
-            lo = __ldg(trowptr + mj);
-            len = __ldg(trowptr + mj + 1) - lo;
+            lo = __ldg(w.trowptr + mj);
+            len = __ldg(w.trowptr + mj + 1) - lo;
             if (lo < 0 || len < 0 || len > nnz - lo) {
                 lo = 0;
                 len = 0;
@@ -1263,9 +1311,9 @@ __device__ __forceinline__ void resolve_lookups(
             const int32_t ss = __shfl_sync(FULL_MASK, lo, src);
             const int32_t sl = __shfl_sync(FULL_MASK, len, src);
             const int32_t sb = __shfl_sync(FULL_MASK, b, src);
-            const int32_t f = coop_last_below(tpos, ss, sl, sb, lane);
+            const int32_t f = coop_last_below(w.tpos, ss, sl, sb, lane);
             if (lane == src) {
-                const int32_t v = f >= 0 ? __ldg(tpos + f) : -1;
+                const int32_t v = f >= 0 ? __ldg(w.tpos + f) : -1;
                 q = v >= a ? v : -1;
                 len = 0;
             }
@@ -1275,22 +1323,22 @@ __device__ __forceinline__ void resolve_lookups(
         int32_t hi = lo + len;
         while (lo < hi) {
             const int32_t mid = (lo + hi) >> 1;
-            if (__ldg(tpos + mid) < b)
+            if (__ldg(w.tpos + mid) < b)
                 lo = mid + 1;
             else
                 hi = mid;
         }
         if (len > 0 && lo > s0) {
-            const int32_t v = __ldg(tpos + lo - 1);
+            const int32_t v = __ldg(w.tpos + lo - 1);
             if (v >= a)
                 q = v;
         }
     } else {
-        if (bloom && len > kBloomMin) {
+        if (w.bloom && len > kBloomMin) {
             // long column: its Bloom filter rules most absent rows out first
             uint32_t word, b;
             bloom_key(mj, lo, lo + len, word, b);
-            if ((__ldg(bloom + word) & b) != b)
+            if ((__ldg(w.bloom + word) & b) != b)
                 len = 0;
         }
         // long columns: the warp searches them together, one request at a time
@@ -1324,26 +1372,91 @@ __device__ __forceinline__ void resolve_lookups(
             }
         }
     }
-    const int2 jp = q >= 0 ? qu.jp[x] : make_int2(0, 0);
+    const int2 jp = act ? qjp[x] : make_int2(-1, -1);
     if (q >= 0 && !(AWPM_IN(ctl, q, nnz) && AWPM_IN(ctl, jp.y, nnz) && AWPM_IN(ctl, jp.x, nrows)))
         q = -1;
+    double gg = 0.0;
+    bool pos = false;
     if (q >= 0) {
-        ++n_found;
-        const int32_t j = jp.x;
-        const int32_t p = jp.y;
-        const double wij = __ldg(wv + p);
-        const double wq = __ldg(wv + q);
-        const double gg = ((wij + wq) - wmi) - __ldg(wm + j);
-        if (gain_positive(gg)) {
-            ++n_pos;
-            Rec r;
-            r.g = gg;
-            r.p = p;
-            r.q = q;
-            rec_combine(best + j, r, ctl);
-            atomicOr(winbits + (j >> 5), 1u << (j & 31));
+        const double wij = __ldg(w.w + jp.y);
+        const double wq = __ldg(w.w + q);
+        gg = ((wij + wq) - wmi) - __ldg(w.wm + jp.x);
+        pos = gain_positive(gg);
+    }
+    // The queue holds entries in the order of their positions, so entries of
+    // one column (and of one tile) sit side by side: each column's best gain
+    // and each tile's bits are combined in the warp first, and one lane per
+    // column or tile goes to memory.
+    const unsigned any_found = __ballot_sync(FULL_MASK, q >= 0);
+    const unsigned any_pos = __ballot_sync(FULL_MASK, pos);
+    if (w.inc && any_found) {
+        const int32_t tile = act ? jp.y >> 5 : -1;
+        uint32_t fb = q >= 0 ? 1u << (jp.y & 31) : 0u;
+        uint32_t pb = pos ? fb : 0u;
+        const bool several = (any_found & (any_found - 1u)) != 0u;
+        if (several) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t tt = __shfl_down_sync(FULL_MASK, tile, o);
+                const uint32_t f2 = __shfl_down_sync(FULL_MASK, fb, o);
+                const uint32_t p2 = __shfl_down_sync(FULL_MASK, pb, o);
+                if (tt == tile) {  // (past lane 31: the lane's own bits)
+                    fb |= f2;
+                    pb |= p2;
+                }
+            }
+        }
+        const int32_t before = __shfl_up_sync(FULL_MASK, tile, 1);
+        if (fb && (!several || lane == 0 || before != tile)) {
+            atomicOr(w.foundbits + tile, fb);
+            if (pb)
+                atomicOr(w.posbits + tile, pb);
         }
     }
+    if (any_pos) {
+        long long gk = pos ? gbits(gg) : 0ll;
+        int best_lane = lane;
+        int32_t best_p = jp.y;
+        const bool several = (any_pos & (any_pos - 1u)) != 0u;
+        if (several) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int32_t jj = __shfl_down_sync(FULL_MASK, jp.x, o);
+                const long long g2 = __shfl_down_sync(FULL_MASK, gk, o);
+                const int l2 = __shfl_down_sync(FULL_MASK, best_lane, o);
+                const int32_t p2 = __shfl_down_sync(FULL_MASK, best_p, o);
+                // larger gain, then lower position
+                if (jj == jp.x && (g2 > gk || (g2 == gk && p2 < best_p))) {
+                    gk = g2;
+                    best_lane = l2;
+                    best_p = p2;
+                }
+            }
+        }
+        const int32_t before = __shfl_up_sync(FULL_MASK, jp.x, 1);
+        Rec r;
+        r.g = __longlong_as_double(gk);
+        r.p = best_p;
+        r.q = __shfl_sync(FULL_MASK, q, best_lane);
+        if (gk > 0ll && (!several || lane == 0 || before != jp.x)) {
+            const int32_t j = jp.x;
+            rec_combine(w.best + j, r, ctl);
+            atomicOr(w.winbits + (j >> 5), 1u << (j & 31));
+        }
+    }
+    return (q >= 0 ? 1u : 0u) | (pos ? 2u : 0u);
+}
+
+// The same out of line, for the searches that spend most of their time
+// elsewhere: with a copy at each place of use their warps wait for
+// instructions (the incremental search of a 27-point stencil of 96^3: 318 us
+// inlined, 267 us with one copy; the full search of the R-MAT graph of scale
+// 22 is the other way round, 280 us inlined, 351 us with one copy).
+template <int kLookup>
+__device__ __noinline__ unsigned resolve_lookups(const Work *__restrict__ W, const int2 *qim,
+                                                 const int2 *qjp, int head, int k)
+{
+    return resolve_inline<kLookup>(W, qim, qjp, head, k);
 }
 
 // One warp per tile of kTile consecutive nonzeros (lane = one nonzero).
@@ -1387,20 +1500,12 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
     const int32_t nnz = W->nnz;
     const int32_t ntiles = W->ntiles;
     const int32_t *__restrict__ rowidx = W->rowidx;
-    const double *__restrict__ wv = W->w;
     const int32_t *__restrict__ tile_col = W->tile_col;
     const uint32_t *__restrict__ starts = W->starts;
     const int32_t *__restrict__ mc = W->mc;
-    const double *__restrict__ wm = W->wm;
     const unsigned long long *__restrict__ rsig = W->rsig;
     const RowRange *__restrict__ rrange = W->rrange;
-    const unsigned long long *__restrict__ htab = W->htab;
-    const uint32_t *__restrict__ bloom = W->bloom;
     const unsigned long long *__restrict__ rowsig = W->rowsig;
-    const int32_t *__restrict__ trowptr = W->trowptr;
-    const int32_t *__restrict__ tpos = W->tpos;
-    Rec *__restrict__ best = W->best;
-    uint32_t *winbits = W->winbits;
     Ctl *ctl = W->ctl;
     const int32_t *__restrict__ tilemat = W->bw.tilemat;
     const int32_t *__restrict__ colmat = W->bw.colmat;
@@ -1417,8 +1522,9 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
 
     auto flush = [&](int k) {
         __syncwarp();
-        resolve_lookups<kLookup>(qu, qhead, k, lane, rowidx, wv, wm, htab, bloom, trowptr,
-                                 tpos, rrange, nnz, W->n, best, winbits, ctl, n_found, n_pos);
+        const unsigned got = resolve_lookups<kLookup>(W, qu.im, qu.jp, qhead, k);
+        n_found += got & 1u;
+        n_pos += got >> 1;
         __syncwarp();
         qhead = (qhead + k) & (kQueue - 1);
         qn -= k;
@@ -1617,20 +1723,12 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
     const int32_t nnz = W->nnz;
     const int32_t ntiles = W->ntiles;
     const int32_t *__restrict__ rowidx = W->rowidx;
-    const double *__restrict__ wv = W->w;
     const int32_t *__restrict__ tile_col = W->tile_col;
     const uint32_t *__restrict__ starts = W->starts;
     const int32_t *__restrict__ mc = W->mc;
-    const double *__restrict__ wm = W->wm;
     const unsigned long long *__restrict__ rsig = W->rsig;
     const RowRange *__restrict__ rrange = W->rrange;
-    const unsigned long long *__restrict__ htab = W->htab;
-    const uint32_t *__restrict__ bloom = W->bloom;
     const unsigned long long *__restrict__ rowsig = W->rowsig;
-    const int32_t *__restrict__ trowptr = W->trowptr;
-    const int32_t *__restrict__ tpos = W->tpos;
-    Rec *__restrict__ best = W->best;
-    uint32_t *winbits = W->winbits;
     Ctl *ctl = W->ctl;
     LookupQueueD &qd = s_queue[threadIdx.x >> 5];
     // a batched solve walks the list of the running matrices' tiles
@@ -1650,8 +1748,9 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
 
     auto flush = [&](int k) {
         __syncwarp();
-        resolve_lookups<kLookup>(qd, qhead, k, lane, rowidx, wv, wm, htab, bloom, trowptr,
-                                 tpos, rrange, nnz, W->n, best, winbits, ctl, n_found, n_pos);
+        const unsigned got = resolve_inline<kLookup>(W, qd.im, qd.jp, qhead, k);
+        n_found += got & 1u;
+        n_pos += got >> 1;
         __syncwarp();
         qhead = (qhead + k) & (kQueue - 1);
         qn -= k;
@@ -1778,23 +1877,272 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
     block_add_u64((unsigned long long)n_pos, &ctl->positive);
 }
 
+// The search of a pass after the first.  An entry (i, j) evaluates to the same
+// outcome as in the pass before unless the last flips changed the mate of row
+// i or of column j, so this search streams the row indices and evaluates
+//   - the entries whose row is in the bitmap of changed rows (folded, in
+//     shared memory: a false positive only evaluates an entry again),
+//   - every entry of a column whose mate changed, and
+//   - of a column whose Step-C record had to go because its row's mate
+//     changed, the entries that had a positive gain (no other unchanged entry
+//     can give the column's maximum).
+// Everything else stands: a column's record is emptied by the flip in just
+// those two cases, and otherwise the maximum over the entries evaluated again
+// joins it.  The pass's counts are the last pass's plus the differences: two
+// bits per entry keep what it counted for.
+//
+// A warp takes chunks of up to eight consecutive tiles (fewer when there are
+// not enough tiles to go round).  The tiles of marked columns are in a bitmap
+// of their own, so a chunk without a changed row or a marked tile costs its
+// row loads, one shared-memory word per entry and a vote.  Entries to evaluate
+// are queued per warp and taken 32 at a time, all lanes busy: the candidate
+// and signature tests, then the lookups as in the full search.  Bound by the
+// row stream and the shared-memory reads of the scan when little is affected,
+// by the lookups' latency when much is.
+struct IncQueue {
+    int2 ij[kQueue];     // row i; column j, with the sign bit set when j is searched whole
+    int32_t p[kQueue];   // position of (i, j)
+    LookupQueue look;
+};
+
+template <bool kLarge>
+struct IncBlock {
+    static constexpr int kThreads = kLarge ? 1024 : 512;
+    static constexpr int kWarps = kThreads / 32;
+    static constexpr unsigned kSmem =
+        kWarps * sizeof(IncQueue) + (kLarge ? kMapLargeBits : kMapSmallBits) / 8;
+};
+
+template <int kLookup, bool kLarge>
+__global__ void __launch_bounds__(IncBlock<kLarge>::kThreads, kLarge ? 1 : 2)
+    k_search_inc(const Work *__restrict__ W)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    __shared__ int s_go;
+    constexpr int kT = 8;
+    uint32_t *s_map = reinterpret_cast<uint32_t *>(s_raw);
+    const Work &w = *W;
+    Ctl *ctl = w.ctl;
+    if (threadIdx.x == 0)
+        s_go = gate(ctl) ? 1 : 0;
+    __syncthreads();
+    if (!s_go)
+        return;
+    const int set = (ctl->iterations - 1) & 1;
+    // the bitmap of changed rows
+    const bool use_large = kLarge && ctl->last_flips > kSmallFlips;
+    const int32_t bits = use_large ? w.map_bits : kMapSmallBits;
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(use_large ? w.map_large[set]
+                                                                     : w.map_small[set]);
+        for (int x = threadIdx.x; x < bits / 128; x += IncBlock<kLarge>::kThreads)
+            reinterpret_cast<uint4 *>(s_map)[x] = __ldcg(src + x);
+    }
+    const uint32_t fold = (uint32_t)bits - 1u;
+    IncQueue &q1 = *reinterpret_cast<IncQueue *>(
+        s_raw + (kLarge ? kMapLargeBits : kMapSmallBits) / 8 + (threadIdx.x >> 5) * sizeof(IncQueue));
+    LookupQueue &q2 = q1.look;
+    __syncthreads();
+
+    [[maybe_unused]] const int32_t n = w.n;
+    const int32_t nnz = w.nnz, ntiles = w.ntiles;
+    const int32_t *__restrict__ rowidx = w.rowidx;
+    const int32_t *__restrict__ mc = w.mc;
+    const int32_t *__restrict__ mc_old = w.mc_old;
+    const unsigned long long *__restrict__ rsig = w.rsig;
+    const uint32_t *__restrict__ colfull = w.colfull[set];
+    const uint32_t *__restrict__ colpos = w.colpos[set];
+    const int lane = threadIdx.x & 31;
+    const unsigned lanes_below = (1u << lane) - 1u;
+    const int32_t nwarps = (int32_t)(gstride() >> 5);
+    const unsigned long long pol = policy_evict_last();
+    int32_t n_cand = 0;
+    uint32_t n_found = 0, n_pos = 0;  // differences, modulo 2^32
+    int h1 = 0, c1 = 0, h2 = 0, c2 = 0;  // the warp's queues (warp-uniform)
+
+    auto lookups = [&](int k) {
+        __syncwarp();
+        const unsigned got = resolve_lookups<kLookup>(W, q2.im, q2.jp, h2, k);
+        n_found += got & 1u;
+        n_pos += got >> 1;
+        __syncwarp();
+        h2 = (h2 + k) & (kQueue - 1);
+        c2 -= k;
+    };
+    // entries h1 .. h1 + k - 1: candidate test, signature test, lookup queue
+    auto evaluate = [&](int k) {
+        __syncwarp();
+        const int x = (h1 + lane) & (kQueue - 1);
+        bool pass = false;
+        int32_t i = 0, j = 0, mj = 0, p = 0;
+        if (lane < k) {
+            const int2 ij = q1.ij[x];
+            i = ij.x;
+            j = ij.y & 0x7fffffff;
+            p = q1.p[x];
+            if (AWPM_IN(ctl, i, n) && AWPM_IN(ctl, j, n)) {
+                mj = ld_i32_last(mc + j, pol);
+                const unsigned long long sig = ld_u64_last(rsig + i, pol);
+                const bool cand = i > mj;
+                if (ij.y < 0)  // a column searched whole may have another mate now
+                    n_cand += (int)cand - (int)(i > __ldg(mc_old + j));
+                pass = cand && AWPM_IN(ctl, mj, n) && sig_has(sig, mj);
+                if (kLookup == AWPM_LOOKUP_ROWMARK && pass)
+                    pass = sig_has(__ldg(w.rowsig + mj), __ldg(&w.rrange[i].s));
+            }
+        }
+        const unsigned need = __ballot_sync(FULL_MASK, pass);
+        if (pass) {
+            const int y = (h2 + c2 + __popc(need & lanes_below)) & (kQueue - 1);
+            q2.im[y] = make_int2(i, mj);
+            q2.jp[y] = make_int2(j, p);
+        }
+        __syncwarp();
+        h1 = (h1 + k) & (kQueue - 1);
+        c1 -= k;
+        c2 += __popc(need);
+        if (c2 >= 32)
+            lookups(32);
+    };
+
+    int T = 1;
+    while (T < kT && ntiles >= 2 * T * nwarps)
+        T *= 2;
+    const int32_t step = T * nwarps;
+    const uint32_t *__restrict__ tmark = w.tilemark[set];
+    const uint32_t tbits = (1u << T) - 1u;
+    // the row indices of the chunk's tiles (-1 past the end), and which of
+    // its tiles hold marked columns
+    int32_t pr[kT];
+    uint32_t pmark = 0u;
+    auto fetch = [&](int32_t t0) {
+        pmark = (__ldg(tmark + (t0 >> 5)) >> (t0 & 31)) & tbits;
+        const int32_t *src = rowidx + ((int64_t)t0 * kTile + lane);
+        if (T == kT && t0 + kT < ntiles) {
+#pragma unroll
+            for (int u = 0; u < kT; ++u)
+                pr[u] = __ldg(src + u * kTile);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kT; ++u) {
+                const int32_t p = (t0 + u) * kTile + lane;
+                pr[u] = u < T && t0 + u < ntiles && p < nnz ? __ldg(src + u * kTile) : -1;
+            }
+        }
+    };
+    const unsigned char *map8 = reinterpret_cast<const unsigned char *>(s_map);
+    const uint32_t fold8 = fold >> 3 & ~3u;  // byte address of a row's word
+    int32_t t0 = T * (int32_t)(gtid() >> 5);
+    if (t0 < ntiles)
+        fetch(t0);
+    for (; t0 < ntiles; t0 += step) {
+        const uint32_t marked = pmark;
+        uint32_t hits = 0u;  // bit u: the lane's entry of tile u is in a changed row
+#pragma unroll
+        for (int u = 0; u < kT; ++u) {
+            const uint32_t r = (uint32_t)pr[u];
+            const uint32_t word = *reinterpret_cast<const uint32_t *>(map8 + ((r >> 3) & fold8));
+            hits |= (__funnelshift_r(word, word, r) & 1u) << u;
+        }
+        // (past the end r = -1 may match: masked below)
+        if (t0 + step < ntiles)
+            fetch(t0 + step);
+        if (!__any_sync(FULL_MASK, hits | marked))
+            continue;
+        // words of the chunk's tiles, one tile per lane
+        int32_t c0 = 0;
+        uint32_t mask = 1u, fw = 0u, pw = 0u, cwin = 0u, pwin = 0u;
+        if (lane < T && t0 + lane < ntiles) {
+            c0 = __ldg(w.tile_col + t0 + lane);
+            mask = __ldg(w.starts + t0 + lane);
+            fw = w.foundbits[t0 + lane];
+            pw = w.posbits[t0 + lane];
+            if ((marked >> lane) & 1u) {
+                // the 32 columns from c0 on: to be searched whole, or by
+                // their entries of positive gain
+                const int32_t x = c0 >> 5;
+                cwin = __funnelshift_r(__ldg(colfull + x), __ldg(colfull + x + 1), c0 & 31);
+                pwin = __funnelshift_r(__ldg(colpos + x), __ldg(colpos + x + 1), c0 & 31);
+            }
+        }
+        // (rolled: the row indices are read again, from L1)
+#pragma unroll 1
+        for (int u = 0; u < T; ++u) {
+            const uint32_t mk = __shfl_sync(FULL_MASK, mask, u);
+            const int32_t rank = lane_column(0, mk, lane);
+            const uint32_t g = __shfl_sync(FULL_MASK, pw, u);
+            bool hit = (hits >> u) & 1u, full = false;
+            if ((marked >> u) & 1u) {
+                full = (__shfl_sync(FULL_MASK, cwin, u) >> rank) & 1u;
+                hit |= full |
+                       (((__shfl_sync(FULL_MASK, pwin, u) >> rank) & (g >> lane) & 1u) != 0u);
+            }
+            const int32_t t = t0 + u, p = t * kTile + lane;
+            hit &= t < ntiles && p < nnz;
+            const unsigned m = __ballot_sync(FULL_MASK, hit);
+            if (!m)
+                continue;
+            const int32_t j = __shfl_sync(FULL_MASK, c0, u) + rank;
+            // what these entries counted for at their last evaluation
+            const uint32_t f = __shfl_sync(FULL_MASK, fw, u);
+            if (lane == 0 && (f & m)) {
+                n_found -= __popc(f & m);
+                n_pos -= __popc(g & m);
+                w.foundbits[t] = f & ~m;
+                w.posbits[t] = g & ~m;
+            }
+            if (hit) {
+                const int x = (h1 + c1 + __popc(m & lanes_below)) & (kQueue - 1);
+                q1.ij[x] = make_int2(__ldg(rowidx + p),
+                                     full ? (int)((uint32_t)j | 0x80000000u) : j);
+                q1.p[x] = p;
+            }
+            c1 += __popc(m);
+            if (c1 >= 32)
+                evaluate(32);
+        }
+    }
+    if (c1 > 0)
+        evaluate(c1);
+    if (c2 > 0)
+        lookups(c2);
+    // (counts taken off and added: signed 32-bit per thread)
+    block_add_u64((unsigned long long)(long long)n_cand, &ctl->d_candidates);
+    block_add_u64((unsigned long long)(long long)(int32_t)n_found, &ctl->d_found);
+    block_add_u64((unsigned long long)(long long)(int32_t)n_pos, &ctl->d_positive);
+}
+
 // ---------------------------------------------------------------------------
 // Step D (Algorithm 6): conflicts, per-key selection, flip
 // ---------------------------------------------------------------------------
 
-// The winners (set bits) of the bitmap words [x0, x0 + 32), 32 at a time
-// with every lane busy: the words' bit counts are scanned across the warp,
-// and in each round lane l takes the winner of rank round * 32 + l (found by
-// a binary search over the scan and the word's rank-th set bit).  Calls
-// f(j) on every lane each round, j = -1 for lanes past the last winner.
-// Called by the whole warp; `clear` zeroes the words as they are read.
-template <typename F>
-__device__ __forceinline__ void for_winners(uint32_t *winbits, int64_t x0, int64_t words, int lane,
-                                            bool clear, F f)
+// Bitmap words a warp takes at a time when `words` of them are spread over
+// `nwarps` warps: 32 (one per lane) when there are enough, fewer, down to 1,
+// when that keeps more warps busy (the winners' accesses are scattered, so
+// the time goes with the winners that one warp takes in turn).
+__device__ __forceinline__ int words_per_warp(int64_t words, int64_t nwarps)
 {
-    const uint32_t mine = x0 + lane < words ? winbits[x0 + lane] : 0u;
+    int k = 1;
+    while (k < 32 && k * nwarps < words)
+        k *= 2;
+    return k;
+}
+
+// The winners (set bits) of the bitmap words [x0, x0 + count), count <= 32,
+// 32 winners at a time with every lane busy: the words' bit counts are
+// scanned across the warp, and in each round lane l takes the winner of rank
+// round * 32 + l (found by a binary search over the scan and the word's
+// rank-th set bit).  Calls f(j) on every lane each round, j = -1 for lanes
+// past the last winner.  Called by the whole warp; `clear` zeroes the words
+// as they are read.
+template <typename F>
+__device__ __forceinline__ void for_winners(uint32_t *winbits, int64_t x0, int count,
+                                            int64_t words, int lane, bool clear, F f)
+{
+    const uint32_t mine = lane < count && x0 + lane < words ? winbits[x0 + lane] : 0u;
     if (clear && mine)
         winbits[x0 + lane] = 0u;
+    __syncwarp();  // f may set a bit of a cleared word again
     const int cnt = __popc(mine);
     int incl = cnt;
 #pragma unroll
@@ -1826,12 +2174,18 @@ __device__ __forceinline__ void for_winners(uint32_t *winbits, int64_t x0, int64
     }
 }
 
+// The epoch of the running pass's Step-D records.
+__device__ __forceinline__ int32_t pass_epoch(const Work &w)
+{
+    return w.epoch0 + w.ctl->iterations + 1;
+}
+
 // For every Step-C winner rooted at j (a set bit of the winner bitmap) with
 // second matched edge at column k = m_i: drop it if column k is itself the
 // root of a Step-C winner, otherwise compete for key k (maximum gain, then
-// lowest root j).  The winner's key (or -1) is kept for the flip.  A warp
-// takes 32 bitmap words at a time and their winners 32 at a time, a lane
-// per winner.
+// lowest root j).  The winner's key (or its complement) is kept for the flip.
+// A warp takes up to 32 bitmap words at a time and their winners 32 at a
+// time, a lane per winner.
 __global__ void k_select(const Work *__restrict__ W)
 {
     const Work &w = *W;
@@ -1840,8 +2194,10 @@ __global__ void k_select(const Work *__restrict__ W)
     const int lane = threadIdx.x & 31;
     const int64_t words = (int64_t)w.n / 32 + 1;
     const int64_t nwarps = gstride() >> 5;
-    for (int64_t x0 = (gtid() >> 5) * 32; x0 < words; x0 += nwarps * 32) {
-        for_winners(w.winbits, x0, words, lane, false, [&](int32_t j) {
+    const int per = words_per_warp(words, nwarps);
+    const int32_t epoch = pass_epoch(w);
+    for (int64_t x0 = (gtid() >> 5) * per; x0 < words; x0 += nwarps * per) {
+        for_winners(w.winbits, x0, per, words, lane, false, [&](int32_t j) {
             if (j < 0 || !AWPM_IN(w.ctl, j, w.n))
                 return;
             const Rec r = w.best[j];
@@ -1854,26 +2210,66 @@ __global__ void k_select(const Work *__restrict__ W)
             if (!AWPM_IN(w.ctl, k, w.n))
                 return;
             if ((w.winbits[k >> 5] >> (k & 31)) & 1u) {
-                w.wkey[j] = -1;
+                w.wkey[j] = ~k;
                 return;
             }
             w.wkey[j] = k;
             Sel sl;
             sl.g = r.g;
             sl.j = j;
-            sl.pad = 0;
+            sl.epoch = epoch;
             sel_combine(w.dsel + k, sl, w.ctl);
         });
     }
 }
 
+// Row r has another mate now: into this pass's bitmaps of changed rows.
+__device__ __forceinline__ void mark_row(const Work &w, int set, int32_t r)
+{
+    const uint32_t s = (uint32_t)r & (kMapSmallBits - 1);
+    atomicOr(w.map_small[set] + (s >> 5), 1u << (s & 31));
+    if (w.map_bits) {
+        const uint32_t b = (uint32_t)r & (uint32_t)(w.map_bits - 1);
+        atomicOr(w.map_large[set] + (b >> 5), 1u << (b & 31));
+    }
+}
+
+// The next pass looks at the tiles of the column at positions [s, e).
+__device__ __forceinline__ void mark_tiles(const Work &w, int set, int32_t s, int32_t e)
+{
+    const int32_t t1 = (e - 1) >> 5;
+    for (int32_t t = s >> 5; t <= t1;) {
+        const int32_t last = min(t1, t | 31);  // last tile of the bitmap word
+        const uint32_t bits = (0xffffffffu >> (31 - (last - t))) << (t & 31);
+        atomicOr(w.tilemark[set] + (t >> 5), bits);
+        t = last + 1;
+    }
+}
+
+// The next pass searches column j whole; `was` is the row its entries were
+// last evaluated with.
+__device__ __forceinline__ void mark_column(const Work &w, int set, int32_t j, int32_t was,
+                                            int32_t s, int32_t e)
+{
+    atomicOr(w.colfull[set] + (j >> 5), 1u << (j & 31));
+    w.mc_old[j] = was;
+    mark_tiles(w, set, s, e);
+}
+
 // Flip every selected cycle: column j takes row i, key column k takes m_j;
 // the row records of rows i and m_j follow their new mates.  The selected
-// cycles are vertex-disjoint, so each lane owns its four vertices.  The
-// Step-C records and winner bits visited are cleared, which leaves them
-// empty for the next pass.  Winners are taken as in k_select; in a batched
-// solve the flips of a round are counted per matrix with one atomic per
-// matrix.
+// cycles are vertex-disjoint, so each lane owns its four vertices.  Winners
+// are taken as in k_select; in a batched solve the flips of a round are
+// counted per matrix with one atomic per matrix.
+//
+// The Step-C records and winner bits visited are cleared, which leaves them
+// empty for the next pass -- except, with incremental passes, those of
+// winners whose row i keeps its mate: their entry's outcome stands, and so
+// does their column's maximum.  Row i's mate is column k; it changes exactly
+// when k is flipped: as the key of the winner selected there (j lost to it),
+// or as the root of the winner that dropped j, if that one was selected.
+// (The greedy selection drops a winner only for sharing a column with a kept
+// cycle, so all its winners' records go.)
 __device__ __forceinline__ unsigned long long flip_body(const Work &w)
 {
     unsigned long long flips = 0;
@@ -1881,19 +2277,39 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
         const int lane = threadIdx.x & 31;
         const int64_t words = (int64_t)w.n / 32 + 1;
         const int64_t nwarps = gstride() >> 5;
-        for (int64_t x0 = (gtid() >> 5) * 32; x0 < words; x0 += nwarps * 32) {
-            for_winners(w.winbits, x0, words, lane, true, [&](int32_t j) {
+        const int per = words_per_warp(words, nwarps);
+        const int32_t epoch = pass_epoch(w);
+        const bool inc = w.inc != 0;
+        const int set = w.ctl->iterations & 1;
+        auto selected = [&](int32_t key, int32_t j) {
+            const Sel sl = w.dsel[key];
+            return sl.epoch == epoch && sl.j == j;
+        };
+        for (int64_t x0 = (gtid() >> 5) * per; x0 < words; x0 += nwarps * per) {
+            for_winners(w.winbits, x0, per, words, lane, true, [&](int32_t j) {
                 int32_t mat = -1;  // matrix of a flipped cycle (batched solve)
                 if (j >= 0 && AWPM_IN(w.ctl, j, w.n)) {
                     const Rec r = w.best[j];
-                    w.best[j] = Rec{0.0, 0, 0};
-                    int32_t k = w.wkey[j];
-                    if (k >= 0 && !(AWPM_IN(w.ctl, k, w.n) && AWPM_IN(w.ctl, r.p, w.nnz) &&
-                                    AWPM_IN(w.ctl, r.q, w.nnz)))
-                        k = -1;
-                    const Sel sl = k >= 0 ? w.dsel[k] : Sel{0.0, 0, 0};
-                    if (k >= 0 && gbits(sl.g) > 0ll && sl.j == j) {
-                        w.dsel[k] = Sel{0.0, 0, 0};
+                    const int32_t key = w.wkey[j];
+                    const int32_t k = key >= 0 ? key : -1;
+                    bool sel = false, stands = false;
+                    if (k >= 0 && AWPM_IN(w.ctl, k, w.n) && AWPM_IN(w.ctl, r.p, w.nnz) &&
+                        AWPM_IN(w.ctl, r.q, w.nnz)) {
+                        sel = selected(k, j);
+                    } else if (inc && !w.psel && key < 0 && AWPM_IN(w.ctl, ~key, w.n)) {
+                        const int32_t k2 = w.wkey[~key];
+                        stands = k2 < 0 || !AWPM_IN(w.ctl, k2, w.n) || !selected(k2, ~key);
+                    }
+                    if (stands) {
+                        atomicOr(w.winbits + (j >> 5), 1u << (j & 31));
+                    } else {
+                        w.best[j] = Rec{0.0, 0, 0};
+                        if (inc && !sel) {
+                            atomicOr(w.colpos[set] + (j >> 5), 1u << (j & 31));
+                            mark_tiles(w, set, w.colptr[j], w.colptr[j + 1]);
+                        }
+                    }
+                    if (sel) {
                         const int32_t i = w.rowidx[r.p];
                         const int32_t mj = w.mc[j];
                         if (AWPM_IN(w.ctl, i, w.n) && AWPM_IN(w.ctl, mj, w.n)) {
@@ -1905,11 +2321,19 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
                             w.mr[mj] = k;
                             w.wm[j] = wij;
                             w.wm[k] = wq;
-                            put_rowrec(w, i, w.colptr[j], w.colptr[j + 1], w.colsig[j], wij);
-                            put_rowrec(w, mj, w.colptr[k], w.colptr[k + 1], w.colsig[k], wq);
+                            const int32_t js = w.colptr[j], je = w.colptr[j + 1];
+                            const int32_t ks = w.colptr[k], ke = w.colptr[k + 1];
+                            put_rowrec(w, i, js, je, w.colsig[j], wij);
+                            put_rowrec(w, mj, ks, ke, w.colsig[k], wq);
                             ++flips;
                             if (w.bw.count > 0)
                                 mat = w.bw.colmat[k];
+                            if (inc) {
+                                mark_row(w, set, i);
+                                mark_row(w, set, mj);
+                                mark_column(w, set, j, mj, js, je);
+                                mark_column(w, set, k, i, ks, ke);
+                            }
                         }
                     }
                 }
@@ -1921,6 +2345,9 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
                 }
             });
         }
+        // the set of bitmaps that this pass's search read, for the next flips
+        if (inc && w.ctl->iterations > 0)
+            inc_clear(w, set ^ 1);
     }
     return flips;
 }
@@ -1932,8 +2359,9 @@ __global__ void k_flip(const Work *__restrict__ W)
 }
 
 // End of a pass (Algorithm 2): count it, stop when nothing was flipped or
-// the pass cap is reached.
-__device__ __forceinline__ int control_step(Ctl *ctl)
+// the pass cap is reached.  An incremental pass counted differences from the
+// pass before.
+__device__ __forceinline__ int control_step(Ctl *ctl, bool inc)
 {
     if (ctl->err) {
         ctl->active = 0;
@@ -1943,6 +2371,19 @@ __device__ __forceinline__ int control_step(Ctl *ctl)
         return 0;
     const unsigned long long f = ctl->pass_flips;
     ctl->pass_flips = 0;
+    if (inc) {
+        if (ctl->iterations == 0) {
+            ctl->cur_candidates = ctl->candidates;
+            ctl->cur_found = ctl->found;
+            ctl->cur_positive = ctl->positive;
+        } else {
+            ctl->candidates += ctl->cur_candidates += ctl->d_candidates;
+            ctl->found += ctl->cur_found += ctl->d_found;
+            ctl->positive += ctl->cur_positive += ctl->d_positive;
+            ctl->d_candidates = ctl->d_found = ctl->d_positive = 0;
+        }
+        ctl->last_flips = f;
+    }
     ctl->iterations += 1;
     ctl->cycles += f;
     if (f == 0) {
@@ -1956,12 +2397,12 @@ __device__ __forceinline__ int control_step(Ctl *ctl)
 
 __global__ void k_control(const Work *__restrict__ W)
 {
-    control_step(W->ctl);
+    control_step(W->ctl, W->inc != 0);
 }
 
 __global__ void k_control_graph(const Work *__restrict__ W, cudaGraphConditionalHandle h)
 {
-    cudaGraphSetConditional(h, control_step(W->ctl) ? 1u : 0u);
+    cudaGraphSetConditional(h, control_step(W->ctl, W->inc != 0) ? 1u : 0u);
 }
 
 // The flip in the graph form of a single problem's pass: the block that
@@ -1977,7 +2418,7 @@ __global__ void k_flip_graph(const Work *__restrict__ W, cudaGraphConditionalHan
         if (prev == gridDim.x - 1) {
             __threadfence();
             w.ctl->flip_done = 0u;
-            cudaGraphSetConditional(h, control_step(w.ctl) ? 1u : 0u);
+            cudaGraphSetConditional(h, control_step(w.ctl, w.inc != 0) ? 1u : 0u);
         }
     }
 }
@@ -2125,7 +2566,7 @@ __global__ void k_ps_name(const Work *__restrict__ W)
             Sel s;
             s.g = w.best[j].g;
             s.j = j;
-            s.pad = 0;
+            s.epoch = 0;
             sel_combine(w.psel + j, s, w.ctl);
             sel_combine(w.psel + w.wkey[j], s, w.ctl);
         }
@@ -2218,7 +2659,7 @@ __global__ void k_ps_end(const Work *__restrict__ W)
                 Sel s;
                 s.g = w.best[j].g;
                 s.j = j;
-                s.pad = 0;
+                s.epoch = pass_epoch(w);
                 w.dsel[k] = s;
                 atomicAnd(w.psused + (j >> 5), ~(1u << (j & 31)));
                 atomicAnd(w.psused + (k >> 5), ~(1u << (k & 31)));
@@ -2935,7 +3376,7 @@ static inline unsigned sum_grid(const Shape &sh)
     return (unsigned)(g < kWsumBlocks ? g : kWsumBlocks);
 }
 
-void Sink::launch(const void *func, unsigned grid, unsigned block, void **args)
+void Sink::launch(const void *func, unsigned grid, unsigned block, void **args, unsigned smem)
 {
     if (err != cudaSuccess)
         return;
@@ -2944,7 +3385,7 @@ void Sink::launch(const void *func, unsigned grid, unsigned block, void **args)
         p.func = const_cast<void *>(func);
         p.gridDim = dim3(grid);
         p.blockDim = dim3(block);
-        p.sharedMemBytes = 0;
+        p.sharedMemBytes = smem;
         p.kernelParams = args;
         p.extra = nullptr;
         cudaGraphNode_t node;
@@ -2952,7 +3393,7 @@ void Sink::launch(const void *func, unsigned grid, unsigned block, void **args)
         if (err == cudaSuccess)
             last = node;
     } else {
-        err = cudaLaunchKernel(func, dim3(grid), dim3(block), args, 0, stream);
+        err = cudaLaunchKernel(func, dim3(grid), dim3(block), args, smem, stream);
     }
 }
 
@@ -3074,6 +3515,45 @@ void launch_search(const Work *d, const Shape &sh, Sink &k)
     const void *f = sh.wide ? search_fn<true>(sh.lookup, sh.batch)
                             : search_fn<false>(sh.lookup, sh.batch);
     k.launch(f, grid, sh.batch ? SearchBlock<true>::kThreads : SearchBlock<false>::kThreads, a);
+}
+
+template <bool kLarge>
+static const void *search_inc_fn(int lookup)
+{
+    if (lookup == AWPM_LOOKUP_ROWMARK)
+        return (const void *)k_search_inc<AWPM_LOOKUP_ROWMARK, kLarge>;
+    if (lookup == AWPM_LOOKUP_HASH)
+        return (const void *)k_search_inc<AWPM_LOOKUP_HASH, kLarge>;
+    return (const void *)k_search_inc<AWPM_LOOKUP_BSEARCH, kLarge>;
+}
+
+cudaError_t search_inc_setup()
+{
+    for (int lookup : {AWPM_LOOKUP_BSEARCH, AWPM_LOOKUP_HASH, AWPM_LOOKUP_ROWMARK}) {
+        cudaError_t e = cudaFuncSetAttribute(search_inc_fn<true>(lookup),
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)IncBlock<true>::kSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(search_inc_fn<false>(lookup),
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)IncBlock<false>::kSmem);
+        if (e != cudaSuccess)
+            return e;
+    }
+    return cudaSuccess;
+}
+
+// One wave: a block of 1,024 threads per SM with the large bitmap, two of 512
+// with the small one.
+void launch_search_inc(const Work *d, const Shape &sh, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    if (sh.large)
+        k.launch(search_inc_fn<true>(sh.lookup), (unsigned)sh.num_sms, IncBlock<true>::kThreads, a,
+                 IncBlock<true>::kSmem);
+    else
+        k.launch(search_inc_fn<false>(sh.lookup), (unsigned)sh.num_sms * 2,
+                 IncBlock<false>::kThreads, a, IncBlock<false>::kSmem);
 }
 
 int search_waves(int num_sms, int search_bps, int32_t ntiles)
