@@ -643,7 +643,8 @@ void ctx_trim(awpm_ctx *c)
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,    &c->gtdead,
                       &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_max,
                       &c->wt_scale, &c->wt_stage, &c->mroot,   &c->mrpar,    &c->mfront,
-                      &c->mnext,   &c->mroff,    &c->mtend,    &c->mtouch,
+                      &c->mreach,  &c->mtmark,   &c->mfl,      &c->mroff,    &c->mtend,
+                      &c->mtouch,
                       &c->mstage,  &c->mcolof,   &c->mtiles,   &c->rowsig,   &c->trowptr,
                       &c->rs_k0,   &c->rs_k1,    &c->rs_v0,    &c->rs_v1,    &c->rs_hist,
                       &c->rs_sums};
@@ -732,7 +733,8 @@ void teardown_ctx(awpm_ctx *c)
                       &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,
                       &c->gtdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
                       &c->wt_max,  &c->wt_scale, &c->wt_stage,
-                      &c->mroot,   &c->mrpar,    &c->mfront,   &c->mnext,    &c->mroff,
+                      &c->mroot,   &c->mrpar,    &c->mfront,   &c->mreach,   &c->mtmark,
+                      &c->mfl,     &c->mroff,
                       &c->mtend,   &c->mtouch,   &c->mstage,   &c->mcolof,
                       &c->mtiles,  &c->rowsig,   &c->trowptr,  &c->rs_k0,    &c->rs_k1,
                       &c->rs_v0,   &c->rs_v1,    &c->rs_hist,  &c->rs_sums};
@@ -1584,12 +1586,13 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
     AWPM_TRY(ensure(c, c->mroff, sizeof(Off) * n));
     AWPM_TRY(ensure(c, c->mtend, sizeof(Off) * n));
     AWPM_TRY(ensure(c, c->mtouch, sizeof(int32_t) * n));
-    AWPM_TRY(ensure(c, c->mfront, sizeof(uint32_t) * words));
+    AWPM_TRY(ensure(c, c->mfront, sizeof(uint32_t) * (words + 1)));
+    AWPM_TRY(ensure(c, c->mreach, sizeof(uint32_t) * (words + 1)));
+    AWPM_TRY(ensure(c, c->mtmark, sizeof(uint32_t) * ((size_t)ntiles / 32 + 1)));
+    AWPM_TRY(ensure(c, c->mfl, sizeof(int32_t) * n));
     AWPM_TRY(ensure(c, c->mcolof, sizeof(int32_t) * ((size_t)nnz + 1)));
-    AWPM_TRY(ensure(c, c->mnext, sizeof(uint32_t) * words));
-    // the level's tile list: at most min(nnz, nnz/32 + 2n) entries
-    const size_t tiles_cap = std::min((size_t)nnz, (size_t)ntiles + 2 * (size_t)n);
-    AWPM_TRY(ensure(c, c->mtiles, sizeof(int32_t) * (tiles_cap + 1)));
+    // the level's tile list: every tile at most once
+    AWPM_TRY(ensure(c, c->mtiles, sizeof(int32_t) * ((size_t)ntiles + 1)));
     AWPM_TRY(ensure(c, c->tile_col, sizeof(int32_t) * ((size_t)ntiles + 1)));
     AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
@@ -1618,14 +1621,16 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
     wk.mroot = (int32_t *)c->mroot.p;
     wk.mrpar = (int32_t *)c->mrpar.p;
     wk.mfront = (uint32_t *)c->mfront.p;
-    wk.mnext = (uint32_t *)c->mnext.p;
+    wk.mreach = (uint32_t *)c->mreach.p;
+    wk.mtmark = (uint32_t *)c->mtmark.p;
+    wk.mfl = (int32_t *)c->mfl.p;
     wk.mroff = (Off *)c->mroff.p;
     wk.mtend = (Off *)c->mtend.p;
     wk.mtouch = (int32_t *)c->mtouch.p;
     wk.mmate = dmate;
     wk.mcolof = (int32_t *)c->mcolof.p;
     wk.mtiles = (int32_t *)c->mtiles.p;
-    wk.mtiles_cap = (int64_t)tiles_cap + 1;
+    wk.mtiles_cap = ntiles;
     CUDA_TRY(cudaMemcpyAsync(c->d_work.p, c->h_work, sizeof(Work), cudaMemcpyHostToDevice,
                              c->stream));
     const Work *d = (const Work *)c->d_work.p;

@@ -45,4 +45,54 @@ __device__ __forceinline__ bool segment_complete(uint32_t mask, int lane, int32_
     return later != 0u || base + kTile >= nnz || (__ldg(starts + t + 1) & 1u);
 }
 
+// Bounded retries for the lock-free arg-max updates (each failed
+// compare-and-swap means another thread stored a strictly better record, so
+// the loop ends long before this; the bound only turns a broken invariant
+// into an error bit instead of a hang).
+constexpr int kCasRetryCap = 1 << 20;
+
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v += __shfl_down_sync(FULL_MASK, v, o);
+    return v;
+}
+
+// Sum v over the block and add it to *dst with one atomic.  All threads call.
+__device__ __forceinline__ void block_add_u64(unsigned long long v, unsigned long long *dst)
+{
+    __shared__ unsigned long long sm[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    v = warp_sum_u64(v);
+    __syncthreads();
+    if (lane == 0)
+        sm[wid] = v;
+    __syncthreads();
+    if (wid == 0) {
+        v = (lane < (int)(blockDim.x >> 5)) ? sm[lane] : 0ull;
+        v = warp_sum_u64(v);
+        if (lane == 0 && v)
+            atomicAdd(dst, v);
+    }
+}
+
+__device__ __forceinline__ void warp_add_i32(int v, int32_t *dst)
+{
+    v = __reduce_add_sync(FULL_MASK, v);
+    if ((threadIdx.x & 31) == 0 && v)
+        atomicAdd(dst, v);
+}
+
+constexpr long long kKeyNone = (long long)0x8000000000000000ull;
+
+// Integer ordered like the weight (-0 taken as +0; finite weights only).
+__device__ __forceinline__ long long order_key(double x)
+{
+    long long b = __double_as_longlong(x);
+    if (b == kKeyNone)
+        b = 0;
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
 }  // namespace awpm

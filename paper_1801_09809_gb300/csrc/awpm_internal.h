@@ -96,10 +96,12 @@ struct Ctl {
     int32_t live;                // greedy selection: winners still undecided
     int32_t nonempty;            // maximum matching: no column is empty
     int32_t phase_levels;        // maximum matching: levels of the running phase
-    int32_t level_tiles;         // maximum matching: tiles listed for the next level
-    int32_t level_listed;        // maximum matching: tiles listed for this level
+    // maximum matching: tiles and columns listed for the next level (counted
+    // with one 64-bit atomic), columns of the running one
+    alignas(8) int32_t level_tiles;
+    int32_t front_next;
+    int32_t front_n;
     uint32_t flip_done;          // blocks done with the pass's flip (graph form)
-    uint32_t pad_fd;
     uint32_t level_done;         // maximum matching: blocks done with the level's last step
     int32_t touched;             // maximum matching: rows listed in mtouch this level
     unsigned long long levels;   // maximum matching: search levels run
@@ -223,15 +225,18 @@ struct Work {
     int32_t wt_mode;
     int32_t wt_pad;
     // maximum cardinality matching: tree of a column, column that reached a
-    // row, frontier bitmaps, per row the best offer (key, column), per tree
-    // its end (key of the last edge, row); mate in/out
+    // row, bitmaps and lists of the levels, per row the best offer (key,
+    // column), per tree its end (key of the last edge, row); mate in/out
     int32_t *mroot;
     int32_t *mrpar;
-    uint32_t *mfront;
-    uint32_t *mnext;
+    uint32_t *mfront;   // bit c: column c is in the frontier
+    uint32_t *mreach;   // bit r: row r was reached in this phase
+    uint32_t *mtmark;   // bit t: tile t, shared by columns, is listed
+    int32_t *mfl;       // columns of the frontier
     Off *mroff;         // per row: the level's best offer (key, column)
     Off *mtend;         // per tree (root column): its end (key of the last edge, row)
-    int32_t *mtouch;    // rows offered something at this level (each once)
+    int32_t *mtouch;    // rows offered something at this level (each once), then
+                        // the columns matched to them
     int32_t *mmate;
     int32_t *mcolof;    // column of every entry
     int32_t *mtiles;    // tiles holding a frontier column, this level
@@ -310,6 +315,10 @@ void launch_greedy_select_begin(const Work *d, const Shape &sh, bool graph,
 void launch_greedy_select_round(const Work *d, const Shape &sh, bool graph,
                                 cudaGraphConditionalHandle h, Sink &k);
 void launch_greedy_select_end_and_flip(const Work *d, const Shape &sh, Sink &k);
+// The checks of the pattern and the entries, and the start marks.
+void launch_check_colptr(const Work *d, const Shape &sh, Sink &k);
+void launch_mark_starts(const Work *d, const Shape &sh, Sink &k);
+void launch_check_entries(const Work *d, const Shape &sh, Sink &k);
 // The column-pointer check with the start marks (k_check_mark).
 void launch_check_mark(const Work *d, const Shape &sh, Sink &k);
 // Weights from matrix values (equilibration, Options A / B).
@@ -320,8 +329,8 @@ void launch_weights(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_load(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_phase(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_level(const Work *d, const Shape &sh, Sink &k);
-// Graph form of a level: its steps, the last one also setting the level
-// loop's condition (no separate condition kernel).
+// Graph form of a level: small levels in a single block, then the steps, the
+// last one also setting the level loop's condition.
 void launch_mcm_level_graph(const Work *d, const Shape &sh, cudaGraphConditionalHandle h,
                             Sink &k);
 void launch_mcm_augment(const Work *d, const Shape &sh, Sink &k);

@@ -20,12 +20,6 @@
 
 namespace awpm {
 
-// Bounded retries for the lock-free arg-max updates (each failed
-// compare-and-swap means another thread stored a strictly better record, so
-// the loop ends long before this; the bound only turns a broken invariant
-// into an error bit instead of a hang).
-constexpr int kCasRetryCap = 1 << 20;
-
 // Closing-edge ranges longer than this go to the warp-cooperative search
 // (shorter ones to a binary search per lane).  On an R-MAT graph of scale 22
 // (n = 4.2 M, 69 M nonzeros) 64 measured 4.5 us per search launch faster
@@ -59,32 +53,6 @@ __device__ __forceinline__ bool gate(const Ctl *ctl)
 {
     return *(volatile const unsigned *)&ctl->err == 0u &&
            *(volatile const int32_t *)&ctl->active != 0;
-}
-
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        v += __shfl_down_sync(FULL_MASK, v, o);
-    return v;
-}
-
-// Sum v over the block and add it to *dst with one atomic.  All threads call.
-__device__ void block_add_u64(unsigned long long v, unsigned long long *dst)
-{
-    __shared__ unsigned long long sm[32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    v = warp_sum_u64(v);
-    __syncthreads();
-    if (lane == 0)
-        sm[wid] = v;
-    __syncthreads();
-    if (wid == 0) {
-        v = (lane < (int)(blockDim.x >> 5)) ? sm[lane] : 0ull;
-        v = warp_sum_u64(v);
-        if (lane == 0 && v)
-            atomicAdd(dst, v);
-    }
 }
 
 // Deterministic block sum (fixed tree).  All threads call.
@@ -2512,13 +2480,6 @@ __global__ void k_export_stepc(const Work *__restrict__ W, double *gain, int32_t
 // end the kept winners are handed to k_flip exactly as Step D hands them:
 // the key column's record names the root, dropped winners get key -1.
 
-__device__ __forceinline__ void warp_add_i32(int v, int32_t *dst)
-{
-    v = __reduce_add_sync(FULL_MASK, v);
-    if ((threadIdx.x & 31) == 0 && v)
-        atomicAdd(dst, v);
-}
-
 // The kernels below take the winners of a bitmap a lane each (for_winners);
 // with a thread per bitmap word, its winners one after another, a solve of a
 // 27-point stencil of 64^3 spent 1.63 ms in them, now 1.23 ms (launch list; most of it launches that
@@ -2657,17 +2618,6 @@ __global__ void k_ps_end(const Work *__restrict__ W)
 // are matched.  Weights are compared through order keys: 64-bit integers
 // ordered like the doubles, so the maxima and minima are plain 64-bit
 // atomics.
-
-constexpr long long kKeyNone = (long long)0x8000000000000000ull;
-
-// Integer ordered like the weight (-0 taken as +0; finite weights only).
-__device__ __forceinline__ long long order_key(double x)
-{
-    long long b = __double_as_longlong(x);
-    if (b == kKeyNone)
-        b = 0;
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
 
 // Clear the matching, the per-round records and the control block.
 __global__ void k_gm_reset(const Work *__restrict__ W)
@@ -2851,466 +2801,6 @@ __global__ void k_gm_rows(const Work *__restrict__ W)
         w.grkey[i] = kKeyNone;
         w.grcol[i] = 0x7fffffff;
     }
-}
-
-// ---------------------------------------------------------------------------
-// Maximum cardinality matching with the heavy-weight tie-break (Section 5.2)
-// ---------------------------------------------------------------------------
-// Phases of breadth-first augmenting-path searches from every free column.
-// Per level, every frontier column offers its rows not reached yet (through
-// unmatched edges); a row goes to the offer with the heaviest edge, then the
-// lowest column (order key and column in one 128-bit record).  A free row so reached ends a path of its tree (the tree keeps
-// the heaviest last edge, then the lowest row, and stops growing); a
-// matched row brings its matched column into the next frontier.  The trees
-// are vertex-disjoint, so all paths found in a phase are augmented at once.
-// A phase that augments nothing ends the search: the matching is maximum.
-// The levels and phases are driven from the host through Ctl::live and
-// Ctl::pass_flips.
-
-// Clear the per-solve state; mr = -1; every row unreached, its offer record
-// empty.
-__global__ void k_mc_reset(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    if (gtid() == 0) {
-        Ctl *c = w.ctl;
-        c->err = 0u;
-        c->active = 1;
-        c->iterations = 0;
-        c->converged = 0;
-        c->live = 0;
-        c->levels = 0ull;
-        c->pass_flips = 0ull;
-        c->cycles = 0ull;
-        c->level_tiles = 0;
-        c->level_listed = 0;
-        c->level_done = 0u;
-        c->touched = 0;
-    }
-    for (int64_t x = gtid(); x < w.n; x += gstride()) {
-        w.mr[x] = -1;
-        w.mrpar[x] = -1;
-        w.mroff[x] = Off{kKeyNone, 0x7fffffff, 0};
-    }
-    const int64_t words = ((int64_t)w.nnz + 31) / 32 + 1;
-    for (int64_t x = gtid(); x < words; x += gstride())
-        w.starts[x] = 0u;
-}
-
-// A column without entries is no error for the maximum matching (it stays
-// unmatched): drop that report of the column-pointer check.
-__global__ void k_mc_allow_empty(const Work *__restrict__ W)
-{
-    Ctl *c = W->ctl;
-    c->nonempty = (c->err & kErrNotPerfect) ? 0 : 1;
-    atomicAnd(&c->err, ~kErrNotPerfect);
-}
-
-// The starting matching: row of every column or -1, each row once, every
-// pair a stored entry (binary search in the sorted column); its size.
-__global__ void k_mc_load(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    unsigned long long have = 0;
-    if (!w.ctl->err) {
-        for (int64_t j = gtid(); j < w.n; j += gstride()) {
-            const int32_t r = w.mmate[j];
-            w.mc[j] = r < 0 ? -1 : r;
-            if (r < 0)
-                continue;
-            if (r >= w.n || atomicCAS(&w.mr[r], -1, (int32_t)j) != -1) {
-                raise_err(w.ctl, kErrNotPerfect);
-                continue;
-            }
-            int32_t lo = w.colptr[j], len = w.colptr[j + 1] - lo;
-            while (len > 0) {
-                const int32_t half = len >> 1;
-                if (w.rowidx[lo + half] < r) {
-                    lo += half + 1;
-                    len -= half + 1;
-                } else {
-                    len = half;
-                }
-            }
-            if (lo >= w.colptr[j + 1] || w.rowidx[lo] != r)
-                raise_err(w.ctl, kErrNotPerfect);
-            ++have;
-        }
-    }
-    block_add_u64(have, &w.ctl->cycles);
-}
-
-// The list of 32-entry tiles holding an entry of a frontier column, built
-// where the frontier is made (the phase start and the end of each level):
-// every frontier column appends the tiles its entries span, one atomic per
-// warp.  A tile shared by two frontier columns is listed twice: the level
-// steps take the same decisions however often, and in whatever order, a
-// tile comes (maxima, minima and writes of equal values), so the list needs
-// neither order nor uniqueness.  It holds at most min(nnz, nnz/32 + 2n)
-// entries (a column spans at most len/32 + 2 tiles, and at most len); an
-// append past the capacity is refused with an internal error.  Called by a
-// whole warp, lane l holding the frontier bits `front` of bitmap word x.
-__device__ __forceinline__ void mc_list_tiles(const Work &w, int64_t x, uint32_t front, int lane)
-{
-    int32_t mine = 0;
-    for (uint32_t bits = front; bits; bits &= bits - 1) {
-        const int64_t c = x * 32 + __ffs(bits) - 1;
-        const int32_t s = __ldg(w.colptr + c), e = __ldg(w.colptr + c + 1);
-        if (e > s)
-            mine += ((e - 1) >> 5) - (s >> 5) + 1;
-    }
-    int32_t incl = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(FULL_MASK, incl, o);
-        if (lane >= o)
-            incl += y;
-    }
-    const int32_t total = __shfl_sync(FULL_MASK, incl, 31);
-    if (total == 0)
-        return;
-    int32_t base = 0;
-    if (lane == 0)
-        base = atomicAdd(&w.ctl->level_tiles, total);
-    base = __shfl_sync(FULL_MASK, base, 0);
-    if ((int64_t)base + total > w.mtiles_cap) {
-        if (lane == 0)
-            raise_err(w.ctl, kErrInternal);
-        return;
-    }
-    int32_t at = base + incl - mine;
-    for (uint32_t bits = front; bits; bits &= bits - 1) {
-        const int64_t c = x * 32 + __ffs(bits) - 1;
-        const int32_t s = __ldg(w.colptr + c), e = __ldg(w.colptr + c + 1);
-        if (e > s)
-            for (int32_t t = s >> 5; t <= ((e - 1) >> 5); ++t)
-                w.mtiles[at++] = t;
-    }
-}
-
-// A phase: every free column roots a tree (its end record cleared) and forms
-// the frontier; rows unreached, offers cleared.  Only the rows the previous
-// phase reached need clearing: a row's offer record fills only at the level
-// that reaches it (its parent is set at that level's join), and the reset
-// cleared every row before the first phase.  End records are read only for
-// the roots of the running phase.
-__global__ void k_mc_phase(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    int live = 0;
-    if (!w.ctl->err) {
-        for (int64_t x = gtid(); x < w.n; x += gstride()) {
-            if (w.mrpar[x] != -1) {
-                w.mrpar[x] = -1;
-                w.mroff[x] = Off{kKeyNone, 0x7fffffff, 0};
-            }
-            if (w.mc[x] < 0) {
-                w.mroot[x] = (int32_t)x;
-                w.mtend[x] = Off{kKeyNone, 0x7fffffff, 0};
-            }
-        }
-        // the frontier and its tile list (the list's count is zero here:
-        // the reset, or the last level of the previous phase, which kept no
-        // column)
-        const int lane = threadIdx.x & 31;
-        const int64_t words = (int64_t)w.n / 32 + 1;
-        for (int64_t x0 = gtid() - lane; x0 < words; x0 += gstride()) {
-            const int64_t x = x0 + lane;
-            uint32_t bits = 0u;
-            if (x < words) {
-                for (int b = 0; b < 32; ++b) {
-                    const int64_t j = x * 32 + b;
-                    if (j < w.n && w.mc[j] < 0)
-                        bits |= 1u << b;
-                }
-                w.mfront[x] = bits;
-                w.mnext[x] = 0u;
-                live += __popc(bits);
-            }
-            mc_list_tiles(w, x, bits, lane);
-        }
-    }
-    if (gtid() == 0) {
-        w.ctl->phase_levels = 0;
-        w.ctl->touched = 0;
-    }
-    warp_add_i32(live, &w.ctl->live);
-}
-
-// Level steps 1-4 run over the listed tiles (one warp per tile): a column of
-// any length, a hub included, is spread over many warps, and the work of a
-// level follows the size of its frontier.  The column of an entry comes from
-// the tile's first column and start bits when no column is empty, else from
-// the colof array.
-#define MC_TILE_LOOP_BEGIN(COUNT)                                                   \
-    const int lane = threadIdx.x & 31;                                              \
-    const int64_t nwarps = gstride() >> 5;                                          \
-    const bool exact = w.ctl->nonempty != 0;                                        \
-    const int64_t listed = (COUNT);                                                 \
-    for (int64_t x = gtid() >> 5; x < listed; x += nwarps) {                        \
-        const int64_t t = w.mtiles[x];                                              \
-        const int32_t p = (int32_t)(t * kTile) + lane;                              \
-        const bool valid = p < w.nnz;                                               \
-        const int32_t c = !valid ? 0                                                \
-                          : exact ? lane_column(__ldg(w.tile_col + t), __ldg(w.starts + t), lane) \
-                                  : __ldg(w.mcolof + p);                            \
-        const bool inf = valid && ((w.mfront[c >> 5] >> (c & 31)) & 1u);           \
-        if (!__any_sync(FULL_MASK, inf))                                            \
-            continue;                                                               \
-        if (!inf)                                                                   \
-            continue;                                                               \
-        const int32_t r = w.rowidx[p];
-#define MC_TILE_LOOP_END }
-
-// (key, who) beats the record cur: heavier key, then lower index.
-__device__ __forceinline__ bool off_better(long long key, int32_t who, const Off &cur)
-{
-    return key > cur.key || (key == cur.key && who < cur.who);
-}
-
-// Fold (key, who) into the record at addr (128-bit compare-and-swap; a
-// failed exchange means another thread stored a better record, so the loop
-// is short; its bound only turns a broken invariant into an error bit).  The
-// first read goes to L2, where the other threads' exchanges land, so fewer
-// exchanges start from a stale copy.
-__device__ bool off_combine(Off *addr, long long key, int32_t who, Ctl *ctl)
-{
-    const int4 v = __ldcg(reinterpret_cast<const int4 *>(addr));
-    Off cur;
-    cur.key = (long long)(((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x);
-    cur.who = v.z;
-    cur.pad = v.w;
-    Off mine{key, who, 0};
-    for (int k = 0; k < kCasRetryCap; ++k) {
-        if (!off_better(key, who, cur))
-            return false;
-        const Off old = atomicCAS(addr, cur, mine);
-        if (old.key == cur.key && old.who == cur.who && old.pad == cur.pad)
-            return old.who == 0x7fffffff;  // this exchange replaced the empty record
-        cur = old;
-    }
-    raise_err(ctl, kErrTimeout);
-    return false;
-}
-
-// Level, step 1: per unreached row the best offer of the level: the
-// heaviest edge from a frontier column, then the lowest column.
-__global__ void k_mc_offer(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    if (w.ctl->err)
-        return;
-    // (the loop of the other level steps, written out: every lane stays to
-    // the warp-wide append of the rows it lists)
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = gstride() >> 5;
-    const bool exact = w.ctl->nonempty != 0;
-    const int64_t listed = w.ctl->level_tiles;
-    for (int64_t x = gtid() >> 5; x < listed; x += nwarps) {
-        const int64_t t = w.mtiles[x];
-        const int32_t p = (int32_t)(t * kTile) + lane;
-        const bool valid = p < w.nnz;
-        const int32_t c = !valid ? 0
-                          : exact ? lane_column(__ldg(w.tile_col + t), __ldg(w.starts + t), lane)
-                                  : __ldg(w.mcolof + p);
-        const bool inf = valid && ((w.mfront[c >> 5] >> (c & 31)) & 1u);
-        if (!__any_sync(FULL_MASK, inf))
-            continue;
-        bool first = false;
-        int32_t r = -1;
-        if (inf) {
-            r = w.rowidx[p];
-            // the exchange that fills a row's empty record lists the row, once
-            if (r != w.mc[c] && w.mrpar[r] == -1)
-                first = off_combine(w.mroff + r, order_key(w.w[p]), c, w.ctl);
-        }
-        const unsigned m = __ballot_sync(FULL_MASK, first);
-        if (m) {
-            int32_t base = 0;
-            if (lane == 0)
-                base = atomicAdd(&w.ctl->touched, __popc(m));
-            base = __shfl_sync(FULL_MASK, base, 0);
-            if (first)
-                w.mtouch[base + __popc(m & ((1u << lane) - 1u))] = r;
-        }
-    }
-}
-
-// Level, step 2: every row offered something at this level (listed by
-// k_mc_offer) joins the tree of its best offer's column.  A free row is a
-// candidate end of the tree: the tree keeps the heaviest last edge, then the
-// lowest row.  A matched row brings its column into the next frontier.
-__global__ void k_mc_join(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    if (w.ctl->err)
-        return;
-    // the next level's tile list starts empty (filled by k_mc_advance)
-    if (gtid() == 0)
-        w.ctl->level_tiles = 0;
-    const int32_t touched = w.ctl->touched;
-    for (int64_t x = gtid(); x < touched; x += gstride()) {
-        const int32_t r = w.mtouch[x];
-        const Off o = w.mroff[r];
-        const int32_t c = o.who;
-        w.mrpar[r] = c;
-        const int32_t t_root = w.mroot[c];
-        const int32_t c2 = w.mr[r];
-        if (c2 < 0) {
-            off_combine(w.mtend + t_root, o.key, r, w.ctl);
-        } else {
-            w.mroot[c2] = t_root;
-            atomicOr(w.mnext + (c2 >> 5), 1u << (c2 & 31));
-        }
-    }
-}
-
-#undef MC_TILE_LOOP_BEGIN
-#undef MC_TILE_LOOP_END
-
-// Column of every entry (a warp per column), for the level kernels.
-__global__ void k_mc_colof(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    if ((w.ctl->err & kErrInvalid) || w.ctl->nonempty)
-        return;
-    const int lane = threadIdx.x & 31;
-    const int64_t nwarps = gstride() >> 5;
-    for (int64_t j = gtid() >> 5; j < w.n; j += nwarps)
-        for (int32_t p = w.colptr[j] + lane; p < w.colptr[j + 1]; p += 32)
-            w.mcolof[p] = (int32_t)j;
-}
-
-// Level, step 3: the next frontier without the trees that have an end; its
-// size into Ctl::live.
-__device__ __forceinline__ void mc_advance(const Work &w)
-{
-    // the next level's offered rows start empty
-    if (gtid() == 0)
-        w.ctl->touched = 0;
-    int live = 0;
-    if (!w.ctl->err) {
-        // the next frontier and its tile list (the list's count was zeroed
-        // by k_mc_join of this level)
-        const int lane = threadIdx.x & 31;
-        const int64_t words = (int64_t)w.n / 32 + 1;
-        for (int64_t x0 = gtid() - lane; x0 < words; x0 += gstride()) {
-            const int64_t x = x0 + lane;
-            uint32_t keep = 0u;
-            if (x < words) {
-                uint32_t bits = w.mnext[x];
-                while (bits) {
-                    const int b = __ffs(bits) - 1;
-                    bits &= bits - 1;
-                    const int32_t c = (int32_t)(x * 32 + b);
-                    if (w.mtend[w.mroot[c]].key == kKeyNone)
-                        keep |= 1u << b;
-                }
-                w.mfront[x] = keep;
-                w.mnext[x] = 0u;
-                live += __popc(keep);
-            }
-            mc_list_tiles(w, x, keep, lane);
-        }
-    }
-    warp_add_i32(live, &w.ctl->live);
-}
-
-__global__ void k_mc_advance(const Work *__restrict__ W)
-{
-    mc_advance(*W);
-}
-
-// The level loop's condition from the live count: count the level, cap the
-// levels of a phase (every level adds a row to the search forest, so n + 1
-// levels mean a broken invariant), continue while a frontier is left.
-__device__ __forceinline__ void mc_level_condition(const Work &w, cudaGraphConditionalHandle h)
-{
-    Ctl *c = w.ctl;
-    const int32_t live = atomicExch(&c->live, 0);
-    if (live > 0) {
-        c->levels += 1;
-        if (++c->phase_levels > w.n + 1)
-            raise_err(c, kErrTimeout);
-    }
-    cudaGraphSetConditional(h, (live > 0 && *(volatile unsigned *)&c->err == 0u) ? 1u : 0u);
-}
-
-// Graph form of step 3: the block that finishes last also sets the level
-// loop's condition (its count of finished blocks orders it after every
-// other block's frontier count).
-__global__ void k_mc_advance_graph(const Work *__restrict__ W, cudaGraphConditionalHandle h)
-{
-    const Work &w = *W;
-    mc_advance(w);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned prev = atomicAdd(&w.ctl->level_done, 1u);
-        if (prev == gridDim.x - 1) {
-            __threadfence();
-            w.ctl->level_done = 0u;
-            mc_level_condition(w, h);
-        }
-    }
-}
-
-// Graph form of the level loop's condition before a phase's first level.
-__global__ void k_mc_cond_level(const Work *__restrict__ W, cudaGraphConditionalHandle h)
-{
-    mc_level_condition(*W, h);
-}
-
-// Graph form of the end of a phase: count it and the paths it augmented;
-// continue while it augmented something.
-__global__ void k_mc_cond_phase(const Work *__restrict__ W, cudaGraphConditionalHandle h)
-{
-    Ctl *c = W->ctl;
-    const unsigned long long aug = c->pass_flips;
-    c->pass_flips = 0ull;
-    c->cycles += aug;
-    c->iterations += 1;
-    const bool go = aug > 0 && c->err == 0u && c->iterations <= W->n;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
-}
-
-// Every tree with an end flips its path; their number into Ctl::pass_flips.
-__global__ void k_mc_augment(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    unsigned long long aug = 0;
-    if (!w.ctl->err) {
-        for (int64_t t = gtid(); t < w.n; t += gstride()) {
-            if (w.mc[t] >= 0 || w.mtend[t].who == 0x7fffffff)
-                continue;
-            int32_t r = w.mtend[t].who;
-            for (int32_t guard = 0; guard <= w.n; ++guard) {
-                const int32_t c = w.mrpar[r];
-                if (c < 0) {  // a broken tree: report instead of walking on
-                    raise_err(w.ctl, kErrInternal);
-                    break;
-                }
-                const int32_t old = w.mc[c];
-                w.mc[c] = r;
-                w.mr[r] = c;
-                if (old < 0)
-                    break;
-                r = old;
-            }
-            ++aug;
-        }
-    }
-    block_add_u64(aug, &w.ctl->pass_flips);
-}
-
-// The result back into the caller's matching array.
-__global__ void k_mc_store(const Work *__restrict__ W)
-{
-    const Work &w = *W;
-    if (w.ctl->err)
-        return;
-    for (int64_t j = gtid(); j < w.n; j += gstride())
-        w.mmate[j] = w.mc[j];
 }
 
 // ---------------------------------------------------------------------------
@@ -3634,72 +3124,28 @@ void launch_greedy_round(const Work *d, const Shape &sh, bool graph, cudaGraphCo
     launch_control(d, sh, graph, h, k);
 }
 
+void launch_check_colptr(const Work *d, const Shape &sh, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    k.launch((const void *)k_check_colptr, init_grid(sh), kThreads, a);
+}
+
+void launch_mark_starts(const Work *d, const Shape &sh, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    k.launch((const void *)k_mark_starts, init_grid(sh), kThreads, a);
+}
+
+void launch_check_entries(const Work *d, const Shape &sh, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    k.launch((const void *)k_gm_check, init_tile_grid(sh), kThreads, a);
+}
+
 void launch_check_mark(const Work *d, const Shape &sh, Sink &k)
 {
     void *a[] = {(void *)&d};
     k.launch((const void *)k_check_mark, init_grid(sh), kThreads, a);
-}
-
-void launch_mcm_load(const Work *d, const Shape &sh, Sink &k)
-{
-    void *a[] = {(void *)&d};
-    k.launch((const void *)k_mc_reset, util_grid(sh), kThreads, a);
-    k.launch((const void *)k_check_colptr, init_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_allow_empty, 1, 1, a);
-    k.launch((const void *)k_mark_starts, init_grid(sh), kThreads, a);
-    k.launch((const void *)k_gm_check, init_tile_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_load, init_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_colof, init_grid(sh), kThreads, a);
-}
-
-void launch_mcm_phase(const Work *d, const Shape &sh, Sink &k)
-{
-    void *a[] = {(void *)&d};
-    k.launch((const void *)k_mc_phase, util_grid(sh), kThreads, a);
-}
-
-void launch_mcm_level(const Work *d, const Shape &sh, Sink &k)
-{
-    void *a[] = {(void *)&d};
-    // one wave of blocks: a level's work follows its frontier, and a small
-    // frontier should not pay for launching idle blocks
-    k.launch((const void *)k_mc_offer, tile_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_join, tile_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_advance, util_grid(sh), kThreads, a);
-}
-
-void launch_mcm_augment(const Work *d, const Shape &sh, Sink &k)
-{
-    void *a[] = {(void *)&d};
-    k.launch((const void *)k_mc_augment, util_grid(sh), kThreads, a);
-}
-
-void launch_mcm_level_graph(const Work *d, const Shape &sh, cudaGraphConditionalHandle h,
-                            Sink &k)
-{
-    void *a[] = {(void *)&d};
-    void *ah[] = {(void *)&d, (void *)&h};
-    k.launch((const void *)k_mc_offer, tile_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_join, tile_grid(sh), kThreads, a);
-    k.launch((const void *)k_mc_advance_graph, util_grid(sh), kThreads, ah);
-}
-
-void launch_mcm_cond_level(const Work *d, const Shape &sh, cudaGraphConditionalHandle h, Sink &k)
-{
-    void *ah[] = {(void *)&d, (void *)&h};
-    k.launch((const void *)k_mc_cond_level, 1, 1, ah);
-}
-
-void launch_mcm_cond_phase(const Work *d, const Shape &sh, cudaGraphConditionalHandle h, Sink &k)
-{
-    void *ah[] = {(void *)&d, (void *)&h};
-    k.launch((const void *)k_mc_cond_phase, 1, 1, ah);
-}
-
-void launch_mcm_store(const Work *d, const Shape &sh, Sink &k)
-{
-    void *a[] = {(void *)&d};
-    k.launch((const void *)k_mc_store, util_grid(sh), kThreads, a);
 }
 
 void launch_export_stepc(const Work *d, const Shape &sh, double *gain, int32_t *row, Sink &k)
