@@ -639,8 +639,8 @@ void ctx_trim(awpm_ctx *c)
                       &c->wpart,   &c->htab,     &c->b_noff,   &c->b_colmat, &c->b_tilemat,
                       &c->b_tlist, &c->b_i32,    &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
-                      &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,    &c->gckey,
-                      &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,    &c->gtdead,
+                      &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,
+                      &c->gmate,   &c->gdead,
                       &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_max,
                       &c->wt_scale, &c->wt_stage, &c->mroot,   &c->mrpar,    &c->mfront,
                       &c->mreach,  &c->mtmark,   &c->mfl,      &c->mroff,    &c->mtend,
@@ -729,9 +729,9 @@ void teardown_ctx(awpm_ctx *c)
                       &c->ctl,     &c->wpart,    &c->htab,     &c->b_noff,   &c->b_colmat,
                       &c->b_tilemat, &c->b_tlist, &c->b_i32,  &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
-                      &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,    &c->gckey,
-                      &c->gcpos,   &c->grkey,    &c->grcol,    &c->gmate,
-                      &c->gtdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
+                      &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,
+                      &c->gmate,
+                      &c->gdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
                       &c->wt_max,  &c->wt_scale, &c->wt_stage,
                       &c->mroot,   &c->mrpar,    &c->mfront,   &c->mreach,   &c->mtmark,
                       &c->mfl,     &c->mroff,
@@ -1457,13 +1457,12 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     AWPM_TRY(ensure(c, c->mc, sizeof(int32_t) * n));
-    AWPM_TRY(ensure(c, c->mr, sizeof(int32_t) * n));
     AWPM_TRY(ensure(c, c->wm, sizeof(double) * n));
-    AWPM_TRY(ensure(c, c->gckey, sizeof(long long) * n));
-    AWPM_TRY(ensure(c, c->gcpos, sizeof(int32_t) * n));
-    AWPM_TRY(ensure(c, c->grkey, sizeof(long long) * n));
-    AWPM_TRY(ensure(c, c->grcol, sizeof(int32_t) * n));
-    AWPM_TRY(ensure(c, c->gtdead, (size_t)ntiles + 1));
+    // (the records share the maximum matching's buffers: the two run one after
+    // the other)
+    AWPM_TRY(ensure(c, c->mroff, sizeof(Off) * n));
+    AWPM_TRY(ensure(c, c->mtend, sizeof(Off) * n));
+    AWPM_TRY(ensure(c, c->gdead, (size_t)ntiles / 8 + 1));
     AWPM_TRY(ensure(c, c->tile_col, sizeof(int32_t) * ((size_t)ntiles + 1)));
     AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
@@ -1492,17 +1491,14 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     AWPM_TRY(stage_in(c, c->s_rowidx, rowidx, (size_t)nnz, l_rowidx, &wk.rowidx));
     AWPM_TRY(stage_in(c, c->s_w, weight, (size_t)nnz, l_w, &wk.w));
     wk.mc = (int32_t *)c->mc.p;
-    wk.mr = (int32_t *)c->mr.p;
     wk.wm = (double *)c->wm.p;
     wk.tile_col = (int32_t *)c->tile_col.p;
     wk.starts = (uint32_t *)c->starts.p;
     wk.ctl = (Ctl *)c->ctl.p;
     wk.wpart = (double *)c->wpart.p;
-    wk.gckey = (long long *)c->gckey.p;
-    wk.gcpos = (int32_t *)c->gcpos.p;
-    wk.grkey = (long long *)c->grkey.p;
-    wk.grcol = (int32_t *)c->grcol.p;
-    wk.gtdead = (uint8_t *)c->gtdead.p;
+    wk.grow = (Off *)c->mroff.p;
+    wk.gcol = (Off *)c->mtend.p;
+    wk.gdead = (uint8_t *)c->gdead.p;
     CUDA_TRY(cudaMemcpyAsync(c->d_work.p, c->h_work, sizeof(Work), cudaMemcpyHostToDevice,
                              c->stream));
     if (host_loop) {

@@ -126,7 +126,7 @@ struct awpm_ctx {
     awpm::DevBuf mc, mr, wm, rr, rsig, colsig, best, dsel, tile_col, starts, ctl, wpart, htab;
     awpm::DevBuf winbits, wkey, bloom;
     awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
-    awpm::DevBuf gckey, gcpos, grkey, grcol, gtdead;  // greedy matching records
+    awpm::DevBuf gdead;                       // greedy matching (records: mroff, mtend)
     awpm::DevBuf gmate;                       // greedy start of awpm_improve_ctx
     awpm::DevBuf psel, pslive, pstaken, psused;  // greedy (Pettie-Sanders) selection
     awpm::DevBuf wt_max, wt_scale, wt_stage;     // weights from matrix values

@@ -95,4 +95,41 @@ __device__ __forceinline__ long long order_key(double x)
     return b ^ ((b >> 63) & 0x7fffffffffffffffll);
 }
 
+// End of a pass (Algorithm 2): count it, stop when nothing was flipped or
+// the pass cap is reached.  An incremental pass counted differences from the
+// pass before.
+__device__ __forceinline__ int control_step(Ctl *ctl, bool inc)
+{
+    if (ctl->err) {
+        ctl->active = 0;
+        return 0;
+    }
+    if (!ctl->active)
+        return 0;
+    const unsigned long long f = ctl->pass_flips;
+    ctl->pass_flips = 0;
+    if (inc) {
+        if (ctl->iterations == 0) {
+            ctl->cur_candidates = ctl->candidates;
+            ctl->cur_found = ctl->found;
+            ctl->cur_positive = ctl->positive;
+        } else {
+            ctl->candidates += ctl->cur_candidates += ctl->d_candidates;
+            ctl->found += ctl->cur_found += ctl->d_found;
+            ctl->positive += ctl->cur_positive += ctl->d_positive;
+            ctl->d_candidates = ctl->d_found = ctl->d_positive = 0;
+        }
+        ctl->last_flips = f;
+    }
+    ctl->iterations += 1;
+    ctl->cycles += f;
+    if (f == 0) {
+        ctl->converged = 1;
+        ctl->active = 0;
+    } else if (ctl->iterations >= ctl->max_passes) {
+        ctl->active = 0;
+    }
+    return ctl->active;
+}
+
 }  // namespace awpm

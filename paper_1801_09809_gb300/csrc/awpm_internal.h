@@ -201,13 +201,12 @@ struct Work {
     Ctl *ctl;
     double *wpart;      // partial sums of the weight reduction
     BatchWork bw;       // batched solve (bw.count > 0), else zero
-    // greedy maximal matching: per column the best free entry (order key,
-    // then position), per row the best free entry (order key, then column)
-    long long *gckey;
-    int32_t *gcpos;
-    long long *grkey;
-    int32_t *grcol;
-    uint8_t *gtdead;    // per tile: every column of the tile is matched
+    // greedy maximal matching: per row the best free entry (order key, column,
+    // round; kMatched once the row is matched), per column (order key,
+    // position, round)
+    Off *grow;
+    Off *gcol;
+    uint8_t *gdead;     // per group of eight tiles: the tiles without a free entry
     // greedy (Pettie-Sanders) selection: per column the first remaining
     // winner touching it; bitmaps of undecided and kept winners and of the
     // columns of kept cycles

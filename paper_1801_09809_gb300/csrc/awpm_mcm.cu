@@ -224,10 +224,10 @@ __device__ __forceinline__ void mc_frontier_made(Ctl *c)
 // blocks orders it after every other block's writes).
 __device__ __forceinline__ bool mc_last_block(Ctl *c)
 {
-    __threadfence();
     __syncthreads();
     if (threadIdx.x != 0)
         return false;
+    __threadfence();
     if (atomicAdd(&c->level_done, 1u) != gridDim.x - 1)
         return false;
     __threadfence();
