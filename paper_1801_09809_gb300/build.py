@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 OBJDIR = os.path.join(ROOT, "_build")
 LIB = os.path.join(HERE, "libawpm.so")
-SOURCES = ["awpm_kernels.cu", "awpm_weights.cu", "awpm_mcm.cu", "awpm_greedy.cu", "awpm_api.cu", "awpm_serve.cu",
+SOURCES = ["awpm_kernels.cu", "awpm_weights.cu", "awpm_mcm.cu", "awpm_greedy.cu", "awpm_small.cu", "awpm_api.cu", "awpm_serve.cu",
            "awpm_noalloc.cu"]
 HEADERS = [os.path.join(CSRC, "awpm_internal.h"), os.path.join(CSRC, "awpm_ctx.h"),
            os.path.join(CSRC, "awpm_dev.h"), os.path.join(CSRC, "awpm_fixed.h"),

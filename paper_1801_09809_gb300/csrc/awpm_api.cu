@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -153,6 +154,29 @@ int32_t inc_min_tiles()
         return kIncTiles;
     }();
     return least;
+}
+
+// Most entries of a single solve by the small-matrix kernel (one cluster of
+// eight blocks).  us per solve, by the kernel against the general path: random
+// n = 300 70 / 138, n = 2,000 with 18,000 entries 75 / 139, 72,000 entries 111
+// / 138, 180,000 entries 158 / 123; banded (19 passes) 4,400 entries 225 / 379,
+// 30,000 entries 423 / 491, 60,000 entries 581 / 500; 5-point 39,000 entries
+// 174 / 188; 27-point 22,000 entries 434 / 546, 51,000 entries 647 / 640.
+constexpr int32_t kSmallOneNnz = 40960;
+// Largest n tried without reading the number of entries first (a round trip
+// of about 10 us): above, an average column of 20 entries is too many.
+constexpr int32_t kSmallOneN = 2048;
+
+// Whether small matrices are solved by a block each (default on; the
+// environment variable AWPM_SMALL=0 switches it off, a tuning knob: results
+// are the same either way).
+bool small_enabled()
+{
+    static const bool on = [] {
+        const char *v = getenv("AWPM_SMALL");
+        return !(v && v[0] == '0' && v[1] == 0);
+    }();
+    return on;
 }
 
 int code_of(unsigned err)
@@ -640,6 +664,7 @@ void ctx_trim(awpm_ctx *c)
                       &c->b_tlist, &c->b_i32,    &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
                       &c->s_row,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,
+                      &c->smallbuf, &c->b_order,
                       &c->gmate,   &c->gdead,
                       &c->psel,    &c->pslive,   &c->pstaken,  &c->psused,   &c->wt_max,
                       &c->wt_scale, &c->wt_stage, &c->mroot,   &c->mrpar,    &c->mfront,
@@ -672,6 +697,7 @@ int setup_ctx(awpm_ctx *c, const awpm_options *opt)
     CUDA_TRY(cudaSetDevice(dev));
     CUDA_TRY(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, dev));
     CUDA_TRY(search_inc_setup());
+    CUDA_TRY(small_setup());
     c->search_wide = default_search_wide();
     for (int b = 0; b < 2; ++b)
         for (int p = 0; p < 2; ++p) {
@@ -730,6 +756,7 @@ void teardown_ctx(awpm_ctx *c)
                       &c->b_tilemat, &c->b_tlist, &c->b_i32,  &c->b_u64,    &c->b_f64,    &c->s_colptr,
                       &c->s_rowidx, &c->s_w,     &c->s_mate,   &c->s_out,    &c->s_gain,
                       &c->s_row,   &c->d_work,   &c->winbits,  &c->wkey,     &c->bloom, &c->incbuf,
+                      &c->smallbuf, &c->b_order,
                       &c->gmate,
                       &c->gdead,  &c->psel,     &c->pslive,   &c->pstaken,  &c->psused,
                       &c->wt_max,  &c->wt_scale, &c->wt_stage,
@@ -756,10 +783,112 @@ void teardown_ctx(awpm_ctx *c)
         cudaEventDestroy(c->ev_a);
     if (c->ev_b)
         cudaEventDestroy(c->ev_b);
+    if (c->small_streams.fork) {
+        for (cudaStream_t s : c->small_streams.side)
+            cudaStreamDestroy(s);
+        for (cudaEvent_t e : c->small_streams.join)
+            cudaEventDestroy(e);
+        cudaEventDestroy(c->small_streams.fork);
+    }
     if (c->own_stream && c->stream)
         cudaStreamDestroy(c->stream);
     cudaGetLastError();
 }
+
+// Copy a batch's per-matrix results to pinned memory.
+int copy_batch_results(awpm_ctx *c, const BatchWork &bw)
+{
+    const int32_t count = bw.count;
+    // per-matrix results: miter, mconv, mnnz (i32), mcycles (u64), mw_in, mw_out (f64)
+    const size_t pm_bytes = (size_t)count * (3 * sizeof(int32_t) + 3 * 8);
+    if (c->h_batch_bytes < pm_bytes) {
+        if (c->h_batch)
+            cudaFreeHost(c->h_batch);
+        c->h_batch = nullptr;
+        c->h_batch_bytes = 0;
+        CUDA_TRY(cudaMallocHost(&c->h_batch, pm_bytes));
+        c->h_batch_bytes = pm_bytes;
+    }
+    char *hb = (char *)c->h_batch;
+    CUDA_TRY(cudaMemcpyAsync(hb, bw.miter, sizeof(int32_t) * 3 * (size_t)count,
+                             cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(hb + 12 * (size_t)count, bw.mcycles, 8 * (size_t)count,
+                             cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(hb + 20 * (size_t)count, bw.mw_in, 16 * (size_t)count,
+                             cudaMemcpyDeviceToHost, c->stream));
+        return AWPM_OK;
+}
+
+// Device arrays of a batch's results (or a single small solve's).
+int batch_arrays(awpm_ctx *c, BatchWork &bw, int32_t count)
+{
+    AWPM_TRY(ensure(c, c->b_i32, sizeof(int32_t) * (5 * (size_t)count + 2 + kSmallClasses)));
+    AWPM_TRY(ensure(c, c->b_u64, sizeof(unsigned long long) * 2 * (size_t)count));
+    AWPM_TRY(ensure(c, c->b_f64, sizeof(double) * 2 * (size_t)count));
+    bw.count = count;
+    int32_t *i32 = (int32_t *)c->b_i32.p;
+    bw.mdone = i32;
+    bw.miter = i32 + count;
+    bw.mconv = i32 + 2 * (size_t)count;
+    bw.mnnz = i32 + 3 * (size_t)count;
+    bw.active = i32 + 5 * (size_t)count;
+    bw.tlist_n = i32 + 5 * (size_t)count + 1;
+    unsigned long long *u64 = (unsigned long long *)c->b_u64.p;
+    bw.mflips = u64;
+    bw.mcycles = u64 + count;
+    double *f64 = (double *)c->b_f64.p;
+    bw.mw_in = f64;
+    bw.mw_out = f64 + count;
+    return AWPM_OK;
+}
+
+// Class of a matrix of n columns for the small-matrix kernel (n at most
+// kSmallMaxN[0]).
+int small_class(int32_t n)
+{
+    return n <= kSmallMaxN[2] ? 2 : n <= kSmallMaxN[1] ? 1 : 0;
+}
+
+// The matrices of a batch by class and, within a class, roughly from the
+// largest to the smallest (buckets of an eighth of an octave), so that the
+// last blocks to run have the short solves.  False when the offsets are not
+// valid or a matrix is too large.
+bool small_batch_order(const int32_t *off, int32_t count, int32_t n, std::vector<int32_t> &order,
+                       int32_t *per_class)
+{
+    constexpr int kBuckets = 8 * 16;
+    if (off[0] != 0 || off[count] != n)
+        return false;
+    std::vector<int32_t> at(kBuckets + 1, 0);
+    std::vector<uint8_t> of((size_t)count);
+    for (int x = 0; x < kSmallClasses; ++x)
+        per_class[x] = 0;
+    for (int32_t b = 0; b < count; ++b) {
+        const int64_t m = (int64_t)off[b + 1] - off[b];
+        if (m < 0 || m > kSmallMaxN[0])
+            return false;
+        ++per_class[small_class((int32_t)m)];
+        // octave and the next three bits, largest first
+        const int l = ilog2(m > 8 ? m : 8);
+        const int bucket = kBuckets - 1 - (8 * (l - 3) + (int)((m >> (l - 3)) & 7));
+        // (class limits fall inside a bucket: the class decides first)
+        of[(size_t)b] = (uint8_t)bucket;
+        ++at[(size_t)bucket + 1];
+    }
+    for (int x = 0; x < kBuckets; ++x)
+        at[(size_t)x + 1] += at[(size_t)x];
+    std::vector<int32_t> by((size_t)count);
+    for (int32_t b = 0; b < count; ++b)
+        by[(size_t)at[of[(size_t)b]]++] = b;
+    int32_t next[kSmallClasses] = {0, per_class[0], per_class[0] + per_class[1]};
+    order.resize((size_t)count);
+    for (int32_t b : by)
+        order[(size_t)next[small_class(off[b + 1] - off[b])]++] = b;
+    return true;
+}
+
+int ctx_enqueue_small(awpm_ctx *c, const Request &r, int32_t nnz, const int32_t *per_class,
+                      int l_colptr, int l_rowidx, int l_w, int l_mate, int l_out);
 
 int ctx_enqueue(awpm_ctx *c, const Request &r)
 {
@@ -792,6 +921,21 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
         l_row < 0 || l_off < 0)
         return AWPM_ERR_INVALID_ARG;
 
+    // Small matrices: a block each, in one kernel.  A single one does not even
+    // have its nnz read back first.
+    const bool small = small_enabled() && !c->general_only && !r.search_only &&
+                       !(c->opt.flags & AWPM_FLAG_TIME_SEARCH) &&
+                       c->opt.select == AWPM_SELECT_STEP_D &&
+                       (c->opt.lookup == AWPM_LOOKUP_AUTO || c->opt.lookup == AWPM_LOOKUP_BSEARCH) &&
+                       r.rowidx && r.weight;
+    if (small && r.count == 0 && n <= kSmallOneN) {
+        const int32_t known = r.nnz >= 0 ? r.nnz : l_colptr == 1 ? -1 : r.colptr[n];
+        // (a size class that once had too many entries has them read first)
+        if (known <= kSmallOneNnz &&
+            (known >= 0 || (l_rowidx == 1 && l_w == 1 && !((c->small_dense >> ilog2(n)) & 1u))))
+            return ctx_enqueue_small(c, r, known, nullptr, l_colptr, l_rowidx, l_w, l_mate, l_out);
+    }
+
     int32_t nnz = r.nnz;
     if (nnz < 0) {
         if (l_colptr == 1) {
@@ -806,6 +950,12 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
     // tile arithmetic is int32: positions up to nnz + 31 must fit
     if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!r.rowidx || !r.weight)))
         return AWPM_ERR_INVALID_ARG;
+    if (small && r.count == 0 && n <= kSmallMaxN[0] && nnz <= kSmallOneNnz)
+        return ctx_enqueue_small(c, r, nnz, nullptr, l_colptr, l_rowidx, l_w, l_mate, l_out);
+    int32_t per_class[kSmallClasses];
+    if (small && r.count > 0 && r.off_host &&
+        small_batch_order(r.off_host, r.count, n, pd.order, per_class))
+        return ctx_enqueue_small(c, r, nnz, per_class, l_colptr, l_rowidx, l_w, l_mate, l_out);
     const bool timed = (c->opt.flags & AWPM_FLAG_TIME_SEARCH) != 0;
     // launch configuration: given, or the autotuner's (AWPM_LOOKUP_AUTO)
     int lookup = pd.lookup;
@@ -985,32 +1135,18 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
     }
     if (count > 0) {
         BatchWork &bw = wk.bw;
-        bw.count = count;
         AWPM_TRY(stage_in(c, c->b_noff, r.n_off, (size_t)count + 1, l_off, &bw.n_off));
         AWPM_TRY(ensure(c, c->b_colmat, sizeof(int32_t) * n));
         AWPM_TRY(ensure(c, c->b_tilemat, sizeof(int32_t) * ((size_t)ntiles + 1)));
-        AWPM_TRY(ensure(c, c->b_i32, sizeof(int32_t) * (5 * (size_t)count + 2)));
+        AWPM_TRY(batch_arrays(c, bw, count));
         AWPM_TRY(ensure(c, c->b_tlist, sizeof(int32_t) * ((size_t)ntiles + 1)));
-        AWPM_TRY(ensure(c, c->b_u64, sizeof(unsigned long long) * 2 * (size_t)count));
-        AWPM_TRY(ensure(c, c->b_f64, sizeof(double) * 2 * (size_t)count));
         bw.colmat = (int32_t *)c->b_colmat.p;
         bw.tilemat = (int32_t *)c->b_tilemat.p;
-        int32_t *i32 = (int32_t *)c->b_i32.p;
-        bw.mdone = i32;
-        bw.miter = i32 + count;
-        bw.mconv = i32 + 2 * (size_t)count;
-        bw.mnnz = i32 + 3 * (size_t)count;
-        bw.active = i32 + 5 * (size_t)count;
-        bw.tlist_n = i32 + 5 * (size_t)count + 1;
         bw.tlist = (int32_t *)c->b_tlist.p;
-        unsigned long long *u64 = (unsigned long long *)c->b_u64.p;
-        bw.mflips = u64;
-        bw.mcycles = u64 + count;
-        double *f64 = (double *)c->b_f64.p;
-        bw.mw_in = f64;
-        bw.mw_out = f64 + count;
         pd.n_off.resize((size_t)count + 1);
-        if (l_off == 1)
+        if (r.off_host)
+            std::memcpy(pd.n_off.data(), r.off_host, sizeof(int32_t) * (count + 1));
+        else if (l_off == 1)
             CUDA_TRY(cudaMemcpyAsync(pd.n_off.data(), r.n_off, sizeof(int32_t) * (count + 1),
                                      cudaMemcpyDeviceToHost, c->stream));
         else
@@ -1053,31 +1189,132 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
                                  l_out == 1 ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                                  c->stream));
     CUDA_TRY(cudaMemcpyAsync(c->h_ctl, wk.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
-    if (count > 0) {
-        // per-matrix results: miter, mconv, mnnz (i32), mcycles (u64), mw_in, mw_out (f64)
-        const size_t pm_bytes = (size_t)count * (3 * sizeof(int32_t) + 3 * 8);
-        if (c->h_batch_bytes < pm_bytes) {
-            if (c->h_batch)
-                cudaFreeHost(c->h_batch);
-            c->h_batch = nullptr;
-            c->h_batch_bytes = 0;
-            CUDA_TRY(cudaMallocHost(&c->h_batch, pm_bytes));
-            c->h_batch_bytes = pm_bytes;
-        }
-        char *hb = (char *)c->h_batch;
-        CUDA_TRY(cudaMemcpyAsync(hb, wk.bw.miter, sizeof(int32_t) * 3 * (size_t)count,
-                                 cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(cudaMemcpyAsync(hb + 12 * (size_t)count, wk.bw.mcycles, 8 * (size_t)count,
-                                 cudaMemcpyDeviceToHost, c->stream));
-        CUDA_TRY(cudaMemcpyAsync(hb + 20 * (size_t)count, wk.bw.mw_in, 16 * (size_t)count,
-                                 cudaMemcpyDeviceToHost, c->stream));
-    }
+    if (count > 0)
+        AWPM_TRY(copy_batch_results(c, wk.bw));
     CUDA_TRY(cudaEventRecord(c->ev_b, c->stream));
     pd.active = true;
     pd.timed = timed && !r.search_only;
     pd.n = n;
     pd.nnz = nnz;
     pd.count = count;
+    return AWPM_OK;
+}
+
+// Enqueue a batch of small matrices (nnz known, per_class given, pd.order
+// filled), or a single one (nnz -1: the kernel reads it).
+int ctx_enqueue_small(awpm_ctx *c, const Request &r, int32_t nnz, const int32_t *per_class,
+                      int l_colptr, int l_rowidx, int l_w, int l_mate, int l_out)
+{
+    Pending &pd = c->pend;
+    const int32_t n = r.n, count = r.count > 0 ? r.count : 1;
+    const int32_t cap = nnz >= 0 ? nnz : kSmallOneNnz;
+    const int32_t max_passes = c->opt.max_iters > 0 ? c->opt.max_iters : AWPM_PASS_CAP;
+    const size_t words = (size_t)cap / 32 + (size_t)count + 1;
+    AWPM_TRY(ensure(c, c->wm, sizeof(double) * n));
+    const void *best_was = c->best.p, *dsel_was = c->dsel.p;
+    AWPM_TRY(ensure(c, c->best, sizeof(Rec) * n));
+    AWPM_TRY(ensure(c, c->dsel, sizeof(Sel) * n));
+    if (c->best.p != best_was || c->dsel.p != dsel_was)
+        c->rec_clean = 0;
+    AWPM_TRY(ensure(c, c->wkey, sizeof(int32_t) * n));
+    AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
+    AWPM_TRY(ensure(c, c->smallbuf, 3 * sizeof(uint32_t) * words));
+    if (l_out != 1)
+        AWPM_TRY(ensure(c, c->mc, sizeof(int32_t) * n));
+    CUDA_TRY(cudaEventRecord(c->ev_a, c->stream));
+    Work &wk = *c->h_work;
+    std::memset(&wk, 0, sizeof(Work));
+    wk.n = n;
+    wk.nnz = nnz;
+    wk.max_passes = max_passes;
+    wk.lookup = AWPM_LOOKUP_BSEARCH;
+    AWPM_TRY(stage_in(c, c->s_colptr, r.colptr, (size_t)n + 1, l_colptr, &wk.colptr));
+    AWPM_TRY(stage_in(c, c->s_rowidx, r.rowidx, (size_t)(nnz > 0 ? nnz : 0), l_rowidx, &wk.rowidx));
+    AWPM_TRY(stage_in(c, c->s_w, r.weight, (size_t)(nnz > 0 ? nnz : 0), l_w, &wk.w));
+    AWPM_TRY(stage_in(c, c->s_mate, r.mate_in, (size_t)n, l_mate, &wk.mate_in));
+    wk.wm = (double *)c->wm.p;
+    wk.best = (Rec *)c->best.p;
+    wk.dsel = (Sel *)c->dsel.p;
+    wk.wkey = (int32_t *)c->wkey.p;
+    wk.ctl = (Ctl *)c->ctl.p;
+    wk.rec_clean =
+        (int64_t)n <= c->rec_clean && c->sel_epoch + max_passes < 0x7fffffff ? 1 : 0;
+    pd.rec_clean_after = std::max<int64_t>(n, wk.rec_clean ? c->rec_clean : 0);
+    pd.rec_clean_capped = 0;
+    pd.epoch0 = wk.rec_clean ? c->sel_epoch : 0;
+    wk.epoch0 = (int32_t)pd.epoch0;
+    c->rec_clean = 0;
+    wk.small_cap = cap;
+    wk.small_fb = (uint32_t *)c->smallbuf.p;
+    wk.small_pb = wk.small_fb + words;
+    wk.small_c0 = (int32_t *)(wk.small_pb + words);
+    wk.small_out = l_out == 1 ? r.mate_out : (int32_t *)c->mc.p;
+    for (int x = 0; x <= kSmallClasses; ++x)
+        wk.small_smem[x] = (int32_t)small_class_smem(x);
+    AWPM_TRY(batch_arrays(c, wk.bw, count));
+    wk.small_next = (int32_t *)c->b_i32.p + 5 * (size_t)count + 2;
+    const Work *d = (const Work *)c->d_work.p;
+    Sink k;
+    k.stream = c->stream;
+    if (r.count > 0) {
+        pd.n_off.assign(r.off_host, r.off_host + count + 1);
+        AWPM_TRY(ensure(c, c->b_order, sizeof(int32_t) * (2 * (size_t)count + 1)));
+        int32_t *dord = (int32_t *)c->b_order.p;
+        // the offsets and the order in one copy
+        pd.order.insert(pd.order.end(), pd.n_off.begin(), pd.n_off.end());
+        CUDA_TRY(cudaMemcpyAsync(dord, pd.order.data(), sizeof(int32_t) * pd.order.size(),
+                                 cudaMemcpyHostToDevice, c->stream));
+        wk.small_order = dord;
+        wk.bw.n_off = dord + count;
+        for (int x = 0, at = 0; x < kSmallClasses; at += per_class[x++]) {
+            wk.small_first[x] = at;
+            wk.small_count[x] = per_class[x];
+        }
+        CUDA_TRY(cudaMemcpyAsync(c->d_work.p, &wk, sizeof(Work), cudaMemcpyHostToDevice,
+                                 c->stream));
+        Shape sh;
+        sh.num_sms = c->num_sms;
+        if (!c->small_streams.fork) {
+            SmallStreams ss;
+            for (cudaStream_t &s : ss.side)
+                CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+            for (cudaEvent_t &e : ss.join)
+                CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+            CUDA_TRY(cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming));
+            c->small_streams = ss;
+        }
+        launch_small_batch(d, sh, per_class, c->small_streams, k);
+    } else {
+        AWPM_TRY(ensure(c, c->winbits, sizeof(uint32_t) * ((size_t)n / 32 + 1)));
+        AWPM_TRY(ensure(c, c->colsig, sizeof(unsigned long long) * n));
+        wk.winbits = (uint32_t *)c->winbits.p;
+        wk.small_sig = (uint32_t *)c->colsig.p;
+        wk.small_off[1] = n;
+        wk.bw.n_off = (const int32_t *)((const char *)d + offsetof(Work, small_off));
+        if (nnz < 0)
+            wk.small_nnz = wk.colptr + n;
+        const size_t need = small_smem(n, kSmallWarps[kSmallOne], true) + 1024;
+        if (need < small_class_smem(kSmallOne))
+            wk.small_smem[kSmallOne] = (int32_t)need;
+        CUDA_TRY(cudaMemcpyAsync(c->d_work.p, &wk, sizeof(Work), cudaMemcpyHostToDevice,
+                                 c->stream));
+        launch_small_one(d, wk.small_smem[kSmallOne], k);
+    }
+    AWPM_TRY(check_sink(k));
+    if (l_out != 1)
+        CUDA_TRY(cudaMemcpyAsync(r.mate_out, wk.small_out, sizeof(int32_t) * n,
+                                 cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(c->h_ctl, wk.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, c->stream));
+    if (r.count > 0)
+        AWPM_TRY(copy_batch_results(c, wk.bw));
+    CUDA_TRY(cudaEventRecord(c->ev_b, c->stream));
+    pd.active = true;
+    pd.small = true;
+    pd.req = r;
+    pd.lookup = AWPM_LOOKUP_BSEARCH;
+    pd.n = n;
+    pd.nnz = nnz;
+    pd.count = r.count;
     return AWPM_OK;
 }
 
@@ -1100,6 +1337,28 @@ int ctx_finish(awpm_ctx *c, awpm_stats *st, awpm_stats *per_matrix)
     }
     CUDA_TRY(cudaEventSynchronize(c->ev_b));
     const Ctl &h = *c->h_ctl;
+    if (pd.small && h.err) {
+        // the general path names the error (or solves what was not for the
+        // small-matrix kernel)
+        Request again = pd.req;
+        if (again.count == 0 && pd.nnz < 0)
+            c->small_dense |= 1u << ilog2(pd.n);
+        const std::vector<int32_t> off = pd.n_off;
+        if (again.off_host)
+            again.off_host = off.data();
+        c->general_only = true;
+        int rc = ctx_enqueue(c, again);
+        c->general_only = false;
+        if (rc != AWPM_OK) {
+            cudaStreamSynchronize(c->stream);
+            cudaGetLastError();
+            c->pend.active = false;
+            return rc;
+        }
+        return ctx_finish(c, st, per_matrix);
+    }
+    if (pd.small && pd.count == 0)
+        pd.nnz = h.small_nnz;
     const int rc = code_of(h.err);
     if (rc != AWPM_OK)
         return rc;
@@ -1396,23 +1655,31 @@ int awpm_improve_batch(awpm_ctx *ctx, int32_t count, const int32_t *n_off, const
         }
         return AWPM_OK;
     }
-    int32_t n = 0;
+    std::vector<int32_t> off;
+    try {
+        off.resize((size_t)count + 1);
+    } catch (const std::bad_alloc &) {
+        return AWPM_ERR_OOM;
+    }
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
         cudaError_t e = cudaSetDevice(ctx->device);
         if (e == cudaSuccess && where(ctx, n_off) == 1)
-            e = cudaMemcpy(&n, n_off + count, sizeof(int32_t), cudaMemcpyDeviceToHost);
+            e = cudaMemcpy(off.data(), n_off, sizeof(int32_t) * off.size(),
+                           cudaMemcpyDeviceToHost);
         else if (e == cudaSuccess)
-            n = n_off[count];
+            std::memcpy(off.data(), n_off, sizeof(int32_t) * off.size());
         if (e != cudaSuccess) {
             note_cuda_error(e, "reading the batch offsets", __LINE__);
             return AWPM_ERR_CUDA;
         }
     }
+    const int32_t n = off[(size_t)count];
     if (n <= 0)
         return AWPM_ERR_INVALID_ARG;
     Request r;
     r.n = n;
+    r.off_host = off.data();
     r.colptr = colptr;
     r.rowidx = rowidx;
     r.weight = weight;

@@ -44,6 +44,7 @@ struct Request {
     int32_t *mate_out = nullptr;
     int32_t count = 0;  // > 0: batched union with offsets n_off
     const int32_t *n_off = nullptr;
+    const int32_t *off_host = nullptr;  // the offsets in host memory
     bool search_only = false;
     double *gain_out = nullptr;
     int32_t *row_out = nullptr;
@@ -79,6 +80,9 @@ struct Pending {
     int64_t epoch0 = 0;
     int passes_enqueued = 0;
     std::vector<int32_t> n_off;  // host copy of the batch offsets
+    bool small = false;          // solved by the small-matrix kernel
+    Request req;                 // the request, to solve it again by the general path
+    std::vector<int32_t> order;  // matrices by class
     int tune_cfg = -1;           // autotuner trial of this solve, or -1
     uint64_t tune_key = 0;
 };
@@ -125,6 +129,10 @@ struct awpm_ctx {
     // per-solve device workspace
     awpm::DevBuf mc, mr, wm, rr, rsig, colsig, best, dsel, tile_col, starts, ctl, wpart, htab;
     awpm::DevBuf winbits, wkey, bloom;
+    awpm::SmallStreams small_streams;  // made by the first small batch
+    awpm::DevBuf smallbuf, b_order;  // small matrices: bits of the entries, order
+    uint32_t small_dense = 0;        // log2(n) classes whose single solves had too many entries
+    bool general_only = false;       // set while a small solve is repeated by the general path
     awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
     awpm::DevBuf gdead;                       // greedy matching (records: mroff, mtend)
     awpm::DevBuf gmate;                       // greedy start of awpm_improve_ctx

@@ -132,4 +132,150 @@ __device__ __forceinline__ int control_step(Ctl *ctl, bool inc)
     return ctl->active;
 }
 
+// ---- gains as integers ----------------------------------------------------------
+// FP64 instructions are scarce on this GPU, so gains are compared through
+// their IEEE bit patterns.  For values in [+0, +inf] the order of the bit
+// patterns read as signed 64-bit integers is the numeric order, and equal
+// patterns are equal values; every stored or compared gain is either +0.0
+// ("none") or a positive gain.
+
+__device__ __forceinline__ long long gbits(double g)
+{
+    return __double_as_longlong(g);
+}
+
+// g > 0.0 exactly as IEEE compares it: sign clear, not zero, not NaN.
+__device__ __forceinline__ bool gain_positive(double g)
+{
+    const long long b = gbits(g);
+    return b > 0ll && b <= 0x7ff0000000000000ll;
+}
+
+// ---- lock-free arg-max records ----------------------------------------------
+
+// (g, p) beats (cg, cp): larger gain, then lower position (gains >= +0).
+__device__ __forceinline__ bool rec_better(double g, int32_t p, double cg, int32_t cp)
+{
+    const long long a = gbits(g), b = gbits(cg);
+    return a > b || (a == b && p < cp);
+}
+
+// Maximum of (g, lowest p) into a Step-C record.
+__device__ __forceinline__ void rec_combine(Rec *addr, Rec mine, Ctl *ctl)
+{
+    Rec cur = *addr;
+    for (int it = 0; it < kCasRetryCap; ++it) {
+        if (!rec_better(mine.g, mine.p, cur.g, cur.p))
+            return;
+        Rec old = atomicCAS(addr, cur, mine);
+        if (__double_as_longlong(old.g) == __double_as_longlong(cur.g) && old.p == cur.p &&
+            old.q == cur.q)
+            return;
+        cur = old;
+    }
+    raise_err(ctl, kErrTimeout);
+}
+
+// (g, j) beats (cg, cj): larger gain, then lower root (gains >= +0).
+__device__ __forceinline__ bool sel_better(double g, int32_t j, double cg, int32_t cj)
+{
+    const long long a = gbits(g), b = gbits(cg);
+    return a > b || (a == b && j < cj);
+}
+
+// A Step-D selection read in one piece: its gain is only meaningful together
+// with its epoch.
+__device__ __forceinline__ Sel ld_sel(const Sel *addr)
+{
+    unsigned long long a, b;
+    asm volatile("{\n\t"
+                 ".reg .b128 t;\n\t"
+                 "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+                 "mov.b128 {%0, %1}, t;\n\t"
+                 "}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(addr)
+                 : "memory");
+    Sel s;
+    s.g = __longlong_as_double((long long)a);
+    s.j = (int32_t)(uint32_t)b;
+    s.epoch = (int32_t)(uint32_t)(b >> 32);
+    return s;
+}
+
+// Maximum of (g, lowest root j) into a Step-D selection (a record of another
+// epoch counts as empty).
+__device__ __forceinline__ void sel_combine(Sel *addr, Sel mine, Ctl *ctl)
+{
+    Sel cur = ld_sel(addr);
+    for (int it = 0; it < kCasRetryCap; ++it) {
+        if (cur.epoch == mine.epoch && !sel_better(mine.g, mine.j, cur.g, cur.j))
+            return;
+        Sel old = atomicCAS(addr, cur, mine);
+        if (__double_as_longlong(old.g) == __double_as_longlong(cur.g) && old.j == cur.j &&
+            old.epoch == cur.epoch)
+            return;
+        cur = old;
+    }
+    raise_err(ctl, kErrTimeout);
+}
+
+// Bitmap words a warp takes at a time when `words` of them are spread over
+// `nwarps` warps: 32 (one per lane) when there are enough, fewer, down to 1,
+// when that keeps more warps busy (the winners' accesses are scattered, so
+// the time goes with the winners that one warp takes in turn).
+__device__ __forceinline__ int words_per_warp(int64_t words, int64_t nwarps)
+{
+    int k = 1;
+    while (k < 32 && k * nwarps < words)
+        k *= 2;
+    return k;
+}
+
+// The winners (set bits) of the bitmap words [x0, x0 + count), count <= 32,
+// 32 winners at a time with every lane busy: the words' bit counts are
+// scanned across the warp, and in each round lane l takes the winner of rank
+// round * 32 + l (found by a binary search over the scan and the word's
+// rank-th set bit).  Calls f(j) on every lane each round, j = -1 for lanes
+// past the last winner.  Called by the whole warp; `clear` zeroes the words
+// as they are read.
+template <typename F>
+__device__ __forceinline__ void for_winners(uint32_t *winbits, int64_t x0, int count,
+                                            int64_t words, int lane, bool clear, F f)
+{
+    const uint32_t mine = lane < count && x0 + lane < words ? winbits[x0 + lane] : 0u;
+    if (clear && mine)
+        winbits[x0 + lane] = 0u;
+    __syncwarp();  // f may set a bit of a cleared word again
+    const int cnt = __popc(mine);
+    int incl = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL_MASK, incl, o);
+        if (lane >= o)
+            incl += y;
+    }
+    const int excl = incl - cnt;
+    const int total = __shfl_sync(FULL_MASK, incl, 31);
+    for (int base = 0; base < total; base += 32) {
+        const int want = base + lane;
+        // the last word whose first rank is <= want
+        int src = 0;
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const int e = __shfl_sync(FULL_MASK, excl, src + step);
+            if (e <= want)
+                src += step;
+        }
+        const int first = __shfl_sync(FULL_MASK, excl, src);
+        const uint32_t word = __shfl_sync(FULL_MASK, mine, src);
+        int32_t j = -1;
+        if (want < total) {
+            const int bit = (int)__fns(word, 0u, want - first + 1);
+            j = (int32_t)((x0 + src) * 32 + bit);
+        }
+        f(j);
+    }
+}
+
 }  // namespace awpm

@@ -23,6 +23,9 @@ constexpr unsigned kErrNotPerfect = 8u;
 constexpr unsigned kErrInternal = 16u;  // a consistency check of the library's own state failed
 constexpr unsigned kErrTimeout = 32u;   // a bounded retry loop or level loop gave up
 constexpr unsigned kErrBounds = 64u;    // AWPM_DEBUG_BOUNDS builds: an index check failed
+constexpr unsigned kErrRetry = 128u;    // small-matrix kernel: something is wrong with the
+                                        // input (or it is not for this kernel); the general
+                                        // path is to solve it
 
 // Public code of a set of device error bits (host side).
 inline int awpm_code_of_bits(unsigned err)
@@ -117,6 +120,8 @@ struct Ctl {
     unsigned long long last_flips;
     double weight_in;
     double weight_out;
+    int32_t small_nnz;           // small single solve: nonzeros
+    int32_t small_pad;
 };
 
 // Batched solve of many independent matrices as one block-diagonal union
@@ -152,6 +157,29 @@ constexpr int kMapSmallBits = 1 << 17;
 constexpr int kMapLargeBits = 1 << 20;
 constexpr unsigned kSmallFlips = 1024;
 
+// Solves of small matrices by one block each: classes of sizes (the largest
+// first), the largest n of each, and the shared memory that a matrix needs
+// with `warps` warps, with or without the columns' signatures (the rings; the
+// column pointers; four bitmaps; signatures; three 16-bit arrays).
+constexpr int kSmallClasses = 3;
+constexpr int32_t kSmallMaxN[kSmallClasses] = {20096, 7168, 2048};
+constexpr int kSmallOne = kSmallClasses;  // the single matrix's class
+constexpr int kSmallWarps[kSmallClasses + 1] = {32, 16, 8, 16};
+__host__ __device__ constexpr size_t small_smem(int32_t n, int warps, bool sigs)
+{
+    return (size_t)warps * 512 + 4 * ((size_t)n + 1) + 16 * ((size_t)n / 32 + 1) +
+           (sigs ? 4 * (size_t)n : 0) + 6 * (size_t)n + 4;
+}
+// Dynamic shared memory of a class's blocks (the largest class keeps no
+// signatures above about 14,700 columns).
+constexpr size_t small_class_smem(int c)
+{
+    // (and room for the bitmap of marked tiles)
+    return c == 0 || c == kSmallOne
+               ? small_smem(kSmallMaxN[0], kSmallWarps[c], false) + 2560
+               : small_smem(kSmallMaxN[c], kSmallWarps[c], true) + 512;
+}
+
 // Descriptor of one solve.  It lives in device memory and every kernel reads
 // it from there, so launch configurations do not depend on the problem and
 // one instantiated CUDA graph serves every problem of a context: a new
@@ -183,6 +211,23 @@ struct Work {
     Sel *dsel;          // Step-D selections
     uint32_t *winbits;  // bit j: column j holds a Step-C winner this pass
     int32_t *wkey;      // key column k of winner j (set by Step D), ~k if dropped
+    // small matrices: numbers of matrices by class (order, first and count of
+    // each class), the classes' queues, found and positive bits of the
+    // matrices' tiles (tile x of matrix b at (p0 >> 5) + b + x, p0 its first
+    // entry), most nonzeros; single solves: where nnz is
+    const int32_t *small_order;
+    int32_t small_first[kSmallClasses];
+    int32_t small_count[kSmallClasses];
+    int32_t small_smem[kSmallClasses + 1];
+    int32_t small_cap;
+    int32_t *small_next;
+    uint32_t *small_fb;
+    uint32_t *small_pb;
+    int32_t *small_c0;      // columns of the tiles' first entries
+    uint32_t *small_sig;    // single solves: the columns' signatures
+    const int32_t *small_nnz;
+    int32_t *small_out;     // the matchings (global rows)
+    int32_t small_off[2];   // single solves: their n_off
     // incremental passes: per entry, a bit each for "closing entry found" and
     // "positive gain" at its last evaluation; per column whose mate changed
     // the row matched to it before; two sets (of alternate passes) of bitmaps:
@@ -291,6 +336,17 @@ struct Sink {
     cudaError_t err = cudaSuccess;
     void launch(const void *func, unsigned grid, unsigned block, void **args, unsigned smem = 0);
 };
+
+// Solves of small matrices: a batch (counts: matrices per class), or one
+// matrix (smem: its Work::small_smem).
+cudaError_t small_setup();
+struct SmallStreams {
+    cudaStream_t side[kSmallClasses - 1] = {};
+    cudaEvent_t fork = nullptr, join[kSmallClasses - 1] = {};
+};
+void launch_small_batch(const Work *d, const Shape &sh, const int32_t *counts,
+                        const SmallStreams &ss, Sink &k);
+void launch_small_one(const Work *d, int32_t smem, Sink &k);
 
 // Launch sequences; `d` is the device copy of the Work.
 void launch_init(const Work *d, const Shape &sh, Sink &k);
