@@ -378,6 +378,17 @@ int build_greedy_graph(awpm_ctx *c, const Shape &sh, cudaGraphExec_t *out)
         rc = AWPM_ERR_CUDA;
         goto done;
     }
+    if (sh.cluster) {
+        // a straight line: the rounds are one kernel
+        launch_greedy_cluster(d, sh, si);
+        launch_weight_sum(d, sh, true, si);
+        if ((e = si.err) != cudaSuccess || (e = cudaGraphInstantiate(out, g_init, 0)) != cudaSuccess) {
+            note_cuda_error(e, "greedy graph", __LINE__);
+            *out = nullptr;
+            rc = AWPM_ERR_CUDA;
+        }
+        goto done;
+    }
     if ((e = cudaGraphAddChildGraphNode(&n_init, top, nullptr, 0, g_init)) != cudaSuccess ||
         (e = cudaGraphConditionalHandleCreate(&h, top, 1, cudaGraphCondAssignDefault)) !=
             cudaSuccess) {
@@ -446,6 +457,17 @@ int build_mcm_graph(awpm_ctx *c, const Shape &sh, cudaGraphExec_t *out)
     if (si.err != cudaSuccess || sf.err != cudaSuccess) {
         note_cuda_error(si.err != cudaSuccess ? si.err : sf.err, "kernel nodes", __LINE__);
         rc = AWPM_ERR_CUDA;
+        goto done;
+    }
+    if (sh.cluster) {
+        // a straight line: the phases and levels are one kernel
+        launch_mcm_cluster(d, sh, si);
+        launch_mcm_store(d, sh, si);
+        if ((e = si.err) != cudaSuccess || (e = cudaGraphInstantiate(out, g_init, 0)) != cudaSuccess) {
+            note_cuda_error(e, "maximum matching graph", __LINE__);
+            *out = nullptr;
+            rc = AWPM_ERR_CUDA;
+        }
         goto done;
     }
     if ((e = cudaGraphAddChildGraphNode(&n_init, top, nullptr, 0, g_init)) != cudaSuccess ||
@@ -740,7 +762,7 @@ void teardown_ctx(awpm_ctx *c)
                                 cudaGraphExecDestroy(g);
                                 g = nullptr;
                             }
-    for (int v = 0; v < 2; ++v) {
+    for (int v = 0; v < 3; ++v) {
         if (c->g_greedy[v]) {
             cudaGraphExecDestroy(c->g_greedy[v]);
             c->g_greedy[v] = nullptr;
@@ -1734,13 +1756,14 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
     AWPM_TRY(ensure(c, c->wpart, sizeof(double) * kWsumBlocks));
-    const Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    sh.cluster = ntiles <= kGmClusterTiles;
     // AWPM_FLAG_TIME_SEARCH: a host loop over the rounds (every kernel a
     // separate stream launch, visible to profilers) instead of the graph
     const bool host_loop = (c->opt.flags & AWPM_FLAG_TIME_SEARCH) != 0;
     cudaGraphExec_t g = nullptr;
     if (!host_loop) {
-        cudaGraphExec_t &gg = c->g_greedy[sh.search_waves - 1];
+        cudaGraphExec_t &gg = c->g_greedy[sh.cluster ? 2 : sh.search_waves - 1];
         if (!gg)
             AWPM_TRY(build_greedy_graph(c, sh, &gg));
         g = gg;
@@ -1866,7 +1889,8 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
         CUDA_TRY(cudaMemcpyAsync(dmate, mate, sizeof(int32_t) * n, cudaMemcpyHostToDevice,
                                  c->stream));
     }
-    const Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    sh.cluster = ntiles <= kMcClusterTiles;
     CUDA_TRY(cudaEventRecord(c->ev_a, c->stream));
     Work &wk = *c->h_work;
     std::memset(&wk, 0, sizeof(Work));
@@ -1900,7 +1924,7 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
     Ctl *dctl = (Ctl *)c->ctl.p;
     if (!(c->opt.flags & AWPM_FLAG_TIME_SEARCH)) {
         // the whole search in one graph launch (loops on the device)
-        cudaGraphExec_t &g = c->g_mcm[sh.search_waves - 1];
+        cudaGraphExec_t &g = c->g_mcm[sh.cluster ? 2 : sh.search_waves - 1];
         if (!g)
             AWPM_TRY(build_mcm_graph(c, sh, &g));
         CUDA_TRY(cudaGraphLaunch(g, c->stream));

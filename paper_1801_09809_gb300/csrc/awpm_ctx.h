@@ -156,8 +156,9 @@ struct awpm_ctx {
     // one instantiated graph per [batch][lookup slot][wide][search waves - 1][select]
     // [passes after the first: whole searches, incremental, incremental large]
     cudaGraphExec_t g_exec[2][3][2][2][2][3] = {};
-    cudaGraphExec_t g_greedy[2] = {};  // greedy matching, [search waves - 1] of the shape
-    cudaGraphExec_t g_mcm[2] = {};     // maximum matching, [search waves - 1] of the shape
+    // greedy and maximum matching, [search waves - 1 of the shape; 2: one cluster]
+    cudaGraphExec_t g_greedy[3] = {};
+    cudaGraphExec_t g_mcm[3] = {};
     std::map<uint64_t, awpm::TuneEntry> tune;  // autotuner state per problem class
     awpm::Pending pend;
     // the request server of this context (awpm_submit), created on first use

@@ -278,4 +278,11 @@ __device__ __forceinline__ void for_winners(uint32_t *winbits, int64_t x0, int c
     }
 }
 
+// Barrier of the cluster's threads, ordering their memory accesses.
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 }  // namespace awpm

@@ -108,9 +108,8 @@ __global__ void k_gm_reset(const Work *__restrict__ W)
 // records.  A column's entries are combined in the warp; the first lane of a
 // column that lies in the tile whole stores its record, a column cut by a
 // tile's end is merged by compare-and-swap.
-__global__ void __launch_bounds__(kThreads, 4) k_gm_best(const Work *__restrict__ W)
+__device__ __forceinline__ void gm_best(const Work &w)
 {
-    const Work &w = *W;
     if (w.ctl->err || !w.ctl->active)
         return;
     constexpr int kU = 4;
@@ -214,6 +213,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_gm_best(const Work *__restrict_
     }
 }
 
+__global__ void __launch_bounds__(kThreads, 4) k_gm_best(const Work *__restrict__ W)
+{
+    gm_best(*W);
+}
+
 // Round, step 2: a free column whose entry is also its row's is matched.
 __device__ __forceinline__ void gm_match(const Work &w)
 {
@@ -259,7 +263,33 @@ __global__ void k_gm_match_graph(const Work *__restrict__ W, cudaGraphConditiona
     }
 }
 
+// All rounds of a small problem in one cluster, with cluster barriers between
+// the steps and no launch per round.
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024)
+    k_gm_cluster(const Work *__restrict__ W)
+{
+    const Work &w = *W;
+    for (;;) {
+        gm_best(w);
+        cluster_sync();
+        gm_match(w);
+        cluster_sync();
+        if (gtid() == 0)
+            control_step(w.ctl, false);
+        cluster_sync();
+        // (last written before the barrier)
+        if (!*(volatile int32_t *)&w.ctl->active)
+            return;
+    }
+}
+
 }  // namespace
+
+void launch_greedy_cluster(const Work *d, const Shape &, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    k.launch((const void *)k_gm_cluster, 8, 1024, a);
+}
 
 void launch_greedy_init(const Work *d, const Shape &sh, Sink &k)
 {

@@ -308,6 +308,14 @@ constexpr int kRsTile = kRsThreads * kRsItems;
 constexpr int kRsBins = 256;
 constexpr int kScanChunk = kRsThreads * 8;
 
+// Most tiles of a problem whose greedy rounds, and whose maximum-matching
+// phases, run in one cluster.  us per call, loops in the graph against one
+// cluster: greedy 16,000 entries 229 / 172, 64,000 248 / 184, 130,000 235 / 237,
+// 260,000 244 / 357 (random; the others alike); maximum matching 16,000 391 /
+// 289, 130,000 757 / 654, 260,000 1,009 / 1,040 (random), 622 / 520 (R-MAT).
+constexpr int32_t kGmClusterTiles = 3584;
+constexpr int32_t kMcClusterTiles = 6144;
+
 // Launch shape of a context: fixed grids sized by the GPU, not the problem.
 struct Shape {
     int num_sms;
@@ -318,6 +326,7 @@ struct Shape {
     int search_waves;   // size class: 2 when there are at least 64 tiles per resident
                         // search warp, else 1 (keys the cached graphs; Step D's grid)
     int select;         // AWPM_SELECT_STEP_D or AWPM_SELECT_GREEDY
+    bool cluster = false;  // greedy and maximum matching: loops run in one cluster
     bool inc = false;   // passes after the first are incremental
     bool large = false; // n > kMapSmallBits: the incremental search's large form
 };
@@ -388,6 +397,8 @@ void launch_mcm_level(const Work *d, const Shape &sh, Sink &k);
 // last one also setting the level loop's condition.
 void launch_mcm_level_graph(const Work *d, const Shape &sh, cudaGraphConditionalHandle h,
                             Sink &k);
+// The phases and levels of a small problem in one kernel.
+void launch_mcm_cluster(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_augment(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_store(const Work *d, const Shape &sh, Sink &k);
 // Graph forms: the condition of the level loop (undecided frontier left),
@@ -400,6 +411,8 @@ void launch_export_stepc(const Work *d, const Shape &sh, double *gain, int32_t *
 // Greedy maximal matching: state reset and input checks; one round (the
 // control kernel ends the loop after a round that matched nothing).
 void launch_greedy_init(const Work *d, const Shape &sh, Sink &k);
+// The rounds of a small problem in one kernel.
+void launch_greedy_cluster(const Work *d, const Shape &sh, Sink &k);
 void launch_greedy_round(const Work *d, const Shape &sh, bool graph, cudaGraphConditionalHandle h,
                          Sink &k);
 // Resident blocks per SM of the search kernel for a lookup strategy.

@@ -239,9 +239,8 @@ __device__ __forceinline__ bool mc_last_block(Ctl *c)
 // the frontier; no row is reached.  (A row's offer record was cleared by the
 // join that reached it.  End records are read only for the roots of the
 // running phase.)
-__global__ void k_mc_phase(const Work *__restrict__ W)
+__device__ __forceinline__ void mc_phase(const Work &w)
 {
-    const Work &w = *W;
     if (!w.ctl->err) {
         const int lane = threadIdx.x & 31;
         const int64_t words = (int64_t)w.n / 32 + 1;
@@ -265,8 +264,13 @@ __global__ void k_mc_phase(const Work *__restrict__ W)
     }
     if (gtid() == 0)
         w.ctl->phase_levels = 0;
-    if (mc_last_block(w.ctl))
-        mc_frontier_made(w.ctl);
+}
+
+__global__ void k_mc_phase(const Work *__restrict__ W)
+{
+    mc_phase(*W);
+    if (mc_last_block(W->ctl))
+        mc_frontier_made(W->ctl);
 }
 
 // (key, who) beats the record cur: heavier key, then lower index.
@@ -520,13 +524,6 @@ __global__ void k_mc_advance_graph(const Work *__restrict__ W, cudaGraphConditio
     }
 }
 
-// Barrier of the cluster's threads, ordering their memory accesses.
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // Graph form, before a level's grid-wide steps: while the frontier is small,
 // one cluster of blocks runs its levels, with cluster barriers between the
 // steps.
@@ -566,23 +563,26 @@ __global__ void k_mc_cond_level(const Work *__restrict__ W, cudaGraphConditional
     cudaGraphSetConditional(h, mc_count_level(*W) ? 1u : 0u);
 }
 
-// Graph form of the end of a phase: count it and the paths it augmented;
-// continue while it augmented something.
-__global__ void k_mc_cond_phase(const Work *__restrict__ W, cudaGraphConditionalHandle h)
+// The end of a phase: count it and the paths it augmented; continue while it
+// augmented something.
+__device__ __forceinline__ bool mc_count_phase(const Work &w)
 {
-    Ctl *c = W->ctl;
+    Ctl *c = w.ctl;
     const unsigned long long aug = c->pass_flips;
     c->pass_flips = 0ull;
     c->cycles += aug;
     c->iterations += 1;
-    const bool go = aug > 0 && c->err == 0u && c->iterations <= W->n;
-    cudaGraphSetConditional(h, go ? 1u : 0u);
+    return aug > 0 && *(volatile unsigned *)&c->err == 0u && c->iterations <= w.n;
+}
+
+__global__ void k_mc_cond_phase(const Work *__restrict__ W, cudaGraphConditionalHandle h)
+{
+    cudaGraphSetConditional(h, mc_count_phase(*W) ? 1u : 0u);
 }
 
 // Every tree with an end flips its path; their number into Ctl::pass_flips.
-__global__ void k_mc_augment(const Work *__restrict__ W)
+__device__ __forceinline__ void mc_augment(const Work &w)
 {
-    const Work &w = *W;
     unsigned long long aug = 0;
     if (!w.ctl->err) {
         for (int64_t t = gtid(); t < w.n; t += gstride()) {
@@ -606,6 +606,52 @@ __global__ void k_mc_augment(const Work *__restrict__ W)
         }
     }
     block_add_u64(aug, &w.ctl->pass_flips);
+}
+
+__global__ void k_mc_augment(const Work *__restrict__ W)
+{
+    mc_augment(*W);
+}
+
+// The whole search of a small problem in one cluster: the phases and their
+// levels with cluster barriers, no launch per step (a phase of the graph is at
+// least eight launches).
+__global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThreads)
+    k_mc_cluster(const Work *__restrict__ W)
+{
+    __shared__ int32_t s_buf[kSmallThreads / 32][kRowBuf];
+    const Work &w = *W;
+    Ctl *c = w.ctl;
+    for (;;) {
+        mc_phase(w);
+        cluster_sync();
+        if (gtid() == 0) {
+            mc_frontier_made(c);
+            mc_count_level(w);
+        }
+        cluster_sync();
+        // (the counters and the error bits are last written before a barrier)
+        while (*(volatile int32_t *)&c->front_n > 0 && *(volatile unsigned *)&c->err == 0u) {
+            mc_offer(w, s_buf[threadIdx.x >> 5]);
+            cluster_sync();
+            mc_join(w);
+            cluster_sync();
+            mc_advance(w);
+            cluster_sync();
+            if (gtid() == 0) {
+                mc_frontier_made(c);
+                mc_count_level(w);
+            }
+            cluster_sync();
+        }
+        mc_augment(w);
+        cluster_sync();
+        if (gtid() == 0)
+            c->active = mc_count_phase(w) ? 1 : 0;
+        cluster_sync();
+        if (!*(volatile int32_t *)&c->active)
+            return;
+    }
 }
 
 // The result back into the caller's matching array.
@@ -662,6 +708,12 @@ void launch_mcm_level_graph(const Work *d, const Shape &sh, cudaGraphConditional
     k.launch((const void *)k_mc_offer, wave(sh, 4), kThreads, a);
     k.launch((const void *)k_mc_join, wave(sh, 8), kThreads, a);
     k.launch((const void *)k_mc_advance_graph, wave(sh, 4), kThreads, ah);
+}
+
+void launch_mcm_cluster(const Work *d, const Shape &, Sink &k)
+{
+    void *a[] = {(void *)&d};
+    k.launch((const void *)k_mc_cluster, kSmallBlocks, kSmallThreads, a);
 }
 
 void launch_mcm_augment(const Work *d, const Shape &sh, Sink &k)

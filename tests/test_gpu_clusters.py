@@ -1,0 +1,83 @@
+"""Greedy and maximum matching around the sizes where their loops move from one
+cluster to the graph (needs a GPU), empty columns and unmatched columns
+included: equal to the oracle on both sides of the line."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1801_09809_gb300 import awpm, gen
+
+pytestmark = pytest.mark.gpu
+GREEDY, MCM = 3584 * 32, 6144 * 32  # most entries of a problem in one cluster
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1801_09809_gb300 import build
+    build.build()
+    c = awpm.awpm_create(device=0)
+    yield c
+    awpm.awpm_destroy(c)
+
+
+def sized(nnz, seed, integer_weights):
+    """About n = nnz / 6 columns, exactly nnz entries: a random graph with
+    entries added to its last columns."""
+    rng = np.random.default_rng(seed)
+    n = nnz // 6
+    g = gen.random_sparse(n, 5, seed)
+    have = g.nnz
+    deg = np.diff(g.colptr)
+    add = np.zeros(n, np.int64)
+    add[n - (nnz - have):] = 1
+    rows = [g.rowidx[g.colptr[j]:g.colptr[j + 1]] for j in range(n)]
+    for j in np.nonzero(add)[0]:
+        r = int(rng.integers(0, n))
+        while r in rows[j]:
+            r = (r + 1) % n
+        rows[j] = np.sort(np.append(rows[j], r)).astype(np.int32)
+    colptr = np.zeros(n + 1, np.int32)
+    np.cumsum(deg + add, out=colptr[1:])
+    rowidx = np.concatenate(rows).astype(np.int32)
+    assert rowidx.size == nnz
+    w = rng.integers(-3, 4, nnz).astype(np.float64) if integer_weights else rng.standard_normal(nnz)
+    return gen.Graph(n, colptr, rowidx, w, g.mate, f"sized({nnz})")
+
+
+@pytest.mark.parametrize("ties", [False, True])
+@pytest.mark.parametrize("nnz", [GREEDY - 31, GREEDY, GREEDY + 1])
+def test_greedy(ctx, nnz, ties):
+    g = sized(nnz, 9970, ties)
+    ref, rst = oracle.get().greedy(g)
+    out = np.empty(g.n, np.int32)
+    st = awpm.awpm_greedy(ctx, g.n, g.colptr, g.rowidx, g.weight, out)
+    assert np.array_equal(out, ref)
+    assert st["cardinality"] == rst["cardinality"] and st["rounds"] == rst["rounds"]
+
+
+@pytest.mark.parametrize("empty", [False, True])
+@pytest.mark.parametrize("nnz", [MCM - 31, MCM, MCM + 1])
+def test_mcm(ctx, nnz, empty):
+    g = sized(nnz, 9980, True)
+    if empty:
+        # the entries of three columns go to their right neighbours' end: the
+        # columns stay empty
+        cp = g.colptr.copy()
+        keep = np.ones(g.nnz, bool)
+        for j in (0, 5, g.n - 1):
+            keep[cp[j]:cp[j + 1]] = False
+        deg = np.add.reduceat(keep, cp[:-1]).astype(np.int32)
+        g.colptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+        g.rowidx, g.weight = g.rowidx[keep], g.weight[keep]
+    rng = np.random.default_rng(3)
+    mate = np.where(rng.random(g.n) < 0.1, -1, g.mate).astype(np.int32)
+    if empty:
+        mate[[0, 5, g.n - 1]] = -1
+    ref, rst = oracle.get().mcm(g, mate)
+    got = mate.copy()
+    st = awpm.awpm_mcm(ctx, g.n, g.colptr, g.rowidx, g.weight, got)
+    assert np.array_equal(got, ref)
+    assert st["cardinality"] == int((ref >= 0).sum())
