@@ -129,11 +129,11 @@ __device__ __forceinline__ int32_t slot_start(int32_t r, int32_t base, int32_t s
 // Long columns are where the 64-bit signature fills up, so this filter keeps
 // most of their absent closing entries away from the search.
 
-// (Filters from 8 or 4 rows up took 8-12 us off a search launch on an
-// R-MAT graph of scale 22, but cost a 27-point stencil of 96^3 8 % and a
-// batch of 4,096 small matrices 2 % of their solve time, so the threshold
-// stays at 32.)
-constexpr int32_t kBloomMin = 32;
+// The line: a filter entry costs the entry pass an atomic (135 of 387 us on
+// the R-MAT graph of scale 22 from 32 rows up), and only the first pass's
+// lookups use many of them.  Whole solves of that graph: 1.447 ms from 32 rows
+// up, 1.435 from 64, 1.439 from 128, 1.53 from 512.
+constexpr int32_t kBloomMin = 64;
 
 __device__ __forceinline__ void bloom_key(int32_t r, int32_t s, int32_t e, uint32_t &word,
                                           uint32_t &bits)
@@ -377,110 +377,191 @@ __global__ void k_mark_starts(const Work *__restrict__ W)
 }
 
 // One pass over the entries: row range, sortedness inside columns, finite
-// weights, the column signatures (OR of sig_mask(row) over each column;
-// lanes of one column are OR-ed in the warp, whole columns stored, columns cut
-// by a tile boundary merged with atomics) and the matched weight of every
-// column: the lane holding (mate_in[j], j) stores its weight as wm[j]; with
-// the binary-search lookup also the Bloom filters of the long columns.  Each
-// warp takes two tiles per round and issues both tiles' loads before using
-// either, so twice the bytes are in flight.  Column numbers come from the
-// start bitmap, exact once no column is empty (empty columns were reported by
-// the column-pointer check and always stay below n).
-#ifndef AWPM_ENTRIES_U
-#define AWPM_ENTRIES_U 2
-#endif
-#ifndef AWPM_ENTRIES_MINB
-#define AWPM_ENTRIES_MINB 6
-#endif
-__global__ void __launch_bounds__(kThreads, AWPM_ENTRIES_MINB) k_entries(const Work *__restrict__ W)
+// weights, the column signatures (OR of sig_mask(row) over each column) and the
+// matched weight of every column: the entry (mate_in[j], j) stores its weight
+// as wm[j]; with the binary-search lookup also the Bloom filters of the long
+// columns.  Column numbers come from the start bitmap, exact once no column is
+// empty (empty columns were reported by the column-pointer check and always
+// stay below n).
+//
+// The kernel is bound by its instructions, not by its 12 bytes per entry, so a
+// lane takes four consecutive entries (a warp 128, with 16-byte loads where the
+// arrays are aligned): rows of one column are OR-ed in the lane, and one
+// segmented ladder over the warp serves four tiles.  A column that lies in the
+// 128 entries whole is stored, one cut by their end merged with atomics.
+// Measured on the R-MAT graph of scale 22: 445 us with a lane per entry (two
+// tiles per round, a ladder each), 387 us so, 252 of them without the
+// filters (three, four and six blocks per SM: 400, 395 and 408 us).
+__global__ void __launch_bounds__(kThreads, 5) k_entries(const Work *__restrict__ W)
 {
     const Work &w = *W;
     if (w.ctl->err & kErrInvalid)
         return;
-    constexpr int kU = AWPM_ENTRIES_U;
     const int lane = threadIdx.x & 31;
-    // 32-bit tile arithmetic: ntiles < 2^26, positions < 2^31
     const int32_t nwarps = (int32_t)(gstride() >> 5);
     const int32_t n = w.n, nnz = w.nnz, ntiles = w.ntiles;
     const int32_t *__restrict__ rowidx = w.rowidx;
+    const double *__restrict__ wv = w.w;
+    const bool aligned = ((((uintptr_t)rowidx) | ((uintptr_t)wv)) & 15u) == 0u;
+    const int32_t blocks = (ntiles + 3) >> 2;
     unsigned bits = 0;
-    for (int32_t t0 = (int32_t)(gtid() >> 5); t0 < ntiles; t0 += kU * nwarps) {
-        int32_t c0[kU], r[kU], prev[kU], mate[kU], j[kU], cs[kU], ce[kU];
-        uint32_t mask[kU];
-        double x[kU];
+    for (int32_t blk = (int32_t)(gtid() >> 5); blk < blocks; blk += nwarps) {
+        const int32_t base = blk * 128;
+        const int32_t p = base + 4 * lane;  // (used where entries are left)
+        int32_t r[4];
+        double x[4];
+        const int32_t left = nnz - base - 4 * lane;
+        const int nv = left >= 4 ? 4 : left;  // entries of this lane (may be <= 0)
+        if (aligned && nnz - base >= 128) {
+            const int4 v = __ldcs(reinterpret_cast<const int4 *>(rowidx + p));
+            const double2 xa = __ldcs(reinterpret_cast<const double2 *>(wv + p));
+            const double2 xb = __ldcs(reinterpret_cast<const double2 *>(wv + p) + 1);
+            r[0] = v.x, r[1] = v.y, r[2] = v.z, r[3] = v.w;
+            x[0] = xa.x, x[1] = xa.y, x[2] = xb.x, x[3] = xb.y;
+        } else {
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int32_t t = t0 + u * nwarps;
-            const bool tv = t < ntiles;
-            const int32_t p = tv ? t * kTile + lane : 0;
-            const bool valid = tv && p < nnz;
-            c0[u] = tv ? __ldg(w.tile_col + t) : 0;
-            mask[u] = tv ? __ldg(w.starts + t) : 1u;
-            r[u] = valid ? __ldcs(rowidx + p) : 0;
-            x[u] = valid ? __ldcs(w.w + p) : 0.0;
-            prev[u] = (valid && lane == 0 && p > 0) ? __ldg(rowidx + p - 1) : 0;
+            for (int u = 0; u < 4; ++u) {
+                r[u] = u < nv ? __ldcs(rowidx + p + u) : 0;
+                x[u] = u < nv ? __ldcs(wv + p + u) : 0.0;
+            }
         }
+        // the lane's tile, its start bits and first column
+        const int32_t t = blk * 4 + (lane >> 3);
+        const int sh = (lane & 7) * 4;
+        const uint32_t word = t < ntiles ? __ldg(w.starts + t) : 0u;
+        const int32_t c0 = t < ntiles ? __ldg(w.tile_col + t) : 0;
+        const int32_t first = lane == 0 && base > 0 ? __ldg(rowidx + base - 1) : 0;
+        // does a column start after the block (or the matrix end there)?
+        const bool ends = nnz - base <= 128 || (__ldg(w.starts + blk * 4 + 4) & 1u);
+        const uint32_t nib = (word >> sh) & 15u;
+        const uint32_t inner = nib & 14u;  // columns starting inside the lane
+        int32_t j[4];
+        j[0] = c0 + __popc(word & ((2u << sh) - 1u) & ~1u);
+        j[1] = j[0] + ((nib >> 1) & 1);
+        j[2] = j[1] + ((nib >> 2) & 1);
+        j[3] = j[2] + ((nib >> 3) & 1);
+        int32_t mate[4];
+        mate[0] = nv > 0 ? __ldg(w.mate_in + j[0]) : -1;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int32_t t = t0 + u * nwarps;
-            const bool valid = t < ntiles && t * kTile + lane < nnz;
-            j[u] = valid ? lane_column(c0[u], mask[u], lane) : -1 - lane;
-            mate[u] = valid ? __ldg(w.mate_in + j[u]) : -1;
-            const bool bl = valid && w.bloom;
-            cs[u] = bl ? __ldg(w.colptr + j[u]) : 0;
-            ce[u] = bl ? __ldg(w.colptr + j[u] + 1) : 0;
+        for (int u = 1; u < 4; ++u)
+            mate[u] = u < nv && ((nib >> u) & 1u) ? __ldg(w.mate_in + j[u]) : -1;
+        // only the lane's first and last columns can be long
+        int32_t s0 = 0, e0 = 0, s3 = 0, e3 = 0;
+        if (w.bloom && nv > 0) {
+            s0 = s3 = __ldg(w.colptr + j[0]);
+            e0 = e3 = __ldg(w.colptr + j[0] + 1);
+            if (inner && nv == 4) {
+                s3 = __ldg(w.colptr + j[3]);
+                e3 = __ldg(w.colptr + j[3] + 1);
+            }
         }
+        int32_t before = __shfl_up_sync(FULL_MASK, r[3], 1);
+        if (lane == 0)
+            before = first;
+        // the lane's OR up to the first inner start (head), from the last one
+        // on (tail), and the columns between
+        uint32_t hl = 0u, hh = 0u, tl = 0u, th = 0u;
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int32_t t = t0 + u * nwarps;
-            const bool tv = t < ntiles;
-            const int32_t base = tv ? t * kTile : 0;
-            const int32_t p = base + lane;
-            const bool valid = tv && p < nnz;
-            const int32_t up = __shfl_up_sync(FULL_MASK, r[u], 1);
-            const int32_t before = lane == 0 ? prev[u] : up;
-            const bool in_range = r[u] >= 0 && r[u] < n;
-            if (valid) {
+        for (int u = 0; u < 4; ++u) {
+            if (u > 0 && !((nib >> u) & 1u))
+                mate[u] = mate[u - 1];
+            if (u > 0 && ((nib >> u) & 1u)) {
+                // a column starts here: the one before ends in this lane
+                if (inner & ((1u << u) - 1u)) {  // and began in it
+                    if (j[u - 1] < n)
+                        w.colsig[j[u - 1]] = ((unsigned long long)th << 32) | tl;
+                } else {
+                    hl = tl;
+                    hh = th;
+                }
+                tl = th = 0u;
+            }
+            if (u < nv) {
+                const bool in_range = r[u] >= 0 && r[u] < n;
                 if (!in_range)
                     bits |= kErrInvalid;
                 if ((__double2hiint(x[u]) & 0x7ff00000) == 0x7ff00000)  // inf or NaN
                     bits |= kErrNonfinite;
-                if (p > 0 && !((mask[u] >> lane) & 1u) && before >= r[u])
+                if (p + u > 0 && !((nib >> u) & 1u) && (u == 0 ? before : r[u - 1]) >= r[u])
                     bits |= kErrUnsorted;
                 if (mate[u] == r[u])
                     w.wm[j[u]] = x[u];
-                if (ce[u] - cs[u] > kBloomMin && in_range) {
-                    uint32_t word, b;
-                    bloom_key(r[u], cs[u], ce[u], word, b);
-                    atomicOr(w.bloom + word, b);
+                if (in_range) {
+                    const uint32_t h = (uint32_t)r[u] * 0x9E3779B1u;  // (sig_mask)
+                    tl |= 1u << (h >> 27);
+                    th |= 1u << ((h >> 22) & 31u);
+                    const bool head = !(inner & ((2u << u) - 1u));
+                    const bool tail = !(inner >> (u + 1));
+                    const int32_t s = head ? s0 : s3, e = head ? e0 : e3;
+                    if ((head || tail) && e - s > kBloomMin) {
+                        uint32_t word_b, b;
+                        bloom_key(r[u], s, e, word_b, b);
+                        atomicOr(w.bloom + word_b, b);
+                    }
                 }
             }
-            unsigned long long v = (valid && in_range) ? sig_mask(r[u]) : 0ull;
-            if (mask[u] <= 1u) {
-                // the whole tile lies in one column: one warp-wide OR
-                const unsigned lo = __reduce_or_sync(FULL_MASK, (unsigned)v);
-                const unsigned hi = __reduce_or_sync(FULL_MASK, (unsigned)(v >> 32));
-                v = ((unsigned long long)hi << 32) | lo;
-            } else {
-                // start bits after this lane (none for lane 31)
-                const uint32_t after = __funnelshift_rc(mask[u], 0u, lane + 1);
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const unsigned long long ov = __shfl_down_sync(FULL_MASK, v, off);
-                    // lane + off is in the same column: no column starts in
-                    // between (past lane 31 the shuffle returns the lane's own
-                    // value, and OR-ing it changes nothing)
-                    if ((after & ((1u << off) - 1u)) == 0u)
-                        v |= ov;
-                }
-            }
-            const bool head = valid && (lane == 0 || ((mask[u] >> lane) & 1u));
-            if (head && j[u] < n) {
-                if (segment_complete(mask[u], lane, base, nnz, w.starts, t))
-                    w.colsig[j[u]] = v;
+        }
+        if (!inner) {
+            hl = tl;
+            hh = th;
+        }
+        if (!__any_sync(FULL_MASK, lane == 0 ? inner : nib)) {
+            // one column: one warp-wide OR
+            const unsigned lo = __reduce_or_sync(FULL_MASK, hl);
+            const unsigned hi = __reduce_or_sync(FULL_MASK, hh);
+            if (lane == 0 && j[0] < n) {
+                const unsigned long long v = ((unsigned long long)hi << 32) | lo;
+                if ((nib & 1u) && ends)
+                    w.colsig[j[0]] = v;
                 else if (v)
-                    atomicOr(w.colsig + j[u], v);
+                    atomicOr(w.colsig + j[0], v);
             }
+            continue;
+        }
+        // head parts of the lanes to the right, as far as the column reaches:
+        // the part of lane l continues in lane l + 1 when no column starts
+        // inside l or at l + 1 (the last lane's after the block)
+        bool next_starts = __shfl_down_sync(FULL_MASK, nib, 1) & 1u;
+        if (lane == 31)
+            next_starts = ends;
+        bool open = !inner && !next_starts;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t l2 = __shfl_down_sync(FULL_MASK, hl, off);
+            const uint32_t h2 = __shfl_down_sync(FULL_MASK, hh, off);
+            const bool o2 = __shfl_down_sync(FULL_MASK, (int)open, off) != 0;
+            if (open && lane + off < 32) {
+                hl |= l2;
+                hh |= h2;
+                open = o2;
+            }
+        }
+        const uint32_t nl = __shfl_down_sync(FULL_MASK, hl, 1);
+        const uint32_t nh = __shfl_down_sync(FULL_MASK, hh, 1);
+        const bool nopen = __shfl_down_sync(FULL_MASK, (int)open, 1) != 0;
+        if (nv > 0 && (lane == 0 || (nib & 1u)) && j[0] < n) {
+            const unsigned long long v = ((unsigned long long)hh << 32) | hl;
+            if ((nib & 1u) && !open)
+                w.colsig[j[0]] = v;
+            else if (v)
+                atomicOr(w.colsig + j[0], v);
+        }
+        if (inner && j[3] < n) {
+            bool more = false;
+            if (!next_starts) {
+                if (lane == 31) {
+                    more = true;
+                } else {
+                    tl |= nl;
+                    th |= nh;
+                    more = nopen;
+                }
+            }
+            const unsigned long long v = ((unsigned long long)th << 32) | tl;
+            if (!more)
+                w.colsig[j[3]] = v;
+            else if (v)
+                atomicOr(w.colsig + j[3], v);
         }
     }
     bits = __reduce_or_sync(FULL_MASK, bits);
