@@ -66,6 +66,18 @@ int scratch_address(unsigned char **out)
     return AWPM_OK;
 }
 
+// The number of entries, read on the device: into the descriptor (0 when it is
+// not one this entry point takes; the pointer check then stops every later
+// kernel) and, as it is, into the control block for the host.
+__global__ void k_noalloc_size(Work *w, const int32_t *nnz_at)
+{
+    const int32_t nnz = *nnz_at;
+    const int32_t use = nnz < 0 || nnz > kMaxNnz ? 0 : nnz;
+    w->ctl->small_nnz = nnz;
+    w->nnz = use;
+    w->ntiles = (use + kTile - 1) / kTile;
+}
+
 bool on_device(const void *p, int device)
 {
     cudaPointerAttributes a;
@@ -105,17 +117,21 @@ extern "C" int awpm_search_noalloc(int32_t n, const int32_t *colptr, const int32
     if (!on_device(colptr, device) || !on_device(mate, device) ||
         !on_device(stepc_gain, device) || !on_device(stepc_row, device))
         return AWPM_ERR_INVALID_ARG;
+    // With both entry arrays in place the kernels read the number of entries
+    // themselves, and the call waits for the device once, at its end; otherwise
+    // it decides whether the arrays are needed.
+    const bool arrays = on_device(rowidx, device) && on_device(weight, device);
     int32_t nnz = 0;
-    if (cudaMemcpyAsync(&nnz, colptr + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) {
-        cudaGetLastError();
-        return AWPM_ERR_CUDA;
+    if (!arrays) {
+        if (cudaMemcpyAsync(&nnz, colptr + n, sizeof(int32_t), cudaMemcpyDeviceToHost, s) !=
+                cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess) {
+            cudaGetLastError();
+            return AWPM_ERR_CUDA;
+        }
+        if (nnz != 0)
+            return AWPM_ERR_INVALID_ARG;
     }
-    if (nnz < 0 || (nnz > 0 && (!on_device(rowidx, device) || !on_device(weight, device))))
-        return AWPM_ERR_INVALID_ARG;
-    if (nnz > kMaxNnz)
-        return AWPM_ERR_TOO_LARGE;
 
     unsigned char *base = nullptr;
     int rc = scratch_address(&base);
@@ -171,9 +187,14 @@ extern "C" int awpm_search_noalloc(int32_t n, const int32_t *colptr, const int32
     sh.search_bps = search_blocks_per_sm(AWPM_LOOKUP_BSEARCH, false, sh.wide);
     sh.lookup = AWPM_LOOKUP_BSEARCH;
     sh.batch = false;
-    sh.search_waves = search_waves(num_sms, sh.search_bps, wk.ntiles);
+    sh.search_waves = 1;
     Sink k;
     k.stream = s;
+    if (arrays) {
+        const int32_t *at = colptr + n;
+        void *a[] = {(void *)&d, (void *)&at};
+        k.launch((const void *)k_noalloc_size, 1, 1, a);
+    }
     launch_init(d, sh, k);
     launch_search(d, sh, k);
     launch_export_stepc(d, sh, stepc_gain, stepc_row, k);
@@ -186,6 +207,13 @@ extern "C" int awpm_search_noalloc(int32_t n, const int32_t *colptr, const int32
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaGetLastError();
         return AWPM_ERR_CUDA;
+    }
+    if (arrays) {
+        nnz = h.small_nnz;
+        if (nnz < 0)
+            return AWPM_ERR_INVALID_ARG;
+        if (nnz > kMaxNnz)
+            return AWPM_ERR_TOO_LARGE;
     }
     if (h.err)
         return awpm_code_of_bits(h.err);
