@@ -97,6 +97,8 @@ struct Ctl {
     int32_t converged;           // last pass flipped nothing
     int32_t max_passes;          // cap on passes
     int32_t live;                // greedy selection: winners still undecided
+    int32_t ps_done;             // greedy selection: the pass was decided by k_ps_small
+    int32_t ps_count;            // its winners, then those undecided
     int32_t nonempty;            // maximum matching: no column is empty
     int32_t phase_levels;        // maximum matching: levels of the running phase
     // maximum matching: tiles and columns listed for the next level (counted

@@ -2393,9 +2393,8 @@ __device__ __forceinline__ void for_all_winners(const Work &w, uint32_t *bits, F
 }
 
 // Keys of all winners; every winner undecided; their number into Ctl::live.
-__global__ void k_ps_begin(const Work *__restrict__ W)
+__device__ __forceinline__ int ps_begin(const Work &w)
 {
-    const Work &w = *W;
     int live = 0;
     if (gate(w.ctl)) {
         const int64_t words = (int64_t)w.n / 32 + 1;
@@ -2408,7 +2407,14 @@ __global__ void k_ps_begin(const Work *__restrict__ W)
             ++live;
         });
     }
-    warp_add_i32(live, &w.ctl->live);
+    return live;
+}
+
+__global__ void k_ps_begin(const Work *__restrict__ W)
+{
+    // (a selection done by k_ps_small leaves nothing to decide)
+    const int live = W->ctl->ps_done ? 0 : ps_begin(*W);
+    warp_add_i32(live, &W->ctl->live);
 }
 
 // Loop condition of the rounds: undecided winners remain (counter reset).
@@ -2421,9 +2427,8 @@ __global__ void k_ps_cond(const Work *__restrict__ W, cudaGraphConditionalHandle
 }
 
 // Round, step 1: every undecided winner names itself at both its columns.
-__global__ void k_ps_name(const Work *__restrict__ W)
+__device__ __forceinline__ void ps_name(const Work &w)
 {
-    const Work &w = *W;
     if (!gate(w.ctl))
         return;
     for_all_winners(w, w.pslive, [&](int32_t j) {
@@ -2437,9 +2442,8 @@ __global__ void k_ps_name(const Work *__restrict__ W)
 
 // Round, step 2: a winner named by both its columns is kept; its columns
 // are marked used.
-__global__ void k_ps_take(const Work *__restrict__ W)
+__device__ __forceinline__ void ps_take(const Work &w)
 {
-    const Work &w = *W;
     if (!gate(w.ctl))
         return;
     for_all_winners(w, w.pslive, [&](int32_t j) {
@@ -2457,9 +2461,8 @@ __global__ void k_ps_take(const Work *__restrict__ W)
 
 // Round, step 3: clear the records this round touched; drop the undecided
 // winners that touch a used column; count the undecided ones left.
-__global__ void k_ps_prune(const Work *__restrict__ W)
+__device__ __forceinline__ int ps_prune(const Work &w)
 {
-    const Work &w = *W;
     int live = 0;
     if (gate(w.ctl)) {
         for_all_winners(w, w.pslive, [&](int32_t j) {
@@ -2477,15 +2480,30 @@ __global__ void k_ps_prune(const Work *__restrict__ W)
                 ++live;
         });
     }
-    warp_add_i32(live, &w.ctl->live);
+    return live;
+}
+
+__global__ void k_ps_name(const Work *__restrict__ W)
+{
+    ps_name(*W);
+}
+
+__global__ void k_ps_take(const Work *__restrict__ W)
+{
+    ps_take(*W);
+}
+
+__global__ void k_ps_prune(const Work *__restrict__ W)
+{
+    const int live = ps_prune(*W);
+    warp_add_i32(live, &W->ctl->live);
 }
 
 // After the rounds: kept winners get their key column's record (the form
 // k_flip reads), dropped ones key -1; the kept-set and used-column bitmaps
 // are cleared for the next pass.
-__global__ void k_ps_end(const Work *__restrict__ W)
+__device__ __forceinline__ void ps_end(const Work &w)
 {
-    const Work &w = *W;
     if (!gate(w.ctl))
         return;
     const int32_t epoch = pass_epoch(w);
@@ -2502,6 +2520,65 @@ __global__ void k_ps_end(const Work *__restrict__ W)
             w.wkey[j] = -1;
         }
     });
+}
+
+__global__ void k_ps_end(const Work *__restrict__ W)
+{
+    if (!W->ctl->ps_done)
+        ps_end(*W);
+}
+
+// The whole selection of a pass with few winners in one cluster of blocks, with
+// cluster barriers between the steps (otherwise five launches or more, each
+// longer than its work).  With more winners it leaves the pass to the kernels
+// above.  Most passes have few: of the 17 of a 27-point stencil of 64^3, ten
+// have less than kPsSmall.
+constexpr int kPsSmall = 8192;
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024)
+    k_ps_small(const Work *__restrict__ W)
+{
+    const Work &w = *W;
+    Ctl *c = w.ctl;
+    // (counted by the blocks' own sums, so that every block decides alike)
+    int mine = 0;
+    if (gate(c))
+        for (int64_t x = gtid(); x < (int64_t)w.n / 32 + 1; x += gstride())
+            mine += __popc(w.winbits[x]);
+    if (gtid() == 0) {
+        c->ps_done = 0;
+        c->ps_count = 0;
+    }
+    cluster_sync();
+    warp_add_i32(mine, &c->ps_count);
+    cluster_sync();
+    const int32_t count = *(volatile int32_t *)&c->ps_count;
+    if (count == 0 || count > kPsSmall)
+        return;
+    ps_begin(w);
+    cluster_sync();
+    for (int round = 0;; ++round) {
+        ps_name(w);
+        cluster_sync();
+        ps_take(w);
+        cluster_sync();
+        const int live = ps_prune(w);
+        if (gtid() == 0)
+            c->ps_count = 0;
+        cluster_sync();
+        warp_add_i32(live, &c->ps_count);
+        cluster_sync();
+        if (*(volatile int32_t *)&c->ps_count == 0)
+            break;
+        if (round > kPsSmall) {  // (every round decides a winner)
+            if (gtid() == 0)
+                raise_err(c, kErrTimeout);
+            break;
+        }
+        cluster_sync();  // (read by all before it is emptied again)
+    }
+    ps_end(w);
+    if (gtid() == 0)
+        c->ps_done = 1;
 }
 
 // ---------------------------------------------------------------------------
@@ -2783,6 +2860,7 @@ void launch_greedy_select_begin(const Work *d, const Shape &sh, bool graph,
 {
     void *a[] = {(void *)&d};
     void *ah[] = {(void *)&d, (void *)&h};
+    k.launch((const void *)k_ps_small, 8, 1024, a);
     k.launch((const void *)k_ps_begin, tile_grid(sh), kThreads, a);
     if (graph)
         k.launch((const void *)k_ps_cond, 1, 1, ah);
