@@ -2008,7 +2008,8 @@ __global__ void __launch_bounds__(IncBlock<kLarge>::kThreads, kLarge ? 1 : 2)
         // (past the end r = -1 may match: masked below)
         if (t0 + step < ntiles)
             fetch(t0 + step);
-        if (!__any_sync(FULL_MASK, hits | marked))
+        unsigned todo = __reduce_or_sync(FULL_MASK, hits) | marked;  // tiles to look at
+        if (!todo)
             continue;
         // words of the chunk's tiles, one tile per lane
         int32_t c0 = 0;
@@ -2028,7 +2029,9 @@ __global__ void __launch_bounds__(IncBlock<kLarge>::kThreads, kLarge ? 1 : 2)
         }
         // (rolled: the row indices are read again, from L1)
 #pragma unroll 1
-        for (int u = 0; u < T; ++u) {
+        while (todo) {
+            const int u = __ffs(todo) - 1;
+            todo &= todo - 1;
             const uint32_t mk = __shfl_sync(FULL_MASK, mask, u);
             const int32_t rank = lane_column(0, mk, lane);
             const uint32_t g = __shfl_sync(FULL_MASK, pw, u);
