@@ -1573,15 +1573,20 @@ int awpm_memory_held(awpm_ctx *ctx, size_t *held, size_t *peak)
 static int solve_sync(awpm_ctx *c, const Request &r, awpm_stats *st, awpm_stats *per_matrix)
 {
     std::lock_guard<std::mutex> lk(c->mu);
-    int rc = ctx_enqueue(c, r);
-    if (rc != AWPM_OK) {
-        if (c->stream)
-            cudaStreamSynchronize(c->stream);
-        cudaGetLastError();
-        c->pend.active = false;
-        return rc;
+    int rc;
+    try {
+        rc = ctx_enqueue(c, r);
+        if (rc == AWPM_OK)
+            return ctx_finish(c, st, per_matrix);
+    } catch (const std::bad_alloc &) {  // (host memory: offsets and order of a batch)
+        c->general_only = false;
+        rc = AWPM_ERR_OOM;
     }
-    return ctx_finish(c, st, per_matrix);
+    if (c->stream)
+        cudaStreamSynchronize(c->stream);
+    cudaGetLastError();
+    c->pend.active = false;
+    return rc;
 }
 
 int awpm_improve_ctx(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *rowidx,
