@@ -76,6 +76,18 @@ void release(awpm_ctx *c, DevBuf &b)
     }
 }
 
+// Give back the buffers of the faster paths if the call does not use them.
+// True if that made room.
+bool release_spares(awpm_ctx *c)
+{
+    if (c->spares_used || !(c->incbuf.p || c->smallbuf.p || c->b_order.p))
+        return false;
+    release(c, c->incbuf);
+    release(c, c->smallbuf);
+    release(c, c->b_order);
+    return true;
+}
+
 int ensure(awpm_ctx *c, DevBuf &b, size_t bytes)
 {
     if (bytes == 0)
@@ -83,21 +95,28 @@ int ensure(awpm_ctx *c, DevBuf &b, size_t bytes)
     if (b.bytes >= bytes)
         return AWPM_OK;
     release(c, b);
+    c->injected = false;
     size_t want = bytes + bytes / 8;  // headroom against small growth steps
     if (c->opt.mem_budget_bytes && c->held + want > c->opt.mem_budget_bytes) {
         want = bytes;
-        if (c->held + want > c->opt.mem_budget_bytes)
+        if (c->held + want > c->opt.mem_budget_bytes &&
+            (!release_spares(c) || c->held + want > c->opt.mem_budget_bytes))
             return AWPM_ERR_BUDGET;
     }
     if (c->fail_after >= 0) {  // injected failure (awpm_inject_alloc_failure)
         if (c->fail_after == 0) {
             c->fail_after = -1;
+            c->injected = true;
             return AWPM_ERR_OOM;
         }
         --c->fail_after;
     }
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, want);
+    if (e == cudaErrorMemoryAllocation && release_spares(c)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, want);
+    }
     if (e != cudaSuccess) {
         note_cuda_error(e, "cudaMalloc", __LINE__);
         cudaGetLastError();
@@ -653,7 +672,8 @@ struct IncLayout {
     }
 };
 
-size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, int select)
+size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, int select,
+                        bool least)
 {
     const size_t N = (size_t)n, Z = (size_t)nnz, T = Z / kTile + 1;
     size_t b = N * (4 + 4 + 8 + sizeof(RowRange) + 8 + 8 + sizeof(Rec) + sizeof(Sel) + 4) + N / 8 +
@@ -669,7 +689,8 @@ size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, in
         b += 4 * (N + 1) + 12 * Z + 8 * N;
     if (select == AWPM_SELECT_GREEDY)  // selection records and three bitmaps
         b += sizeof(Sel) * N + 3 * 4 * (N / 32 + 1);
-    b += IncLayout(n, (int32_t)T).bytes;
+    if (!least)
+        b += IncLayout(n, (int32_t)T).bytes;
     return b + b / 8;
 }
 
@@ -912,9 +933,29 @@ bool small_batch_order(const int32_t *off, int32_t count, int32_t n, std::vector
 int ctx_enqueue_small(awpm_ctx *c, const Request &r, int32_t nnz, const int32_t *per_class,
                       int l_colptr, int l_rowidx, int l_w, int l_mate, int l_out);
 
+int enqueue_once(awpm_ctx *c, const Request &r);
+
 int ctx_enqueue(awpm_ctx *c, const Request &r)
 {
     NvtxRange nvtx_range("enqueue");
+    c->spares_used = false;
+    int rc = enqueue_once(c, r);
+    const bool no_room = rc == AWPM_ERR_BUDGET || (rc == AWPM_ERR_OOM && !c->injected);
+    if (no_room && c->spares_used) {
+        if (c->stream)
+            CUDA_TRY(cudaStreamSynchronize(c->stream));
+        cudaGetLastError();
+        c->spares_used = false;
+        release_spares(c);
+        c->least_memory = true;
+        rc = enqueue_once(c, r);
+        c->least_memory = false;
+    }
+    return rc;
+}
+
+int enqueue_once(awpm_ctx *c, const Request &r)
+{
     Pending &pd = c->pend;
     pd = Pending();
     const int32_t n = r.n;
@@ -945,7 +986,7 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
 
     // Small matrices: a block each, in one kernel.  A single one does not even
     // have its nnz read back first.
-    const bool small = small_enabled() && !c->general_only && !r.search_only &&
+    const bool small = small_enabled() && !c->general_only && !c->least_memory && !r.search_only &&
                        !(c->opt.flags & AWPM_FLAG_TIME_SEARCH) &&
                        c->opt.select == AWPM_SELECT_STEP_D &&
                        (c->opt.lookup == AWPM_LOOKUP_AUTO || c->opt.lookup == AWPM_LOOKUP_BSEARCH) &&
@@ -1058,10 +1099,11 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
     // searches all.
     Shape sh = shape_of(c, count > 0, lookup, wide, ntiles);
     const IncLayout il(n, ntiles);
-    if (count == 0 && !r.search_only && max_passes > 1 && ntiles >= inc_min_tiles()) {
-        const bool injected = c->fail_after == 0;
+    if (count == 0 && !r.search_only && max_passes > 1 && ntiles >= inc_min_tiles() &&
+        !c->least_memory) {
+        c->spares_used = true;
         const int rc = ensure(c, c->incbuf, il.bytes);
-        if (rc == AWPM_ERR_OOM && injected)
+        if (rc == AWPM_ERR_OOM && c->injected)
             return rc;
         sh.inc = rc == AWPM_OK;
         sh.large = sh.inc && il.map_bits > 0;
@@ -1232,6 +1274,7 @@ int ctx_enqueue_small(awpm_ctx *c, const Request &r, int32_t nnz, const int32_t 
     const int32_t cap = nnz >= 0 ? nnz : kSmallOneNnz;
     const int32_t max_passes = c->opt.max_iters > 0 ? c->opt.max_iters : AWPM_PASS_CAP;
     const size_t words = (size_t)cap / 32 + (size_t)count + 1;
+    c->spares_used = true;
     AWPM_TRY(ensure(c, c->wm, sizeof(double) * n));
     const void *best_was = c->best.p, *dsel_was = c->dsel.p;
     AWPM_TRY(ensure(c, c->best, sizeof(Rec) * n));
@@ -1358,6 +1401,7 @@ int ctx_finish(awpm_ctx *c, awpm_stats *st, awpm_stats *per_matrix)
         return AWPM_OK;
     }
     CUDA_TRY(cudaEventSynchronize(c->ev_b));
+    c->spares_used = false;
     const Ctl &h = *c->h_ctl;
     if (pd.small && h.err) {
         // the general path names the error (or solves what was not for the
@@ -1549,7 +1593,8 @@ int awpm_bytes_needed(awpm_ctx *ctx, int32_t n, int32_t nnz, int32_t host_inputs
 {
     if (!ctx || !bytes || n < 0 || nnz < 0)
         return AWPM_ERR_INVALID_ARG;
-    *bytes = ctx_bytes_needed(n, nnz, host_inputs != 0, ctx->opt.lookup, ctx->opt.select);
+    *bytes = ctx_bytes_needed(n, nnz, host_inputs != 0, ctx->opt.lookup, ctx->opt.select,
+                              false);
     return AWPM_OK;
 }
 
@@ -1586,6 +1631,7 @@ static int solve_sync(awpm_ctx *c, const Request &r, awpm_stats *st, awpm_stats 
         cudaStreamSynchronize(c->stream);
     cudaGetLastError();
     c->pend.active = false;
+    c->spares_used = false;
     return rc;
 }
 
@@ -1751,7 +1797,6 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     AWPM_TRY(ensure(c, c->mc, sizeof(int32_t) * n));
-    AWPM_TRY(ensure(c, c->wm, sizeof(double) * n));
     // (the records share the maximum matching's buffers: the two run one after
     // the other)
     AWPM_TRY(ensure(c, c->mroff, sizeof(Off) * n));
@@ -1763,6 +1808,7 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     AWPM_TRY(ensure(c, c->wpart, sizeof(double) * kWsumBlocks));
     Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
     sh.cluster = ntiles <= kGmClusterTiles;
+    sh.greedy = true;
     // AWPM_FLAG_TIME_SEARCH: a host loop over the rounds (every kernel a
     // separate stream launch, visible to profilers) instead of the graph
     const bool host_loop = (c->opt.flags & AWPM_FLAG_TIME_SEARCH) != 0;
@@ -1786,7 +1832,6 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     AWPM_TRY(stage_in(c, c->s_rowidx, rowidx, (size_t)nnz, l_rowidx, &wk.rowidx));
     AWPM_TRY(stage_in(c, c->s_w, weight, (size_t)nnz, l_w, &wk.w));
     wk.mc = (int32_t *)c->mc.p;
-    wk.wm = (double *)c->wm.p;
     wk.tile_col = (int32_t *)c->tile_col.p;
     wk.starts = (uint32_t *)c->starts.p;
     wk.ctl = (Ctl *)c->ctl.p;
@@ -2007,17 +2052,10 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
     return AWPM_OK;
 }
 
-int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *rowidx,
-                 const double *values, int32_t mode, double *weight_out)
+static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *rowidx,
+                        const double *values, int32_t mode, double *weight_out, bool thin)
 {
-    NvtxRange nvtx_range("awpm_weights");
-    if (!ctx || n < 0 || (n > 0 && !colptr) ||
-        (mode != AWPM_WEIGHTS_SUM && mode != AWPM_WEIGHTS_PRODUCT))
-        return AWPM_ERR_INVALID_ARG;
-    std::lock_guard<std::mutex> lk(ctx->mu);
     awpm_ctx *c = ctx;
-    if (n == 0)
-        return AWPM_OK;
     CUDA_TRY(cudaSetDevice(c->device));
     const int l_colptr = where(c, colptr), l_rowidx = where(c, rowidx), l_a = where(c, values),
               l_out = where(c, weight_out);
@@ -2036,9 +2074,11 @@ int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t 
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     AWPM_TRY(ensure(c, c->wt_max, sizeof(unsigned long long) * n));
-    AWPM_TRY(ensure(c, c->wt_scale, sizeof(Scale) * n));
-    AWPM_TRY(ensure(c, c->tile_col, sizeof(int32_t) * ((size_t)ntiles + 1)));
-    AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
+    if (!thin) {
+        AWPM_TRY(ensure(c, c->wt_scale, sizeof(Scale) * n));
+        AWPM_TRY(ensure(c, c->tile_col, sizeof(int32_t) * ((size_t)ntiles + 1)));
+        AWPM_TRY(ensure(c, c->starts, sizeof(uint32_t) * (((size_t)nnz + 31) / 32 + 1)));
+    }
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
     double *dout = weight_out;
     if (l_out != 1) {
@@ -2056,16 +2096,18 @@ int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t 
     AWPM_TRY(stage_in(c, c->s_w, values, (size_t)nnz, l_a, &wk.wt_a));
     wk.wt_out = dout;
     wk.wt_max = (unsigned long long *)c->wt_max.p;
-    wk.wt_scale = (Scale *)c->wt_scale.p;
-    wk.tile_col = (int32_t *)c->tile_col.p;
-    wk.starts = (uint32_t *)c->starts.p;
+    if (!thin) {
+        wk.wt_scale = (Scale *)c->wt_scale.p;
+        wk.tile_col = (int32_t *)c->tile_col.p;
+        wk.starts = (uint32_t *)c->starts.p;
+    }
     wk.wt_mode = mode;
     wk.ctl = (Ctl *)c->ctl.p;
     CUDA_TRY(cudaMemcpyAsync(c->d_work.p, c->h_work, sizeof(Work), cudaMemcpyHostToDevice,
                              c->stream));
     Sink k;
     k.stream = c->stream;
-    launch_weights((const Work *)c->d_work.p, sh, k);
+    launch_weights((const Work *)c->d_work.p, sh, thin, k);
     AWPM_TRY(check_sink(k));
     if (l_out != 1 && nnz > 0)
         CUDA_TRY(cudaMemcpyAsync(weight_out, dout, sizeof(double) * (size_t)nnz,
@@ -2074,6 +2116,29 @@ int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t 
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     // a column without entries is no error here (no matching is asked for)
     return code_of(c->h_ctl->err & ~kErrNotPerfect);
+}
+
+int awpm_weights(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *rowidx,
+                 const double *values, int32_t mode, double *weight_out)
+{
+    NvtxRange nvtx_range("awpm_weights");
+    if (!ctx || n < 0 || (n > 0 && !colptr) ||
+        (mode != AWPM_WEIGHTS_SUM && mode != AWPM_WEIGHTS_PRODUCT))
+        return AWPM_ERR_INVALID_ARG;
+    if (n == 0)
+        return AWPM_OK;
+    std::lock_guard<std::mutex> lk(ctx->mu);
+    int rc = weights_once(ctx, n, colptr, rowidx, values, mode, weight_out, false);
+    if (rc == AWPM_ERR_BUDGET || (rc == AWPM_ERR_OOM && !ctx->injected)) {
+        // no room for the columns' scales and the tiles' columns: the form
+        // that keeps only the row maxima
+        CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+        release(ctx, ctx->wt_scale);
+        release(ctx, ctx->tile_col);
+        release(ctx, ctx->starts);
+        rc = weights_once(ctx, n, colptr, rowidx, values, mode, weight_out, true);
+    }
+    return rc;
 }
 
 int awpm_search(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *rowidx,

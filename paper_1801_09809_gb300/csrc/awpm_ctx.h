@@ -91,12 +91,16 @@ int setup_ctx(struct ::awpm_ctx *c, const awpm_options *opt);
 void teardown_ctx(struct ::awpm_ctx *c);
 // Enqueue a whole solve on the context's stream without waiting for it;
 // the context's done event is recorded after the last copy.
+// Where there is no room for it on the faster path, on the one that needs the
+// least memory.
 int ctx_enqueue(struct ::awpm_ctx *c, const Request &r);
 // Wait for the enqueued solve (a no-op if it already finished) and fill the
 // statistics (per_matrix: count entries for a batch, may be null).
 int ctx_finish(struct ::awpm_ctx *c, awpm_stats *st, awpm_stats *per_matrix);
-// Device bytes a context needs to solve a problem of this size.
-size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, int select);
+// Device bytes a context needs to solve a problem of this size: the least it
+// can do with, or with what the incremental passes take.
+size_t ctx_bytes_needed(int32_t n, int32_t nnz, bool host_inputs, int lookup, int select,
+                        bool least);
 size_t ctx_bytes_held(const struct ::awpm_ctx *c);
 // Free the per-solve workspace of an idle context (its descriptor and graphs
 // stay; the next solve allocates again).
@@ -134,6 +138,13 @@ struct awpm_ctx {
     uint32_t small_dense = 0;        // log2(n) classes whose single solves had too many entries
     bool general_only = false;       // set while a small solve is repeated by the general path
     awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
+    // The buffers that only a faster path needs (incbuf, smallbuf, b_order) are
+    // given back where another allocation finds no room, unless the call being
+    // enqueued uses them; then the call starts again on the path that needs
+    // the least memory.
+    bool spares_used = false;
+    bool least_memory = false;
+    bool injected = false;  // the last failed allocation was the test hook's
     awpm::DevBuf gdead;                       // greedy matching (records: mroff, mtend)
     awpm::DevBuf gmate;                       // greedy start of awpm_improve_ctx
     awpm::DevBuf psel, pslive, pstaken, psused;  // greedy (Pettie-Sanders) selection

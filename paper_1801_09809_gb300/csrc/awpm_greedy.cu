@@ -92,7 +92,6 @@ __global__ void k_gm_reset(const Work *__restrict__ W)
     }
     for (int64_t x = gtid(); x < w.n; x += gstride()) {
         w.mc[x] = -1;
-        w.wm[x] = 0.0;
         w.grow[x] = Off{0, 0, 0};
         w.gcol[x] = Off{0, 0, 0};
     }
@@ -234,7 +233,9 @@ __device__ __forceinline__ void gm_match(const Work &w)
             if (w.grow[i].who != (int32_t)j || w.grow[i].pad != round)
                 continue;
             w.mc[j] = i;
-            w.wm[j] = w.w[c.who];
+            // (a matched column's record is not looked at again: it keeps the
+            // weight for the sum)
+            w.gcol[j].key = __double_as_longlong(w.w[c.who]);
             w.grow[i].pad = kMatched;  // (only this column's thread gets here for row i)
             ++matched;
         }

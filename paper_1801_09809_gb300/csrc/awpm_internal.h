@@ -329,6 +329,7 @@ struct Shape {
                         // search warp, else 1 (keys the cached graphs; Step D's grid)
     int select;         // AWPM_SELECT_STEP_D or AWPM_SELECT_GREEDY
     bool cluster = false;  // greedy and maximum matching: loops run in one cluster
+    bool greedy = false;   // greedy matching: the matched weights are in gcol
     bool inc = false;   // passes after the first are incremental
     bool large = false; // n > kMapSmallBits: the incremental search's large form
 };
@@ -388,7 +389,8 @@ void launch_check_entries(const Work *d, const Shape &sh, Sink &k);
 // The column-pointer check with the start marks (k_check_mark).
 void launch_check_mark(const Work *d, const Shape &sh, Sink &k);
 // Weights from matrix values (equilibration, Options A / B).
-void launch_weights(const Work *d, const Shape &sh, Sink &k);
+// thin: the form without wt_scale, tile_col and starts.
+void launch_weights(const Work *d, const Shape &sh, bool thin, Sink &k);
 // Maximum cardinality matching: load and check the starting matching; start
 // a phase (Ctl::live = free columns); one level of the searches (Ctl::live =
 // next frontier); augment (Ctl::pass_flips = paths augmented); write back.

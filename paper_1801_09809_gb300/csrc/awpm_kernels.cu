@@ -696,13 +696,15 @@ __global__ void __launch_bounds__(kThreads) k_hash_build(const Work *__restrict_
     }
 }
 
+// kGreedy: the weights are in the matched columns' records (gcol).
+template <bool kGreedy>
 __global__ void k_wsum_partial(const Work *__restrict__ W)
 {
     const Work &w = *W;
     double s = 0.0;
     if (w.ctl->err == 0u)
         for (int64_t j = gtid(); j < w.n; j += gstride())
-            s += w.wm[j];
+            s += !kGreedy ? w.wm[j] : w.mc[j] >= 0 ? __longlong_as_double(w.gcol[j].key) : 0.0;
     s = block_sum_f64(s);
     if (threadIdx.x == 0)
         w.wpart[blockIdx.x] = s;
@@ -2738,7 +2740,9 @@ void launch_weight_sum(const Work *d, const Shape &sh, bool out, Sink &k)
     void *ao[] = {(void *)&d, (void *)&o};
     void *af[] = {(void *)&d, (void *)&o, (void *)&parts};
     if (!from_init)
-        k.launch((const void *)k_wsum_partial, kWsumBlocks, kWsumThreads, a);
+        k.launch(sh.greedy ? (const void *)k_wsum_partial<true>
+                           : (const void *)k_wsum_partial<false>,
+                 kWsumBlocks, kWsumThreads, a);
     k.launch((const void *)k_wsum_final, 1, kWsumBlocks, af);
     if (sh.batch)
         k.launch((const void *)k_batch_wsum, util_grid(sh), kThreads, ao);

@@ -171,7 +171,7 @@ void size_item(awpm_server_impl *s, Item *it)
         }
     }
     it->need = ctx_bytes_needed(it->p.n, nnz > 0 ? nnz : 0, it->host_in, s->owner->opt.lookup,
-                                s->owner->opt.select);
+                                s->owner->opt.select, true);
 }
 
 // Pick the queued request to start on free slot k, or -1.  Requests that can
@@ -420,7 +420,7 @@ int awpm_submit(awpm_ctx *ctx, const awpm_problem *p, uint64_t *ticket)
     // a device colptr without nnz is read at admission (size_item)
     it->sized = it->p.nnz >= 0 || p->n == 0 || !p->colptr;
     it->need = ctx_bytes_needed(p->n, it->p.nnz > 0 ? it->p.nnz : 0, it->host_in,
-                                ctx->opt.lookup, ctx->opt.select);
+                                ctx->opt.lookup, ctx->opt.select, true);
     {
         std::lock_guard<std::mutex> lk(s->mu);
         it->ticket = s->next_ticket++;

@@ -87,7 +87,7 @@ __global__ void k_wt_reset(const Work *__restrict__ W)
     for (int64_t x = gtid(); x < w.n; x += gstride()) {
         w.wt_max[x] = 0ull;
     }
-    const int64_t words = ((int64_t)w.nnz + 31) / 32 + 1;
+    const int64_t words = w.starts ? ((int64_t)w.nnz + 31) / 32 + 1 : 0;
     for (int64_t x = gtid(); x < words; x += gstride())
         w.starts[x] = 0u;
 }
@@ -227,7 +227,54 @@ __global__ void __launch_bounds__(kThreads, 6) k_wt_rowmax(const Work *__restric
     }
 }
 
+// The thin form of the column maxima and the row maxima, for where there is no
+// room for the columns' scales and the tiles' columns: a warp per column, its
+// entries read once for the checks and, when all are good, twice for the
+// maximum and the quotients.
+__global__ void __launch_bounds__(kThreads) k_wt_thin_check(const Work *__restrict__ W)
+{
+    const Work &w = *W;
+    if (w.ctl->err & kErrInvalid)
+        return;
+    unsigned bits = 0;
+    for (int64_t p = gtid(); p < w.nnz; p += gstride()) {
+        const int32_t r = w.rowidx[p];
+        const unsigned long long v = fx_bits(w.wt_a[p]) & kAbs;
+        if (r < 0 || r >= w.n)
+            bits |= kErrInvalid;
+        if (v == 0ull || v >= 0x7ff0000000000000ull)
+            bits |= kErrNonfinite;
+    }
+    bits = __reduce_or_sync(FULL_MASK, bits);
+    if ((threadIdx.x & 31) == 0 && bits)
+        raise_err(w.ctl, bits);
+}
+
+__global__ void __launch_bounds__(kThreads) k_wt_thin_rowmax(const Work *__restrict__ W)
+{
+    const Work &w = *W;
+    if (!wt_gate(w.ctl))
+        return;
+    const int lane = threadIdx.x & 31;
+    for (int64_t j = gtid() >> 5; j < w.n; j += gstride() >> 5) {
+        const int32_t p0 = w.colptr[j], p1 = w.colptr[j + 1];
+        unsigned long long m = 0ull;
+        for (int64_t p = (int64_t)p0 + lane; p < p1; p += 32)
+            m = max(m, fx_bits(w.wt_a[p]) & kAbs);
+#pragma unroll
+        for (int off = 16; off; off >>= 1)
+            m = max(m, __shfl_xor_sync(FULL_MASK, m, off));
+        const Scale s = make_scale(m);
+        for (int64_t p = (int64_t)p0 + lane; p < p1; p += 32) {
+            const unsigned long long q = divide(fx_bits(w.wt_a[p]) & kAbs, s);
+            w.wt_out[p] = fx_double(q);
+            atomicMax(w.wt_max + w.rowidx[p], q);
+        }
+    }
+}
+
 // The weights, from the column-scaled magnitudes and the row maxima.
+template <bool kThin>
 __global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
 {
     __shared__ LogEntry s_log[512];
@@ -258,7 +305,7 @@ __global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
             s[u].v = kFxOne;
             s[u].inv = 0;
             if (r[u] >= 0)
-                s[u] = ld_scale(w.wt_scale + r[u]);
+                s[u] = kThin ? make_scale(__ldg(w.wt_max + r[u])) : ld_scale(w.wt_scale + r[u]);
         }
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
@@ -280,17 +327,24 @@ __global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
 
 }  // namespace
 
-void launch_weights(const Work *d, const Shape &sh, Sink &k)
+void launch_weights(const Work *d, const Shape &sh, bool thin, Sink &k)
 {
     void *a[] = {(void *)&d};
     const unsigned grid = (unsigned)(sh.num_sms * 8);
     k.launch((const void *)k_wt_reset, grid, kThreads, a);
+    if (thin) {
+        launch_check_colptr(d, sh, k);
+        k.launch((const void *)k_wt_thin_check, 2 * grid, kThreads, a);
+        k.launch((const void *)k_wt_thin_rowmax, 2 * grid, kThreads, a);
+        k.launch((const void *)k_wt_out<true>, 2 * grid, kThreads, a);
+        return;
+    }
     launch_check_mark(d, sh, k);
     k.launch((const void *)k_wt_colmax, 2 * grid, kThreads, a);
     k.launch((const void *)k_wt_scale, grid, kThreads, a);
     k.launch((const void *)k_wt_rowmax, 2 * grid, kThreads, a);
     k.launch((const void *)k_wt_scale, grid, kThreads, a);
-    k.launch((const void *)k_wt_out, 2 * grid, kThreads, a);
+    k.launch((const void *)k_wt_out<false>, 2 * grid, kThreads, a);
 }
 
 }  // namespace awpm

@@ -96,3 +96,45 @@ def test_budget_without_room(torch):
         assert awpm.awpm_memory_held(c)[1] <= held - buffer
     finally:
         awpm.awpm_destroy(c)
+
+
+@forced
+def test_budget_buffer_before_staging(torch):
+    """Host arrays are staged after the incremental buffer is taken: where the
+    two don't fit together the buffer is given back; and a buffer kept from an
+    earlier solve makes room for another entry point."""
+    g = CASES["banded_131073"]()
+    ref, rst, _ = oracle.get().improve(g)
+    sizes = []
+    for passes in (0, 1):  # (one pass needs no buffer)
+        c = awpm.awpm_create(device=0, lookup=awpm.LOOKUP_BSEARCH, max_iters=passes)
+        run_gpu(c, g)
+        sizes.append(awpm.awpm_memory_held(c)[0])
+        awpm.awpm_destroy(c)
+    held, buffer = sizes[0], sizes[0] - sizes[1]
+    # The mate array is staged last, 4 n with n / 2 of headroom: a budget short
+    # of all that by 2 n has no room for it beside the buffer.
+    assert buffer > 2 * g.n
+    budget = held - 2 * g.n
+    c = awpm.awpm_create(device=0, lookup=awpm.LOOKUP_BSEARCH, mem_budget_bytes=budget)
+    try:
+        for _ in range(2):
+            got, st = run_gpu(c, g)
+            assert_same_as_oracle(g, got, st, ref, rst, "budget")
+            assert awpm.awpm_memory_held(c)[1] <= budget
+    finally:
+        awpm.awpm_destroy(c)
+    # the search's staged results (12 n, 13.5 n with headroom) have room only in
+    # the buffer's place
+    budget = held + max(0, 14 * g.n - buffer)
+    assert budget < held + 12 * g.n
+    c = awpm.awpm_create(device=0, lookup=awpm.LOOKUP_BSEARCH, mem_budget_bytes=budget)
+    gain, row = np.empty(g.n), np.empty(g.n, np.int32)
+    try:
+        run_gpu(c, g)
+        awpm.awpm_search(c, g.n, g.colptr, g.rowidx, g.weight, g.mate, gain, row)
+        assert awpm.awpm_memory_held(c)[1] <= budget
+        got, st = run_gpu(c, g)
+        assert_same_as_oracle(g, got, st, ref, rst, "after the search")
+    finally:
+        awpm.awpm_destroy(c)

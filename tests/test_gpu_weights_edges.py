@@ -76,3 +76,44 @@ def test_edges(ctx, name, span, mode):
             fine = np.isfinite(want)
             assert np.array_equal(got[~fine], want[~fine], equal_nan=True)
             assert np.all(np.abs(got[fine] - want[fine]) <= 2 * np.spacing(np.abs(want[fine])))
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("where", ["device", "in_place", "host"])
+def test_budget_without_room(ctx, mode, where):
+    """A budget that holds the row maxima and the staged arrays but neither the
+    columns' scales nor the tiles' columns gives the same bits."""
+    import torch
+    n, colptr, rowidx, a = matrix(CASES["empty_columns"] * 40 + [3000] + [0, 1, 2, 40] * 100, 5, 300)
+
+    def solve(c, a):
+        if where == "host":
+            out = np.empty_like(a)
+            awpm.awpm_weights(c, n, colptr, rowidx, a, mode, out)
+            return out
+        cp, ri, av = (torch.from_numpy(x).cuda() for x in (colptr, rowidx, a))
+        out = av if where == "in_place" else torch.empty_like(av)
+        awpm.awpm_weights(c, n, cp, ri, av, mode, out)
+        return out.cpu().numpy()
+
+    full = awpm.awpm_create(device=0)
+    want = solve(full, a)
+    held = awpm.awpm_memory_held(full)[0]
+    awpm.awpm_destroy(full)
+    # Allocations take an eighth of headroom while it fits, so a budget short of
+    # what the full form held by 18 n (its scales, with their headroom) has
+    # room for the thin form; the full form could save only the headroom of its
+    # last allocation, at most nnz bytes.
+    assert a.size < 18 * n
+    budget = held - 18 * n
+    c = awpm.awpm_create(device=0, mem_budget_bytes=budget)
+    try:
+        assert np.array_equal(solve(c, a), want, equal_nan=True)
+        assert awpm.awpm_memory_held(c)[1] <= budget
+        bad = a.copy()
+        bad[a.size // 2] = 0.0
+        with pytest.raises(awpm.AwpmError):
+            solve(c, bad)
+        assert np.array_equal(solve(c, a), want, equal_nan=True)
+    finally:
+        awpm.awpm_destroy(c)
