@@ -2073,6 +2073,8 @@ static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const i
     if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!rowidx || !values || !weight_out)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
+    const bool small = ntiles <= kWtClusterTiles;
+    thin = thin || ntiles <= kWtThinTiles;
     AWPM_TRY(ensure(c, c->wt_max, sizeof(unsigned long long) * n));
     if (!thin) {
         AWPM_TRY(ensure(c, c->wt_scale, sizeof(Scale) * n));
@@ -2085,7 +2087,8 @@ static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const i
         AWPM_TRY(ensure(c, c->wt_stage, sizeof(double) * (size_t)nnz));
         dout = (double *)c->wt_stage.p;
     }
-    const Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
+    sh.cluster = small;
     Work &wk = *c->h_work;
     std::memset(&wk, 0, sizeof(Work));
     wk.n = n;

@@ -16,7 +16,8 @@
 //
 // The work is spread by entries (a warp per 32-entry tile, four tiles per
 // round with their loads side by side), not by columns: a warp per column
-// left most lanes idle on short columns and one warp alone on a hub's.
+// left most lanes idle on short columns and one warp alone on a hub's.  Small
+// matrices, whose time is launches, take a form with fewer of them.
 #include <math.h>
 
 #include "awpm.h"
@@ -80,9 +81,8 @@ __device__ __forceinline__ Scale ld_scale(const Scale *p)
 }
 
 // The state the weights' kernels start from.
-__global__ void k_wt_reset(const Work *__restrict__ W)
+__device__ __forceinline__ void wt_reset(const Work &w)
 {
-    const Work &w = *W;
     if (gtid() == 0) {
         w.ctl->err = 0u;
         w.ctl->active = 1;
@@ -93,6 +93,11 @@ __global__ void k_wt_reset(const Work *__restrict__ W)
     const int64_t words = w.starts ? ((int64_t)w.nnz + 31) / 32 + 1 : 0;
     for (int64_t x = gtid(); x < words; x += gstride())
         w.starts[x] = 0u;
+}
+
+__global__ void k_wt_reset(const Work *__restrict__ W)
+{
+    wt_reset(*W);
 }
 
 // Checks (rows in range; values finite and nonzero) and the column maxima: a
@@ -230,16 +235,18 @@ __global__ void __launch_bounds__(kThreads, 6) k_wt_rowmax(const Work *__restric
     }
 }
 
-// The thin form of the column maxima and the row maxima, for where there is no
-// room for the columns' scales and the tiles' columns: a warp per column, its
-// entries read once for the checks and, when all are good, twice for the
+// The thin form of the column maxima and the row maxima, without the columns'
+// scales and the tiles' columns: a warp per column, its entries read once for
+// the checks (and the column pointers') and, when all are good, twice for the
 // maximum and the quotients.
-__global__ void __launch_bounds__(kThreads) k_wt_thin_check(const Work *__restrict__ W)
+__device__ __forceinline__ void wt_thin_check(const Work &w)
 {
-    const Work &w = *W;
-    if (w.ctl->err & kErrInvalid)
-        return;
     unsigned bits = 0;
+    for (int64_t j = gtid(); j <= w.n; j += gstride()) {
+        const int32_t c = w.colptr[j];
+        if ((j == 0 && c != 0) || (j < w.n && w.colptr[j + 1] < c) || (j == w.n && c != w.nnz))
+            bits |= kErrInvalid;
+    }
     for (int64_t p = gtid(); p < w.nnz; p += gstride()) {
         const int32_t r = w.rowidx[p];
         const unsigned long long v = fx_bits(w.wt_a[p]) & kAbs;
@@ -253,9 +260,13 @@ __global__ void __launch_bounds__(kThreads) k_wt_thin_check(const Work *__restri
         raise_err(w.ctl, bits);
 }
 
-__global__ void __launch_bounds__(kThreads) k_wt_thin_rowmax(const Work *__restrict__ W)
+__global__ void __launch_bounds__(kThreads) k_wt_thin_check(const Work *__restrict__ W)
 {
-    const Work &w = *W;
+    wt_thin_check(*W);
+}
+
+__device__ __forceinline__ void wt_thin_rowmax(const Work &w)
+{
     if (!wt_gate(w.ctl))
         return;
     const int lane = threadIdx.x & 31;
@@ -276,17 +287,20 @@ __global__ void __launch_bounds__(kThreads) k_wt_thin_rowmax(const Work *__restr
     }
 }
 
+__global__ void __launch_bounds__(kThreads) k_wt_thin_rowmax(const Work *__restrict__ W)
+{
+    wt_thin_rowmax(*W);
+}
+
 // The weights, from the column-scaled magnitudes and the row maxima.
 template <bool kThin>
-__global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
+__device__ __forceinline__ void wt_out(const Work &w, LogEntry *s_log)
 {
-    __shared__ LogEntry s_log[512];
-    const Work &w = *W;
     if (!wt_gate(w.ctl))
         return;
     const bool logs = w.wt_mode != 0;
     if (logs) {
-        for (int x = threadIdx.x; x < 512; x += kThreads)
+        for (int x = threadIdx.x; x < 512; x += (int)blockDim.x)
             s_log[x] = g_log_table.e[x];
         __syncthreads();
     }
@@ -308,7 +322,7 @@ __global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
             s[u].v = kFxOne;
             s[u].inv = 0;
             if (r[u] >= 0)
-                s[u] = kThin ? make_scale(__ldg(w.wt_max + r[u])) : ld_scale(w.wt_scale + r[u]);
+                s[u] = kThin ? make_scale(w.wt_max[r[u]]) : ld_scale(w.wt_scale + r[u]);
         }
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
@@ -328,15 +342,41 @@ __global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
     }
 }
 
+template <bool kThin>
+__global__ void __launch_bounds__(kThreads) k_wt_out(const Work *__restrict__ W)
+{
+    __shared__ LogEntry s_log[512];
+    wt_out<kThin>(*W, s_log);
+}
+
+// A small matrix: the thin form in one cluster, with cluster barriers between
+// the steps.
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(1024)
+    k_wt_cluster(const Work *__restrict__ W)
+{
+    __shared__ LogEntry s_log[512];
+    const Work &w = *W;
+    wt_reset(w);
+    cluster_sync();
+    wt_thin_check(w);
+    cluster_sync();
+    wt_thin_rowmax(w);
+    cluster_sync();
+    wt_out<true>(w, s_log);
+}
+
 }  // namespace
 
 void launch_weights(const Work *d, const Shape &sh, bool thin, Sink &k)
 {
     void *a[] = {(void *)&d};
     const unsigned grid = (unsigned)(sh.num_sms * 8);
+    if (sh.cluster) {
+        k.launch((const void *)k_wt_cluster, 8, 1024, a);
+        return;
+    }
     k.launch((const void *)k_wt_reset, grid, kThreads, a);
     if (thin) {
-        launch_check_colptr(d, sh, k);
         k.launch((const void *)k_wt_thin_check, 2 * grid, kThreads, a);
         k.launch((const void *)k_wt_thin_rowmax, 2 * grid, kThreads, a);
         k.launch((const void *)k_wt_out<true>, 2 * grid, kThreads, a);

@@ -46,6 +46,9 @@ def reference(n, colptr, rowidx, a, mode):
         return np.log(x) if mode else x
 
 
+# sizes at the ends of the ranges of the three forms (tiles of 32 entries)
+SIZES = [384 * 32 + x for x in (-1, 0, 1, 32)] + [4096 * 32 + x for x in (-31, 0, 1)]
+
 CASES = {
     "empty_columns": [0, 0, 3, 0, 31, 32, 33, 0, 1, 0, 0, 64, 65, 0, 0, 1] + [0, 1, 2] * 40,
     "hub": [200] + [1] * 199,
@@ -78,13 +81,52 @@ def test_edges(ctx, name, span, mode):
             assert np.all(np.abs(got[fine] - want[fine]) <= 2 * np.spacing(np.abs(want[fine])))
 
 
+@pytest.mark.parametrize("nnz", SIZES)
+def test_forms(ctx, nnz):
+    """Either side of the lines between the forms, with a long column, empty
+    ones and a remainder: the quotients bit for bit, in place too."""
+    import torch
+    rng = np.random.default_rng(nnz)
+    n = nnz // 6
+    degrees = rng.integers(0, 10, n)
+    degrees[n // 3] = 1500
+    while degrees.sum() != nnz:
+        j = rng.integers(0, n)
+        if degrees.sum() < nnz:
+            degrees[j] += 1
+        elif degrees[j]:
+            degrees[j] -= min(degrees[j], degrees.sum() - nnz)
+    n, colptr, rowidx, a = matrix(list(degrees), nnz, 300)
+    want = reference(n, colptr, rowidx, a, 0)
+    for in_place in (False, True):
+        cp, ri, av = (torch.from_numpy(x).cuda() for x in (colptr, rowidx, a))
+        out = av if in_place else torch.empty_like(av)
+        awpm.awpm_weights(ctx, n, cp, ri, av, 0, out)
+        assert np.array_equal(out.cpu().numpy(), want, equal_nan=True)
+    # what is refused: a value of zero, a row out of range, a bad column pointer
+    for k in range(3):
+        c2, r2, a2 = colptr.copy(), rowidx.copy(), a.copy()
+        if k == 0:
+            a2[nnz - 1] = 0.0
+        elif k == 1:
+            r2[nnz // 2] = n
+        else:
+            c2[n // 2] = nnz + 1
+        cp, ri, av = (torch.from_numpy(x).cuda() for x in (c2, r2, a2))
+        with pytest.raises(awpm.AwpmError):
+            awpm.awpm_weights(ctx, n, cp, ri, av, 0, torch.empty_like(av))
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 @pytest.mark.parametrize("where", ["device", "in_place", "host"])
 def test_budget_without_room(ctx, mode, where):
     """A budget that holds the row maxima and the staged arrays but neither the
     columns' scales nor the tiles' columns gives the same bits."""
     import torch
-    n, colptr, rowidx, a = matrix(CASES["empty_columns"] * 40 + [3000] + [0, 1, 2, 40] * 100, 5, 300)
+    # (more tiles than the small matrices', which take the thin form anyway)
+    n, colptr, rowidx, a = matrix(CASES["empty_columns"] * 450 + [3000] + [0, 1, 2, 40] * 100, 5,
+                                  300)
+    assert a.size > 4096 * 32
 
     def solve(c, a):
         if where == "host":
