@@ -119,8 +119,8 @@ __device__ __forceinline__ int control_step(Ctl *ctl, bool inc)
             ctl->positive += ctl->cur_positive += ctl->d_positive;
             ctl->d_candidates = ctl->d_found = ctl->d_positive = 0;
         }
-        ctl->last_flips = f;
     }
+    ctl->last_flips = f;
     ctl->iterations += 1;
     ctl->cycles += f;
     if (f == 0) {
