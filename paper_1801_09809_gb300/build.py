@@ -20,6 +20,7 @@ SOURCES = ["awpm_kernels.cu", "awpm_weights.cu", "awpm_mcm.cu", "awpm_greedy.cu"
            "awpm_noalloc.cu"]
 HEADERS = [os.path.join(CSRC, "awpm_internal.h"), os.path.join(CSRC, "awpm_ctx.h"),
            os.path.join(CSRC, "awpm_dev.h"), os.path.join(CSRC, "awpm_fixed.h"),
+           os.path.join(CSRC, "awpm_rules.h"),
            os.path.join(INCLUDE, "awpm.h")]
 
 NVCC = os.environ.get("NVCC", "nvcc")

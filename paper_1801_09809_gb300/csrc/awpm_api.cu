@@ -59,8 +59,6 @@ namespace {
             return rc_;        \
     } while (0)
 
-// Largest nnz: positions up to nnz + 31 (a tile's last lane) stay in int32.
-constexpr int32_t kMaxNnz = 0x7fffffff - 63;
 // Largest nnz served by the hash lookup (slot 2 * position in int32).
 constexpr int32_t kMaxHashNnz = (1 << 30) - 1;
 constexpr int kLookahead = 2;
@@ -1010,8 +1008,7 @@ int enqueue_once(awpm_ctx *c, const Request &r)
             nnz = r.colptr[n];
         }
     }
-    // tile arithmetic is int32: positions up to nnz + 31 must fit
-    if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!r.rowidx || !r.weight)))
+    if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!r.rowidx || !r.weight)))
         return AWPM_ERR_INVALID_ARG;
     if (small && r.count == 0 && n <= kSmallMaxN[0] && nnz <= kSmallOneNnz)
         return ctx_enqueue_small(c, r, nnz, nullptr, l_colptr, l_rowidx, l_w, l_mate, l_out);
@@ -1793,7 +1790,7 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     } else {
         nnz = colptr[n];
     }
-    if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!rowidx || !weight)))
+    if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!rowidx || !weight)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     AWPM_TRY(ensure(c, c->mc, sizeof(int32_t) * n));
@@ -1911,7 +1908,7 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
     } else {
         nnz = colptr[n];
     }
-    if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!rowidx || !weight)))
+    if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!rowidx || !weight)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     const size_t words = (size_t)n / 32 + 1;
@@ -2070,7 +2067,7 @@ static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const i
     } else {
         nnz = colptr[n];
     }
-    if (nnz < 0 || nnz > kMaxNnz || (nnz > 0 && (!rowidx || !values || !weight_out)))
+    if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!rowidx || !values || !weight_out)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
     const bool small = ntiles <= kWtClusterTiles;

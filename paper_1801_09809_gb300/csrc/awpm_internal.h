@@ -6,13 +6,9 @@
 
 #include "awpm.h"
 #include "awpm_fixed.h"
+#include "awpm_rules.h"
 
 namespace awpm {
-
-// Nonzeros handled by one warp per tile of the edge-parallel kernels; tiles
-// start at multiples of kTile, so tile t owns word t of the column-start
-// bitmap.
-constexpr int kTile = 32;
 
 // Error bits raised on the device; the host maps them to the public code
 // (priority INVALID > UNSORTED > NONFINITE > NOTPERF > INTERNAL > TIMEOUT).

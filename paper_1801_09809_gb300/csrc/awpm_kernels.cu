@@ -1642,8 +1642,8 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
 // carry a round's tiles through the stages; the loop body is written out
 // three times with the slots' roles rotated, so no value is copied from one
 // stage's registers to the next.  Tile loads take the tile index clamped to
-// ntiles (always in bounds) and a lane is valid exactly when its position is
-// below nnz; a lane's request goes to its queue slot, or to a discard slot
+// ntiles (always in bounds) and a lane is valid exactly when its position, of
+// the clamped tile (see tile_pos), is below nnz; a lane's request goes to its queue slot, or to a discard slot
 // of its own when it does not pass, so the stores need no branch.  All tile
 // arithmetic is 32-bit (ntiles < 2^26).
 #ifndef AWPM_PIPE_U_WIDE
@@ -1738,7 +1738,7 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
             const int32_t tl = tu < ntiles ? tu : ntiles;  // in bounds
             sj[s][u] = __ldg(tile_col + tl);
             sx[s][u] = (int32_t)__ldg(starts + tl);
-            const int32_t p = tu * kTile + lane;
+            const int32_t p = tl * kTile + lane;
             si[s][u] = p < nnz ? __ldcs(rowidx + p) : 0;
         }
     };
@@ -1747,8 +1747,7 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
             const int32_t tu = kBatch ? stile[s][u] : tr + u * nwarps;
-            const int32_t p = tu * kTile + lane;
-            bool valid = p < nnz;
+            bool valid = tile_pos(tu, ntiles, lane) < nnz;
             const int32_t j = lane_column(sj[s][u], (uint32_t)sx[s][u], lane);
             if (kBatch && valid) {
                 // lanes of finished matrices take no part
@@ -1791,7 +1790,9 @@ __global__ void __launch_bounds__(SearchBlock<kBatch>::kThreads,
             const int x = pass ? ((qhead + qn + __popc(need & lanes_below)) & (kQueue - 1))
                                : kQueue + lane;
             qd.im[x] = make_int2(si[s][u], sx[s][u]);
-            qd.jp[x] = make_int2(sj[s][u], (kBatch ? stile[s][u] : tr + u * nwarps) * kTile + lane);
+            // (past the last tile no lane passes: that position is discarded)
+            const uint32_t tu = (uint32_t)(kBatch ? stile[s][u] : tr + u * nwarps);
+            qd.jp[x] = make_int2(sj[s][u], (int32_t)(tu * kTile + (uint32_t)lane));
             qn += __popc(need);
             if (qn >= 32)
                 flush(32);

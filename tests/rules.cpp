@@ -1,0 +1,23 @@
+// Host harness of csrc/awpm_rules.h: a rule's name and its arguments from the
+// command line, its value to standard output.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+
+#include "awpm_rules.h"
+
+using namespace awpm;
+
+int main(int argc, char **argv)
+{
+    auto arg = [&](int k) { return argc > k ? std::atoll(argv[k]) : 0ll; };
+    const char *what = argc > 1 ? argv[1] : "";
+    if (!std::strcmp(what, "max_entries"))
+        std::printf("%lld\n", (long long)kMaxEntries);
+    else if (!std::strcmp(what, "tile_pos"))
+        std::printf("%lld\n",
+                    (long long)tile_pos((int32_t)arg(2), (int32_t)arg(3), (int)arg(4)));
+    else
+        return 1;
+    return 0;
+}

@@ -1,0 +1,38 @@
+"""The index arithmetic and size rules of the library (csrc/awpm_rules.h),
+compiled for the CPU."""
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1801_09809_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("rules") / "rules")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-I" + CSRC, "-o", exe,
+                           os.path.join(HERE, "rules.cpp")])
+
+    def call(*args):
+        out = subprocess.run([exe, *map(str, args)], stdout=subprocess.PIPE, check=True).stdout
+        return int(out.split()[0])
+    return call
+
+
+def test_tiles_past_the_last_never_wrap(rule):
+    """The search looks ahead by up to three rounds of two tiles per warp: with
+    the most entries accepted those tiles' lanes are still past the end, while
+    t * 32 + lane would be negative in 32 bits, hence "below nnz"."""
+    nnz = rule("max_entries")
+    ntiles = -(-nnz // 32)
+    ahead = 4 * 2 * 160 * 32  # rounds x tiles x SMs x warps, rounded up
+    wrapped = ((ntiles + ahead) * 32 + 2 ** 31) % 2 ** 32 - 2 ** 31
+    assert wrapped < 0
+    for t in (ntiles, ntiles + 1, ntiles + 2, ntiles + ahead):
+        for lane in (0, 31):
+            assert nnz <= rule("tile_pos", t, ntiles, lane) < 2 ** 31
+    for t in (0, 1, ntiles - 1):
+        for lane in (0, 31):
+            assert rule("tile_pos", t, ntiles, lane) == t * 32 + lane
