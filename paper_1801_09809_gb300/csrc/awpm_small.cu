@@ -406,8 +406,9 @@ __device__ void solve_matrix(const Work &w, int32_t b, unsigned char *smem)
     }
     solve_sync<kC>();
     // (the same in every thread)
+    // (the pointers run from 0 to exactly nnz, which a served request states)
     const bool fits = p0 >= 0 && p1 <= nnz && nz >= n && nnz <= w.small_cap &&
-                      (o != 0 || p0 == 0);
+                      (o != 0 || p0 == 0) && (o + n != w.n || p1 == nnz);
     if (fits) {
         bool bad = false;
         for (int32_t j = tid; j <= n; j += kThr) {

@@ -144,3 +144,20 @@ def test_errors_named_in_place(ctx, torch, batch):
         assert e.value.name == name
     ref, _, _ = oracle.get().improve(g)
     assert np.array_equal(call(g)[1 if batch else 0], ref)
+
+
+@pytest.mark.parametrize("off", [-1, 1])
+@pytest.mark.parametrize("n", [300, 3000])
+def test_stated_entries(ctx, torch, n, off):
+    """A served request whose stated number of entries is not colptr[n] is
+    refused, by one too many as by one too few (the arrays are one longer than
+    the matrix), and the same request with the right number is solved."""
+    g = gen.banded(n, 5, 9960)
+    cp, ri, w, m = to_device(g, torch)
+    ri, w = torch.cat([ri, ri[:1]]), torch.cat([w, w[:1]])
+    out = torch.empty_like(m)
+    with pytest.raises(awpm.AwpmError) as e:
+        awpm.awpm_wait(ctx, awpm.awpm_submit(ctx, n, cp, ri, w, m, out, nnz=g.nnz + off))
+    assert e.value.name == "INVALID_ARG"
+    awpm.awpm_wait(ctx, awpm.awpm_submit(ctx, n, cp, ri, w, m, out, nnz=g.nnz))
+    assert np.array_equal(out.cpu().numpy(), oracle.get().improve(g)[0])
