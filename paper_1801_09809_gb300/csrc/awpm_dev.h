@@ -49,7 +49,10 @@ __device__ __forceinline__ bool segment_complete(uint32_t mask, int lane, int32_
 // compare-and-swap means another thread stored a strictly better record, so
 // the loop ends long before this; the bound only turns a broken invariant
 // into an error bit instead of a hang).
-constexpr int kCasRetryCap = 1 << 20;
+#ifndef AWPM_CAS_RETRY_CAP
+#define AWPM_CAS_RETRY_CAP (1 << 20)
+#endif
+constexpr int kCasRetryCap = AWPM_CAS_RETRY_CAP;
 
 __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
 {

@@ -88,7 +88,8 @@ struct alignas(16) Sel {
 // Device-resident control block of one solve.
 struct Ctl {
     unsigned int err;            // kErr* bits
-    int32_t active;              // 1 while the pass loop continues
+    int32_t active;              // 1 while the pass loop continues; maximum matching: the
+                                 // next step is one cluster's
     int32_t iterations;          // passes run
     int32_t converged;           // last pass flipped nothing
     int32_t max_passes;          // cap on passes
@@ -404,8 +405,8 @@ void launch_weights(const Work *d, const Shape &sh, bool thin, Sink &k);
 void launch_mcm_load(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_phase(const Work *d, const Shape &sh, Sink &k);
 void launch_mcm_level(const Work *d, const Shape &sh, Sink &k);
-// Graph form of a level: small levels in a single block, then the steps, the
-// last one also setting the level loop's condition.
+// Graph form of a level: small levels in one cluster, then the steps, the last
+// one also setting the level loop's condition.
 void launch_mcm_level_graph(const Work *d, const Shape &sh, cudaGraphConditionalHandle h,
                             Sink &k);
 // The phases and levels of a small problem in one kernel.

@@ -512,12 +512,20 @@ __device__ __forceinline__ bool mc_count_level(const Work &w)
     return *(volatile unsigned *)&c->err == 0u;
 }
 
+// Whether the next level, if there is one, is k_mc_small's, into Ctl::active:
+// decided by one thread, before the threads that act on it start, so that all
+// of them agree (an error bit may be set while they are reading).
+__device__ __forceinline__ void mc_next_small(const Work &w, bool go)
+{
+    w.ctl->active = go && w.ctl->level_tiles <= kSmallTiles ? 1 : 0;
+}
+
 // Graph form of step 3: the block that finishes last also sets the level
 // loop's condition.
 __global__ void k_mc_advance_graph(const Work *__restrict__ W, cudaGraphConditionalHandle h)
 {
     const Work &w = *W;
-    // (after the single-block levels ended the phase there is nothing left)
+    // (after k_mc_small's levels ended the phase there is nothing left)
     const bool run = w.ctl->front_n > 0;
     if (run && !w.ctl->err)
         mc_advance(w);
@@ -527,6 +535,7 @@ __global__ void k_mc_advance_graph(const Work *__restrict__ W, cudaGraphConditio
             mc_frontier_made(w.ctl);
             go = mc_count_level(w);
         }
+        mc_next_small(w, go);
         cudaGraphSetConditional(h, go ? 1u : 0u);
     }
 }
@@ -538,18 +547,9 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
     k_mc_small(const Work *__restrict__ W)
 {
     __shared__ int32_t s_buf[kSmallThreads / 32][kRowBuf];
-    __shared__ int s_go;
     const Work &w = *W;
     Ctl *c = w.ctl;
-    for (;;) {
-        if (threadIdx.x == 0)
-            s_go = *(volatile unsigned *)&c->err == 0u && *(volatile int32_t *)&c->front_n > 0 &&
-                   *(volatile int32_t *)&c->level_tiles <= kSmallTiles;
-        __syncthreads();
-        // the same for all blocks: these counters were last written before a
-        // cluster barrier (the error bits by raise_err before it, too)
-        if (!s_go)
-            return;
+    while (*(volatile int32_t *)&c->active) {
         mc_offer(w, s_buf[threadIdx.x >> 5]);
         cluster_sync();
         mc_join(w);
@@ -558,7 +558,7 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
         cluster_sync();
         if (gtid() == 0) {
             mc_frontier_made(c);
-            mc_count_level(w);
+            mc_next_small(w, mc_count_level(w));
         }
         cluster_sync();
     }
@@ -567,7 +567,9 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
 // Graph form of the level loop's condition before a phase's first level.
 __global__ void k_mc_cond_level(const Work *__restrict__ W, cudaGraphConditionalHandle h)
 {
-    cudaGraphSetConditional(h, mc_count_level(*W) ? 1u : 0u);
+    const bool go = mc_count_level(*W);
+    mc_next_small(*W, go);
+    cudaGraphSetConditional(h, go ? 1u : 0u);
 }
 
 // The end of a phase: count it and the paths it augmented; continue while it
@@ -632,13 +634,15 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
     for (;;) {
         mc_phase(w);
         cluster_sync();
+        // (one thread decides whether a level runs, between two barriers:
+        // threads that read the error bits for themselves could disagree, and
+        // wait at different barriers)
         if (gtid() == 0) {
             mc_frontier_made(c);
-            mc_count_level(w);
+            c->active = mc_count_level(w) ? 1 : 0;
         }
         cluster_sync();
-        // (the counters and the error bits are last written before a barrier)
-        while (*(volatile int32_t *)&c->front_n > 0 && *(volatile unsigned *)&c->err == 0u) {
+        while (*(volatile int32_t *)&c->active) {
             mc_offer(w, s_buf[threadIdx.x >> 5]);
             cluster_sync();
             mc_join(w);
@@ -647,7 +651,7 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
             cluster_sync();
             if (gtid() == 0) {
                 mc_frontier_made(c);
-                mc_count_level(w);
+                c->active = mc_count_level(w) ? 1 : 0;
             }
             cluster_sync();
         }

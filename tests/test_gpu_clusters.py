@@ -1,6 +1,12 @@
 """Greedy and maximum matching around the sizes where their loops move from one
 cluster to the graph (needs a GPU), empty columns and unmatched columns
-included: equal to the oracle on both sides of the line."""
+included: equal to the oracle on both sides of the line; and the end of a
+maximum matching whose bounded retries give up."""
+import os
+import subprocess
+import sys
+import textwrap
+
 import numpy as np
 import pytest
 
@@ -81,3 +87,41 @@ def test_mcm(ctx, nnz, empty):
     st = awpm.awpm_mcm(ctx, g.n, g.colptr, g.rowidx, g.weight, got)
     assert np.array_equal(got, ref)
     assert st["cardinality"] == int((ref >= 0).sum())
+
+
+NO_RETRIES = textwrap.dedent("""
+    import sys
+    sys.path[:0] = [{root!r}, {tests!r}]
+    import numpy as np
+    import pytest
+    from paper_1801_09809_gb300 import awpm
+    from test_gpu_clusters import MCM, sized
+    assert awpm.LIB_PATH == {lib!r}
+    ctx = awpm.awpm_create(device=0)
+    for nnz in (2000, MCM, MCM + 32, 2 * MCM):
+        g = sized(nnz, 9990, True)
+        with pytest.raises(awpm.AwpmError) as e:
+            awpm.awpm_mcm(ctx, g.n, g.colptr, g.rowidx, g.weight, np.full(g.n, -1, np.int32))
+        assert e.value.name == "TIMEOUT", e.value.name
+    awpm.awpm_destroy(ctx)
+    print("NO_RETRIES_OK")
+""")
+
+
+def test_mcm_retries_given_up(ctx, tmp_path):
+    """With no retries allowed (AWPM_CAS_RETRY_CAP = 0 in this file's kernels) a
+    level's first offers raise the timeout bit while other blocks are still on
+    their way into the level: the cluster and the graph form both end with
+    AWPM_ERR_TIMEOUT."""
+    from paper_1801_09809_gb300 import build
+    obj, lib = str(tmp_path / "awpm_mcm.o"), str(tmp_path / "libawpm_retry.so")
+    subprocess.check_call([build.NVCC, *build.ARCH, *build.FLAGS, "-DAWPM_CAS_RETRY_CAP=0", "-c",
+                           os.path.join(build.CSRC, "awpm_mcm.cu"), "-o", obj])
+    objs = [os.path.join(build.OBJDIR, os.path.splitext(s)[0] + ".o") for s in build.SOURCES]
+    subprocess.check_call([build.NVCC, "-shared", *build.ARCH, "-o", lib, obj,
+                           *(o for o in objs if not o.endswith("awpm_mcm.o"))])
+    tests = os.path.dirname(os.path.abspath(__file__))
+    child = NO_RETRIES.format(root=build.ROOT, tests=tests, lib=lib)
+    r = subprocess.run([sys.executable, "-c", child], env=dict(os.environ, AWPM_LIBRARY=lib),
+                       capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0 and "NO_RETRIES_OK" in r.stdout, r.stdout + r.stderr
