@@ -720,6 +720,10 @@ __global__ void k_small_reset(const Work *__restrict__ W)
     small_reset(*W);
 }
 
+// Nothing: what a stream does before a class's kernel to let the kernels of the
+// larger classes, submitted before, take their places first.
+__global__ void k_small_later() {}
+
 // The matrices of one class, largest first, from a queue.
 template <int kClass>
 __global__ void __launch_bounds__(Cls<kClass>::kThreads, Cls<kClass>::kBlocks)
@@ -809,29 +813,36 @@ void launch_small_batch(const Work *d, const Shape &sh, const int32_t *counts,
                                     (const void *)k_small<2>};
     const unsigned threads[kSmallClasses] = {Cls<0>::kThreads, Cls<1>::kThreads, Cls<2>::kThreads};
     const unsigned blocks[kSmallClasses] = {Cls<0>::kBlocks, Cls<1>::kBlocks, Cls<2>::kBlocks};
-    // the classes side by side: as the blocks of one run out of matrices, the
-    // next one's take their SMs
+    // The classes side by side, the largest first: as the blocks of one run out of
+    // matrices, the next one's take their SMs.  A class that starts before a
+    // larger one keeps the SMs until its queue is empty, which made some calls
+    // longer (4,096 matrices of 200 to 20,000 columns 13.3 ms instead of 12.2), so
+    // each class lets those before it go first.
     auto note = [&k](cudaError_t e) {
         if (k.err == cudaSuccess)
             k.err = e;
     };
     note(cudaEventRecord(ss.fork, k.stream));
+    int before = 0;  // classes launched
     for (int c = 0; c < kSmallClasses; ++c) {
         const unsigned most = sms * blocks[c];
         if (counts[c] <= 0)
             continue;
         Sink s;
-        s.stream = c == 0 ? k.stream : ss.side[c - 1];
-        if (c > 0)
+        s.stream = before == 0 ? k.stream : ss.side[before - 1];
+        if (before > 0)
             note(cudaStreamWaitEvent(s.stream, ss.fork, 0));
+        for (int x = 0; x < before; ++x)
+            s.launch((const void *)k_small_later, 1, 32, nullptr);
         s.launch(f[c], (unsigned)counts[c] < most ? (unsigned)counts[c] : most, threads[c], a,
                  (unsigned)small_class_smem(c));
         note(s.err);
-        if (c > 0) {
-            note(cudaEventRecord(ss.join[c - 1], s.stream));
-            note(cudaStreamWaitEvent(k.stream, ss.join[c - 1], 0));
-        }
+        if (before > 0)
+            note(cudaEventRecord(ss.join[before - 1], s.stream));
+        ++before;
     }
+    for (int x = 0; x + 1 < before; ++x)
+        note(cudaStreamWaitEvent(k.stream, ss.join[x], 0));
     k.launch((const void *)k_small_total, 1, 1024, a);
 }
 
