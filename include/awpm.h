@@ -216,9 +216,11 @@ int awpm_improve_ctx(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int3
  * matrix; a matrix stops at its first empty pass (or after max_iters
  * passes) and its tiles are skipped from then on.  Each matrix's matching,
  * pass count, cycle count and weights equal those of awpm_improve on that
- * matrix alone.  Matrices of up to 20,096 columns are solved by a thread block
- * each (three kernels, one per size class, side by side); a batch with a larger
- * one, or an invalid one, runs as a union in one CUDA-graph launch.
+ * matrix alone.  A batch whose matrices have up to 20,096 columns each, and
+ * entries enough in all that the largest one is not what the call would wait
+ * for, is solved by a thread block per matrix (three kernels, one per size class,
+ * side by side); any other (few matrices, one much larger than the rest, an
+ * invalid one) runs as a union in one CUDA-graph launch.
  *   per_matrix[count] (may be NULL): iterations, converged, cycles_applied,
  *     edge_checks, weight_in, weight_out of each matrix (candidate counters
  *     are 0 there); total (may be NULL): the union (candidates, closing_found,

@@ -184,16 +184,14 @@ constexpr int32_t kSmallOneNnz = 40960;
 // of about 10 us): above, an average column of 20 entries is too many.
 constexpr int32_t kSmallOneN = 2048;
 
-// Whether small matrices are solved by a block each (default on; the
-// environment variable AWPM_SMALL=0 switches it off, a tuning knob: results
-// are the same either way).
-bool small_enabled()
+// Whether small matrices are solved by a block (or a cluster) each: where the
+// rules say so (1), never (0), or every batch whose matrices fit (2).  The
+// environment variable AWPM_SMALL=0 or 1, read when a context is made, selects
+// the latter two (a tuning knob: results are the same either way).
+int small_mode()
 {
-    static const bool on = [] {
-        const char *v = getenv("AWPM_SMALL");
-        return !(v && v[0] == '0' && v[1] == 0);
-    }();
-    return on;
+    const char *v = getenv("AWPM_SMALL");
+    return v && v[0] == '0' && v[1] == 0 ? 0 : v && v[0] == '1' && v[1] == 0 ? 2 : 1;
 }
 
 int code_of(unsigned err)
@@ -740,6 +738,7 @@ int setup_ctx(awpm_ctx *c, const awpm_options *opt)
     CUDA_TRY(search_inc_setup());
     CUDA_TRY(small_setup());
     c->search_wide = default_search_wide();
+    c->small_mode = small_mode();
     for (int b = 0; b < 2; ++b)
         for (int p = 0; p < 2; ++p) {
             c->search_bps[b][0][p] = search_blocks_per_sm(AWPM_LOOKUP_BSEARCH, b == 1, p == 1);
@@ -836,20 +835,27 @@ void teardown_ctx(awpm_ctx *c)
     cudaGetLastError();
 }
 
+// Room in pinned memory for a batch's per-matrix results (miter, mconv, mnnz
+// (i32), mcycles (u64), mw_in, mw_out (f64)).
+int ensure_pinned(awpm_ctx *c, int32_t count)
+{
+    const size_t bytes = (size_t)count * (3 * sizeof(int32_t) + 3 * 8);
+    if (c->h_batch_bytes >= bytes)
+        return AWPM_OK;
+    if (c->h_batch)
+        cudaFreeHost(c->h_batch);
+    c->h_batch = nullptr;
+    c->h_batch_bytes = 0;
+    CUDA_TRY(cudaMallocHost(&c->h_batch, bytes));
+    c->h_batch_bytes = bytes;
+    return AWPM_OK;
+}
+
 // Copy a batch's per-matrix results to pinned memory.
 int copy_batch_results(awpm_ctx *c, const BatchWork &bw)
 {
     const int32_t count = bw.count;
-    // per-matrix results: miter, mconv, mnnz (i32), mcycles (u64), mw_in, mw_out (f64)
-    const size_t pm_bytes = (size_t)count * (3 * sizeof(int32_t) + 3 * 8);
-    if (c->h_batch_bytes < pm_bytes) {
-        if (c->h_batch)
-            cudaFreeHost(c->h_batch);
-        c->h_batch = nullptr;
-        c->h_batch_bytes = 0;
-        CUDA_TRY(cudaMallocHost(&c->h_batch, pm_bytes));
-        c->h_batch_bytes = pm_bytes;
-    }
+    AWPM_TRY(ensure_pinned(c, count));
     char *hb = (char *)c->h_batch;
     CUDA_TRY(cudaMemcpyAsync(hb, bw.miter, sizeof(int32_t) * 3 * (size_t)count,
                              cudaMemcpyDeviceToHost, c->stream));
@@ -857,13 +863,18 @@ int copy_batch_results(awpm_ctx *c, const BatchWork &bw)
                              cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaMemcpyAsync(hb + 20 * (size_t)count, bw.mw_in, 16 * (size_t)count,
                              cudaMemcpyDeviceToHost, c->stream));
-        return AWPM_OK;
+    return AWPM_OK;
+}
+
+size_t batch_i32_bytes(int32_t count)
+{
+    return sizeof(int32_t) * (5 * (size_t)count + 2 + kSmallClasses);
 }
 
 // Device arrays of a batch's results (or a single small solve's).
 int batch_arrays(awpm_ctx *c, BatchWork &bw, int32_t count)
 {
-    AWPM_TRY(ensure(c, c->b_i32, sizeof(int32_t) * (5 * (size_t)count + 2 + kSmallClasses)));
+    AWPM_TRY(ensure(c, c->b_i32, batch_i32_bytes(count)));
     AWPM_TRY(ensure(c, c->b_u64, sizeof(unsigned long long) * 2 * (size_t)count));
     AWPM_TRY(ensure(c, c->b_f64, sizeof(double) * 2 * (size_t)count));
     bw.count = count;
@@ -881,13 +892,6 @@ int batch_arrays(awpm_ctx *c, BatchWork &bw, int32_t count)
     bw.mw_in = f64;
     bw.mw_out = f64 + count;
     return AWPM_OK;
-}
-
-// Class of a matrix of n columns for the small-matrix kernel (n at most
-// kSmallMaxN[0]).
-int small_class(int32_t n)
-{
-    return n <= kSmallMaxN[2] ? 2 : n <= kSmallMaxN[1] ? 1 : 0;
 }
 
 // The matrices of a batch by class and, within a class, roughly from the
@@ -926,6 +930,44 @@ bool small_batch_order(const int32_t *off, int32_t count, int32_t n, std::vector
     for (int32_t b : by)
         order[(size_t)next[small_class(off[b + 1] - off[b])]++] = b;
     return true;
+}
+
+// The entries of a batch of small matrices (valid offsets): their number into
+// *nnz, the tiles of each matrix (its own, rounded up) into *load.  Column
+// pointers on the device are read by a kernel that writes them to pinned memory
+// (a round trip as for nnz alone; copied back, they made it 5 us longer).
+int read_batch(awpm_ctx *c, const Request &r, int l_colptr, int l_off, int32_t *nnz,
+               BatchLoad *load)
+{
+    const size_t count = (size_t)r.count;
+    const int32_t *off = r.off_host, *at = nullptr;
+    std::vector<int32_t> own;
+    if (l_colptr == 1) {
+        AWPM_TRY(ensure_pinned(c, r.count));
+        int32_t *h = (int32_t *)c->h_batch;  // the pointers, then the offsets
+        const int32_t *koff = r.n_off;
+        if (l_off != 1) {
+            std::memcpy(h + count + 1, off, sizeof(int32_t) * (count + 1));
+            koff = h + count + 1;
+        }
+        Sink k;
+        k.stream = c->stream;
+        launch_small_entries(koff, r.colptr, r.n, r.count, h, k);
+        AWPM_TRY(check_sink(k));
+        CUDA_TRY(cudaStreamSynchronize(c->stream));
+        at = h;
+    } else {
+        own.resize(count + 1);
+        for (size_t b = 0; b <= count; ++b)
+            own[b] = r.colptr[off[b]];
+        at = own.data();
+    }
+    *nnz = at[count];
+    for (size_t b = 0; b < count; ++b) {
+        const int64_t nz = (int64_t)at[b + 1] - at[b];
+        load->add(off[b + 1] - off[b], nz > 0 ? (nz + kTile - 1) / kTile : 0);
+    }
+    return AWPM_OK;
 }
 
 int ctx_enqueue_small(awpm_ctx *c, const Request &r, int32_t nnz, const int32_t *per_class,
@@ -984,7 +1026,7 @@ int enqueue_once(awpm_ctx *c, const Request &r)
 
     // Small matrices: a block each, in one kernel.  A single one does not even
     // have its nnz read back first.
-    const bool small = small_enabled() && !c->general_only && !c->least_memory && !r.search_only &&
+    const bool small = c->small_mode && !c->general_only && !c->least_memory && !r.search_only &&
                        !(c->opt.flags & AWPM_FLAG_TIME_SEARCH) &&
                        c->opt.select == AWPM_SELECT_STEP_D &&
                        (c->opt.lookup == AWPM_LOOKUP_AUTO || c->opt.lookup == AWPM_LOOKUP_BSEARCH) &&
@@ -998,7 +1040,16 @@ int enqueue_once(awpm_ctx *c, const Request &r)
     }
 
     int32_t nnz = r.nnz;
-    if (nnz < 0) {
+    int32_t per_class[kSmallClasses];
+    const bool small_batch = small && r.count > 0 && r.off_host &&
+                             small_batch_order(r.off_host, r.count, n, pd.order, per_class);
+    bool blocks = false;
+    if (small_batch) {
+        BatchLoad load;
+        AWPM_TRY(read_batch(c, r, l_colptr, l_off, &nnz, &load));
+        blocks = c->small_mode == 2 || load.blocks_pay();
+    }
+    if (nnz < 0 && !small_batch) {
         if (l_colptr == 1) {
             CUDA_TRY(cudaMemcpyAsync(c->h_ctl, r.colptr + n, sizeof(int32_t),
                                      cudaMemcpyDeviceToHost, c->stream));
@@ -1012,9 +1063,7 @@ int enqueue_once(awpm_ctx *c, const Request &r)
         return AWPM_ERR_INVALID_ARG;
     if (small && r.count == 0 && n <= kSmallMaxN[0] && nnz <= kSmallOneNnz)
         return ctx_enqueue_small(c, r, nnz, nullptr, l_colptr, l_rowidx, l_w, l_mate, l_out);
-    int32_t per_class[kSmallClasses];
-    if (small && r.count > 0 && r.off_host &&
-        small_batch_order(r.off_host, r.count, n, pd.order, per_class))
+    if (blocks)
         return ctx_enqueue_small(c, r, nnz, per_class, l_colptr, l_rowidx, l_w, l_mate, l_out);
     const bool timed = (c->opt.flags & AWPM_FLAG_TIME_SEARCH) != 0;
     // launch configuration: given, or the autotuner's (AWPM_LOOKUP_AUTO)

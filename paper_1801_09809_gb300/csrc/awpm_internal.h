@@ -156,12 +156,10 @@ constexpr int kMapSmallBits = 1 << 17;
 constexpr int kMapLargeBits = 1 << 20;
 constexpr unsigned kSmallFlips = 1024;
 
-// Solves of small matrices by one block each: classes of sizes (the largest
-// first), the largest n of each, and the shared memory that a matrix needs
-// with `warps` warps, with or without the columns' signatures (the rings; the
-// column pointers; four bitmaps; signatures; three 16-bit arrays).
-constexpr int kSmallClasses = 3;
-constexpr int32_t kSmallMaxN[kSmallClasses] = {20096, 7168, 2048};
+// Solves of small matrices by one block each (classes: kSmallMaxN): the shared
+// memory that a matrix needs with `warps` warps, with or without the columns'
+// signatures (the rings; the column pointers; four bitmaps; signatures; three
+// 16-bit arrays).
 constexpr int kSmallOne = kSmallClasses;  // the single matrix's class
 constexpr int kSmallWarps[kSmallClasses + 1] = {32, 16, 8, 16};
 __host__ __device__ constexpr size_t small_smem(int32_t n, int warps, bool sigs)
@@ -367,6 +365,9 @@ struct SmallStreams {
 void launch_small_batch(const Work *d, const Shape &sh, const int32_t *counts,
                         const SmallStreams &ss, Sink &k);
 void launch_small_one(const Work *d, int32_t smem, Sink &k);
+// The column pointers at count + 1 offsets in [0, n], into at[].
+void launch_small_entries(const int32_t *off, const int32_t *colptr, int32_t n, int32_t count,
+                          int32_t *at, Sink &k);
 
 // Launch sequences; `d` is the device copy of the Work.
 void launch_init(const Work *d, const Shape &sh, Sink &k);

@@ -25,4 +25,55 @@ AWPM_HD int32_t tile_pos(int32_t t, int32_t ntiles, int lane)
     return (t < ntiles ? t : ntiles) * kTile + lane;
 }
 
+// Solves of small matrices by one block each: classes of sizes (the largest
+// first) and the largest n of each.
+constexpr int kSmallClasses = 3;
+constexpr int32_t kSmallMaxN[kSmallClasses] = {20096, 7168, 2048};
+
+// Class of a matrix of n columns, n at most kSmallMaxN[0].
+inline int small_class(int32_t n)
+{
+    return n <= kSmallMaxN[2] ? 2 : n <= kSmallMaxN[1] ? 1 : 0;
+}
+
+// Whether a batch of small matrices is solved by a block per matrix, rather than
+// as a union over the whole GPU.  A block has one SM at most, so the call lasts
+// as long as its slowest matrix there, however idle the other SMs are; the union
+// spreads all tiles over the GPU, but launches its kernels again for every pass.
+// Both go with the number of passes, which nobody knows beforehand, so the
+// rule compares what a pass costs, in ns:
+//   a matrix in its block: 14,000 + 100, 58 or 34 per tile by class (256, 512 or
+//     1,024 threads);
+//   the union: 44,000 + 0.42 per tile still searched.  With matrices alike all
+//     are to the last pass; with mixed sizes most converge before the largest.
+//     Where the average has a small share of the largest's tiles, 0.4 of them
+//     count.
+// ms per call, union / blocks: banded, 2,000 columns (562 tiles each), 4
+// matrices 0.61 / 0.91, 64 0.86 / 1.00, 256 1.86 / 1.31; banded, 20,000 (5,624),
+// 16 matrices 1.15 / 2.90, 64 3.08 / 3.52; banded, 16,371 (3,581), 96 2.69 /
+// 2.05; 5-point, 2,000 (311), 1 matrix 0.341 / 0.347; 27-point, 1,728 (1,228), 64
+// 1.74 / 3.33, 256 4.82 / 4.33; random, 300 (83), 4 matrices 0.250 / 0.127, 2,000
+// (562), 64 0.322 / 0.285 (the rule's loss: few passes); random with 100 entries
+// a column, 10,000 (31,400), 4 matrices 1.26 / 11.4; sizes from 200 to 20,000, 32
+// matrices 0.83 / 3.07, 512 3.58 / 6.89, 1,024 6.45 / 7.77, 2,048 12.1 / 9.43.
+struct BatchLoad {
+    int64_t count = 0, all = 0, largest = 0;  // matrices, their tiles, the most of one
+    double block_ns = 0;                      // the slowest matrix's pass in its block
+    void add(int32_t n, int64_t tiles)
+    {
+        constexpr double kTileNs[kSmallClasses] = {34, 58, 100};
+        const double ns = 14000 + kTileNs[small_class(n)] * (double)tiles;
+        ++count;
+        all += tiles;
+        largest = largest > tiles ? largest : tiles;
+        block_ns = block_ns > ns ? block_ns : ns;
+    }
+    double union_ns() const
+    {
+        const double share = largest > 0 ? (double)all / ((double)count * (double)largest) : 1.0;
+        return 44000 + 0.42 * (0.4 + 0.6 * share) * (double)all;
+    }
+    bool blocks_pay() const { return block_ns <= union_ns(); }
+};
+
 }  // namespace awpm

@@ -18,6 +18,8 @@
 // solve at 44 % issue utilisation) and the lookups' latency.  Measured: 4,096
 // matrices of 200 to 20,000 columns, 21.2 ms over the union, now 12.0 ms; a
 // single random matrix of 2,000 columns and 16,000 entries 128 us, now 67 us.
+// With few matrices most SMs are idle and the call lasts as long as its largest
+// one: BatchLoad (awpm_rules.h) says which batches come here.
 //
 // The kernel only reports that something is wrong with an input (kErrRetry);
 // the caller then solves the batch by the general path, which names the error.
@@ -783,6 +785,14 @@ __global__ void k_small_total(const Work *__restrict__ W)
     }
 }
 
+__global__ void k_small_entries(const int32_t *__restrict__ off, const int32_t *__restrict__ colptr,
+                                int32_t n, int32_t count, int32_t *__restrict__ at)
+{
+    // (the host has checked its copy of the offsets)
+    for (int64_t b = gtid(); b <= count; b += gstride())
+        at[b] = __ldg(colptr + min(max(__ldg(off + b), 0), n));
+}
+
 cudaError_t allow(const void *f, int c)
 {
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -844,6 +854,14 @@ void launch_small_batch(const Work *d, const Shape &sh, const int32_t *counts,
     for (int x = 0; x + 1 < before; ++x)
         note(cudaStreamWaitEvent(k.stream, ss.join[x], 0));
     k.launch((const void *)k_small_total, 1, 1024, a);
+}
+
+void launch_small_entries(const int32_t *off, const int32_t *colptr, int32_t n, int32_t count,
+                          int32_t *at, Sink &k)
+{
+    void *a[] = {(void *)&off, (void *)&colptr, (void *)&n, (void *)&count, (void *)&at};
+    const int64_t blocks = ((int64_t)count + kThreads) / kThreads;
+    k.launch((const void *)k_small_entries, (unsigned)(blocks < 1024 ? blocks : 1024), kThreads, a);
 }
 
 void launch_small_one(const Work *d, int32_t smem, Sink &k)

@@ -17,7 +17,12 @@ int main(int argc, char **argv)
     else if (!std::strcmp(what, "tile_pos"))
         std::printf("%lld\n",
                     (long long)tile_pos((int32_t)arg(2), (int32_t)arg(3), (int)arg(4)));
-    else
+    else if (!std::strcmp(what, "blocks_pay")) {  // n and tiles of each matrix
+        BatchLoad load;
+        for (int k = 2; k + 1 < argc; k += 2)
+            load.add((int32_t)arg(k), arg(k + 1));
+        std::printf("%d\n", load.blocks_pay() ? 1 : 0);
+    } else
         return 1;
     return 0;
 }

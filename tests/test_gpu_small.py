@@ -1,9 +1,9 @@
 """Solves of small matrices by a block (batches) or a cluster (single ones)
-each (needs a GPU): the edges of the size classes against the oracle, inputs
-that go back to the general path, and the existing parity, batch and record
-tests with the small-matrix kernel switched off (in a child process, since
-the library reads AWPM_SMALL once), so that the general path keeps its
-coverage at small sizes."""
+each (needs a GPU): the edges of the size classes against the oracle, both
+sides of the line up to which a batch takes a block per matrix, inputs that go
+back to the general path, and the existing parity, batch and record tests with
+the small-matrix kernel switched off (in a child process), so that the general
+path keeps its coverage at small sizes."""
 import os
 import subprocess
 import sys
@@ -29,6 +29,13 @@ def torch():
     return _t
 
 
+@pytest.fixture(autouse=True)
+def blocks(monkeypatch):
+    """Batches go to the small-matrix kernel whenever their matrices fit it,
+    whether that pays or not (read when a context is made)."""
+    monkeypatch.setenv("AWPM_SMALL", "1")
+
+
 @pytest.fixture
 def ctx(torch):
     c = awpm.awpm_create(device=0)
@@ -45,14 +52,22 @@ def test_switched_off(torch, which):
     assert r.returncode == 0, r.stdout[-3000:] + r.stderr[-1000:]
 
 
-def batch_check(ctx, torch, graphs, max_iters=0):
+def batch_check(ctx, torch, graphs, max_iters=0, host=False, times=2):
+    """Solves a batch several times (each starts from the records that the one
+    before left); returns the lookups used."""
     n_off, u = gen.union(graphs)
-    cp, ri, w, m = to_device(u, torch)
-    off = torch.from_numpy(n_off).cuda()
-    out = torch.empty_like(m)
-    for _ in range(2):  # the second batch starts from the first one's records
+    if host:
+        (cp, ri, w, m), off = (u.colptr, u.rowidx, u.weight, u.mate), n_off
+        out = np.empty_like(m)
+    else:
+        cp, ri, w, m = to_device(u, torch)
+        off = torch.from_numpy(n_off).cuda()
+        out = torch.empty_like(m)
+    used = []
+    for _ in range(times):
         tot, per = awpm.awpm_improve_batch(ctx, len(graphs), off, cp, ri, w, m, out)
-        got = gen.split(n_off, out.cpu().numpy())
+        used.append(tot["lookup_used"])
+        got = gen.split(n_off, out if host else out.cpu().numpy())
         sums = dict.fromkeys(("candidates", "closing_found", "positive", "cycles_applied"), 0)
         for b, g in enumerate(graphs):
             ref, rst, _ = oracle.get().improve(g, max_iters=max_iters)
@@ -62,6 +77,34 @@ def batch_check(ctx, torch, graphs, max_iters=0):
             for k in sums:
                 sums[k] += rst[k]
         assert {k: tot[k] for k in sums} == sums
+    return used
+
+
+def line_batches():
+    """A batch on either side of the line (14,000 + 100 or 58 per tile of the
+    slowest matrix against the union's 44,000 + 0.42 per tile): four alike, and
+    one larger among many small ones."""
+    small = [gen.banded(300, 9, 9970 + k) for k in range(100)]
+    return [([gen.banded(1950, 5, 9971 + k) for k in range(4)], True),
+            ([gen.banded(1965, 5, 9972 + k) for k in range(4)], False),
+            (small + [gen.banded(3300, 5, 9973)], True),
+            (small + [gen.banded(3800, 5, 9974)], False)]
+
+
+@pytest.mark.parametrize("host", [False, True])
+@pytest.mark.parametrize("which", range(4))
+def test_lines(torch, monkeypatch, which, host):
+    """Both sides of the line equal the oracle and go where they should: the
+    third solve that a new context does as a union tries the hash lookup, the
+    small-matrix kernel has none."""
+    monkeypatch.delenv("AWPM_SMALL")
+    graphs, blocks = line_batches()[which]
+    c = awpm.awpm_create(device=0)
+    try:
+        used = batch_check(c, torch, graphs, host=host, times=3)
+        assert used[2] == (awpm.LOOKUP_BSEARCH if blocks else awpm.LOOKUP_HASH)
+    finally:
+        awpm.awpm_destroy(c)
 
 
 def test_class_edges(ctx, torch):

@@ -36,3 +36,21 @@ def test_tiles_past_the_last_never_wrap(rule):
     for t in (0, 1, ntiles - 1):
         for lane in (0, 31):
             assert rule("tile_pos", t, ntiles, lane) == t * 32 + lane
+
+
+def test_batches_by_work(rule):
+    """A block per matrix where the largest matrix is no more than its share of
+    the work: not for few large matrices, nor dense ones, whatever their n."""
+    def blocks(*matrices):
+        return rule("blocks_pay", *(x for n, tiles, count in matrices for x in (n, tiles) * count))
+    assert blocks((300, 84, 1)) and blocks((300, 84, 4)) and blocks((300, 84, 1024))
+    assert not blocks((2000, 562, 1)) and not blocks((2000, 562, 16)) and blocks((2000, 562, 256))
+    assert not blocks((20000, 5624, 1)) and not blocks((20000, 5624, 64))
+    assert blocks((20000, 5624, 256))
+    assert not blocks((1000, 15750, 4)) and not blocks((10000, 152700, 4))
+    assert not blocks((600, 167, 512), (20000, 10620, 1))
+    # the line for four matrices of the smallest class
+    assert blocks((1950, 305, 4)) and not blocks((1960, 306, 4))
+    # empty matrices, and one class's largest n beside the next
+    assert blocks((0, 0, 3)) and blocks((0, 0, 100), (20, 3, 1))
+    assert not blocks((2048, 400, 4)) and blocks((2049, 400, 4)) and blocks((7169, 800, 4))
