@@ -512,6 +512,29 @@ __device__ __forceinline__ bool mc_count_level(const Work &w)
     return *(volatile unsigned *)&c->err == 0u;
 }
 
+// The two together, with their reads side by side: in a level of one cluster
+// everyone waits for them (2 % of a small problem's search).
+__device__ __forceinline__ bool mc_level_made(const Work &w)
+{
+    Ctl *c = w.ctl;
+    const int32_t next = c->front_next, done = c->phase_levels;
+    const unsigned long long levels = c->levels;
+    const unsigned err = *(volatile unsigned *)&c->err;
+    c->front_n = next;
+    c->live = next;
+    c->front_next = 0;
+    c->touched = 0;
+    if (next <= 0)
+        return false;
+    c->levels = levels + 1;
+    c->phase_levels = done + 1;
+    if (done >= w.n + 1) {
+        raise_err(c, kErrTimeout);
+        return false;
+    }
+    return err == 0u;
+}
+
 // Whether the next level, if there is one, is k_mc_small's, into Ctl::active:
 // decided by one thread, before the threads that act on it start, so that all
 // of them agree (an error bit may be set while they are reading).
@@ -530,11 +553,7 @@ __global__ void k_mc_advance_graph(const Work *__restrict__ W, cudaGraphConditio
     if (run && !w.ctl->err)
         mc_advance(w);
     if (mc_last_block(w.ctl)) {
-        bool go = false;
-        if (run) {
-            mc_frontier_made(w.ctl);
-            go = mc_count_level(w);
-        }
+        const bool go = run && mc_level_made(w);
         mc_next_small(w, go);
         cudaGraphSetConditional(h, go ? 1u : 0u);
     }
@@ -556,10 +575,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
         cluster_sync();
         mc_advance(w);
         cluster_sync();
-        if (gtid() == 0) {
-            mc_frontier_made(c);
-            mc_next_small(w, mc_count_level(w));
-        }
+        if (gtid() == 0)
+            mc_next_small(w, mc_level_made(w));
         cluster_sync();
     }
 }
@@ -637,10 +654,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
         // (one thread decides whether a level runs, between two barriers:
         // threads that read the error bits for themselves could disagree, and
         // wait at different barriers)
-        if (gtid() == 0) {
-            mc_frontier_made(c);
-            c->active = mc_count_level(w) ? 1 : 0;
-        }
+        if (gtid() == 0)
+            c->active = mc_level_made(w) ? 1 : 0;
         cluster_sync();
         while (*(volatile int32_t *)&c->active) {
             mc_offer(w, s_buf[threadIdx.x >> 5]);
@@ -649,10 +664,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
             cluster_sync();
             mc_advance(w);
             cluster_sync();
-            if (gtid() == 0) {
-                mc_frontier_made(c);
-                c->active = mc_count_level(w) ? 1 : 0;
-            }
+            if (gtid() == 0)
+                c->active = mc_level_made(w) ? 1 : 0;
             cluster_sync();
         }
         mc_augment(w);
