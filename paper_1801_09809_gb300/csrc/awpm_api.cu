@@ -194,6 +194,16 @@ int small_mode()
     return v && v[0] == '0' && v[1] == 0 ? 0 : v && v[0] == '1' && v[1] == 0 ? 2 : 1;
 }
 
+// Whether greedy and maximum matching and the weights of small problems run in
+// one cluster (default on; the environment variable AWPM_CLUSTER=0, read when a
+// context is made, switches it off, a tuning knob: results are the same either
+// way).
+bool cluster_enabled()
+{
+    const char *v = getenv("AWPM_CLUSTER");
+    return !(v && v[0] == '0' && v[1] == 0);
+}
+
 int code_of(unsigned err)
 {
     return awpm_code_of_bits(err);
@@ -739,6 +749,7 @@ int setup_ctx(awpm_ctx *c, const awpm_options *opt)
     CUDA_TRY(small_setup());
     c->search_wide = default_search_wide();
     c->small_mode = small_mode();
+    c->clusters = cluster_enabled();
     for (int b = 0; b < 2; ++b)
         for (int p = 0; p < 2; ++p) {
             c->search_bps[b][0][p] = search_blocks_per_sm(AWPM_LOOKUP_BSEARCH, b == 1, p == 1);
@@ -1853,7 +1864,7 @@ int awpm_greedy(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *
     AWPM_TRY(ensure(c, c->ctl, sizeof(Ctl)));
     AWPM_TRY(ensure(c, c->wpart, sizeof(double) * kWsumBlocks));
     Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
-    sh.cluster = ntiles <= kGmClusterTiles;
+    sh.cluster = c->clusters && ntiles <= kGmClusterTiles;
     sh.greedy = true;
     // AWPM_FLAG_TIME_SEARCH: a host loop over the rounds (every kernel a
     // separate stream launch, visible to profilers) instead of the graph
@@ -1986,7 +1997,7 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
                                  c->stream));
     }
     Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
-    sh.cluster = ntiles <= kMcClusterTiles;
+    sh.cluster = c->clusters && ntiles <= kMcClusterTiles;
     CUDA_TRY(cudaEventRecord(c->ev_a, c->stream));
     Work &wk = *c->h_work;
     std::memset(&wk, 0, sizeof(Work));
@@ -2119,7 +2130,7 @@ static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const i
     if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!rowidx || !values || !weight_out)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
-    const bool small = ntiles <= kWtClusterTiles;
+    const bool small = c->clusters && ntiles <= kWtClusterTiles;
     thin = thin || ntiles <= kWtThinTiles;
     AWPM_TRY(ensure(c, c->wt_max, sizeof(unsigned long long) * n));
     if (!thin) {

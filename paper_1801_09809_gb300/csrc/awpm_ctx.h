@@ -137,6 +137,7 @@ struct awpm_ctx {
     awpm::DevBuf smallbuf, b_order;  // small matrices: bits of the entries, order
     uint32_t small_dense = 0;        // log2(n) classes whose single solves had too many entries
     int small_mode = 1;              // see small_mode()
+    bool clusters = true;            // see cluster_enabled()
     bool general_only = false;       // set while a small solve is repeated by the general path
     awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
     // The buffers that only a faster path needs (incbuf, smallbuf, b_order) are

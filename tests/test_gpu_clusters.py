@@ -64,20 +64,25 @@ def test_greedy(ctx, nnz, ties):
     assert st["cardinality"] == rst["cardinality"] and st["rounds"] == rst["rounds"]
 
 
+def emptied(nnz, seed):
+    """As sized(), with three columns empty."""
+    g = sized(nnz + 120, seed, True)
+    cp, col = g.colptr, np.repeat(np.arange(g.n), np.diff(g.colptr))
+    keep = np.ones(g.nnz, bool)
+    for j in (0, 5, g.n - 1):
+        keep[cp[j]:cp[j + 1]] = False
+    spare = np.nonzero(keep & (g.rowidx != g.mate[col]))[0]  # (the matched entries stay)
+    keep[np.random.default_rng(4).choice(spare, keep.sum() - nnz, replace=False)] = False
+    deg = np.bincount(col[keep], minlength=g.n)
+    colptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
+    return gen.Graph(g.n, colptr, g.rowidx[keep], g.weight[keep], g.mate, f"emptied({nnz})")
+
+
 @pytest.mark.parametrize("empty", [False, True])
-@pytest.mark.parametrize("nnz", [MCM - 31, MCM, MCM + 1])
-def test_mcm(ctx, nnz, empty):
-    g = sized(nnz, 9980, True)
-    if empty:
-        # the entries of three columns go to their right neighbours' end: the
-        # columns stay empty
-        cp = g.colptr.copy()
-        keep = np.ones(g.nnz, bool)
-        for j in (0, 5, g.n - 1):
-            keep[cp[j]:cp[j + 1]] = False
-        deg = np.add.reduceat(keep, cp[:-1]).astype(np.int32)
-        g.colptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.int32)
-        g.rowidx, g.weight = g.rowidx[keep], g.weight[keep]
+@pytest.mark.parametrize("nnz,clusters", [(MCM - 31, True), (MCM, True), (MCM + 1, False)])
+def test_mcm(ctx, nnz, clusters, empty):
+    g = emptied(nnz, 9980) if empty else sized(nnz, 9980, True)
+    assert (-(-g.nnz // 32) <= 6144) == clusters
     rng = np.random.default_rng(3)
     mate = np.where(rng.random(g.n) < 0.1, -1, g.mate).astype(np.int32)
     if empty:
@@ -86,7 +91,25 @@ def test_mcm(ctx, nnz, empty):
     got = mate.copy()
     st = awpm.awpm_mcm(ctx, g.n, g.colptr, g.rowidx, g.weight, got)
     assert np.array_equal(got, ref)
-    assert st["cardinality"] == int((ref >= 0).sum())
+    assert st["cardinality"] == int((ref >= 0).sum()) and st["phases"] == rst["phases"]
+
+
+@pytest.mark.parametrize("name", ["from_empty_and_from_greedy", "hand_tie_breaks", "bad_start",
+                                  "hand_cases_equal_weights", "small_and_ties", "structures",
+                                  "long_columns_and_equal_weights"])
+def test_graph_form(monkeypatch, name):
+    """The small problems of the maximum and the greedy matching's own tests, which
+    take the cluster by their size, through the graph's loops."""
+    import torch
+    import test_gpu_greedy
+    import test_gpu_mcm
+    monkeypatch.setenv("AWPM_CLUSTER", "0")
+    c = awpm.awpm_create(device=0)
+    try:
+        module = test_gpu_mcm if hasattr(test_gpu_mcm, "test_" + name) else test_gpu_greedy
+        getattr(module, "test_" + name)(c, torch)
+    finally:
+        awpm.awpm_destroy(c)
 
 
 NO_RETRIES = textwrap.dedent("""
