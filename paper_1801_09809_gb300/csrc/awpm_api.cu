@@ -1997,7 +1997,7 @@ int awpm_mcm(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const int32_t *row
                                  c->stream));
     }
     Shape sh = shape_of(c, false, AWPM_LOOKUP_BSEARCH, true, ntiles);
-    sh.cluster = c->clusters && ntiles <= kMcClusterTiles;
+    sh.cluster = c->clusters && mcm_cluster(ntiles, n);
     CUDA_TRY(cudaEventRecord(c->ev_a, c->stream));
     Work &wk = *c->h_work;
     std::memset(&wk, 0, sizeof(Work));
@@ -2130,8 +2130,8 @@ static int weights_once(awpm_ctx *ctx, int32_t n, const int32_t *colptr, const i
     if (nnz < 0 || nnz > kMaxEntries || (nnz > 0 && (!rowidx || !values || !weight_out)))
         return AWPM_ERR_INVALID_ARG;
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kTile - 1) / kTile);
-    const bool small = c->clusters && ntiles <= kWtClusterTiles;
-    thin = thin || ntiles <= kWtThinTiles;
+    const bool small = c->clusters && weights_cluster(ntiles, n);
+    thin = thin || small || weights_thin(ntiles, n);
     AWPM_TRY(ensure(c, c->wt_max, sizeof(unsigned long long) * n));
     if (!thin) {
         AWPM_TRY(ensure(c, c->wt_scale, sizeof(Scale) * n));

@@ -305,25 +305,6 @@ constexpr int kRsTile = kRsThreads * kRsItems;
 constexpr int kRsBins = 256;
 constexpr int kScanChunk = kRsThreads * 8;
 
-// Most tiles of a problem whose greedy rounds, and whose maximum-matching
-// phases, run in one cluster.  us per call, loops in the graph against one
-// cluster: greedy 16,000 entries 229 / 172, 64,000 248 / 184, 130,000 235 / 237,
-// 260,000 244 / 357 (random; the others alike); maximum matching 16,000 391 /
-// 289, 130,000 757 / 654, 260,000 1,009 / 1,040 (random), 622 / 520 (R-MAT).
-constexpr int32_t kGmClusterTiles = 3584;
-constexpr int32_t kMcClusterTiles = 6144;
-
-// Most tiles of a matrix whose weights one cluster computes, and of one that
-// takes the thin form (a warp per column, no scales and tile map to build, five
-// launches).  us per call, full / thin / cluster (and three warp-per-column
-// kernels on the FP64 units, the former form): random, 8 entries a column,
-// 8,000 entries 73 / 55 / 49 (57), 30,000 73 / 55 / 67 (69), 120,000
-// 71 / 55 / 161 (98), 250,000 76 / 67 / 296 (156), 1 M 96 / 108 / 1,049
-// (458); R-MAT 8,000 73 / 56 / 41 (69), 120,000 74 / 68 / 136 (191), 250,000
-// 75 / 87 / 235 (313); 27-point stencil 8,000 72 / 55 / 40 (56).
-constexpr int32_t kWtClusterTiles = 384;
-constexpr int32_t kWtThinTiles = 4096;
-
 // Launch shape of a context: fixed grids sized by the GPU, not the problem.
 struct Shape {
     int num_sms;

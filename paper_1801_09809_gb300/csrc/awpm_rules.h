@@ -25,6 +25,46 @@ AWPM_HD int32_t tile_pos(int32_t t, int32_t ntiles, int lane)
     return (t < ntiles ? t : ntiles) * kTile + lane;
 }
 
+// Most tiles of a problem whose greedy rounds run in one cluster (no column is
+// empty, so they bound n).  us per call, loops in the graph against one cluster:
+// 16,000 entries 229 / 172, 64,000 248 / 184, 130,000 235 / 237, 260,000 244 /
+// 357 (random; the others alike).
+constexpr int32_t kGmClusterTiles = 3584;
+
+// Whether the phases and levels of a maximum matching run in one cluster.  Each
+// phase walks all columns, which may be empty, 32 by 32, as its levels do the
+// tiles.  us per call, loops in the graph against one cluster: random, 8,000
+// columns and 100,000 entries 993 / 824, 16,000 and 190,000 1,106 / 1,067, 32,000
+// and 190,000 2,536 / 2,793, 65,536 and 100,000 1,353 / 1,458, 131,072 and 10,000
+// 292 / 289, 262,144 and 10,000 318 / 399, 4 M and 10,000 590 / 2,950.
+constexpr int64_t kMcClusterTiles = 6656;
+inline bool mcm_cluster(int32_t ntiles, int32_t n)
+{
+    return ntiles + (int64_t)n / 32 <= kMcClusterTiles;
+}
+
+// Forms of the weights: one cluster (a warp per column), the thin form (a warp
+// per column, no scales and tile map to build, five launches), the full one.  us
+// per call, full / thin / cluster (and three warp-per-column kernels on the FP64
+// units, the former form): random, 8 entries a column, 8,000 entries 73 / 55 / 49
+// (57), 30,000 73 / 55 / 67 (69), 120,000 71 / 55 / 161 (98), 250,000 76 / 67 /
+// 296 (156), 1 M 96 / 108 / 1,049 (458); R-MAT 8,000 73 / 56 / 41 (69), 120,000
+// 74 / 68 / 136 (191), 250,000 75 / 87 / 235 (313); 27-point stencil 8,000 72 /
+// 55 / 40 (56).  Mostly empty columns, thin / cluster: 8,000 columns and 1,000
+// entries 62 / 62, 32,000 and 1,000 62 / 98, 4,000 and 10,000 62 / 72, 4 M and
+// 1,000 433 / 6,494 (the former form 1,777); 100,000 entries thin, 190,000 full:
+// 131,072 columns 90, 92, 262,144 111, 92, 4 M 460, 222.
+constexpr int64_t kWtClusterTiles = 384;
+constexpr int32_t kWtThinTiles = 4096;
+inline bool weights_cluster(int32_t ntiles, int32_t n)
+{
+    return ntiles + (int64_t)n / 32 <= kWtClusterTiles;
+}
+inline bool weights_thin(int32_t ntiles, int32_t n)
+{
+    return ntiles <= kWtThinTiles && n / 32 <= kWtThinTiles;
+}
+
 // Solves of small matrices by one block each: classes of sizes (the largest
 // first) and the largest n of each.
 constexpr int kSmallClasses = 3;

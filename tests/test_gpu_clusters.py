@@ -14,7 +14,9 @@ import oracle
 from paper_1801_09809_gb300 import awpm, gen
 
 pytestmark = pytest.mark.gpu
-GREEDY, MCM = 3584 * 32, 6144 * 32  # most entries of a problem in one cluster
+# most entries of a problem of nnz / 6 columns in one cluster (the maximum
+# matching counts 32 columns as a tile of 32 entries)
+GREEDY, MCM = 3584 * 32, 182591
 
 
 @pytest.fixture(scope="module")
@@ -81,8 +83,9 @@ def emptied(nnz, seed):
 @pytest.mark.parametrize("empty", [False, True])
 @pytest.mark.parametrize("nnz,clusters", [(MCM - 31, True), (MCM, True), (MCM + 1, False)])
 def test_mcm(ctx, nnz, clusters, empty):
-    g = emptied(nnz, 9980) if empty else sized(nnz, 9980, True)
-    assert (-(-g.nnz // 32) <= 6144) == clusters
+    # (emptied() has 20 columns more for its entries)
+    g = emptied(nnz - (40 if clusters else 20), 9980) if empty else sized(nnz, 9980, True)
+    assert (-(-g.nnz // 32) + g.n // 32 <= 6656) == clusters
     rng = np.random.default_rng(3)
     mate = np.where(rng.random(g.n) < 0.1, -1, g.mate).astype(np.int32)
     if empty:
@@ -92,6 +95,27 @@ def test_mcm(ctx, nnz, clusters, empty):
     st = awpm.awpm_mcm(ctx, g.n, g.colptr, g.rowidx, g.weight, got)
     assert np.array_equal(got, ref)
     assert st["cardinality"] == int((ref >= 0).sum()) and st["phases"] == rst["phases"]
+
+
+@pytest.mark.parametrize("n,on", [(60000, "0"), (70000, "0"), (200000, "1"), (230000, "1")])
+def test_mcm_mostly_empty(monkeypatch, ctx, n, on):
+    """4,000 entries: n decides whether the graph's first level is one cluster's
+    (up to 65,567 columns), and between cluster and graph."""
+    monkeypatch.setenv("AWPM_CLUSTER", on)
+    rng = np.random.default_rng(n)
+    key = np.unique(rng.integers(0, n // 50, 4000) * 50 * n + rng.integers(0, 1500, 4000))
+    colptr = np.concatenate([[0], np.cumsum(np.bincount(key // n, minlength=n))]).astype(np.int32)
+    g = gen.Graph(n, colptr, (key % n).astype(np.int32),
+                  rng.integers(0, 4, key.size).astype(np.float64), None, "mostly empty")
+    start = np.full(n, -1, np.int32)
+    ref, rst = oracle.get().mcm(g, start)
+    got = start.copy()
+    c = awpm.awpm_create(device=0)
+    try:
+        st = awpm.awpm_mcm(c, n, g.colptr, g.rowidx, g.weight, got)
+    finally:
+        awpm.awpm_destroy(c)
+    assert np.array_equal(got, ref) and st["phases"] == rst["phases"]
 
 
 @pytest.mark.parametrize("name", ["from_empty_and_from_greedy", "hand_tie_breaks", "bad_start",

@@ -46,8 +46,10 @@ def reference(n, colptr, rowidx, a, mode):
         return np.log(x) if mode else x
 
 
-# sizes at the ends of the ranges of the three forms (tiles of 32 entries)
-SIZES = [384 * 32 + x for x in (-1, 0, 1, 32)] + [4096 * 32 + x for x in (-31, 0, 1)]
+# sizes at the ends of the ranges of the three forms (tiles of 32 entries, and
+# with nnz / 6 columns a sixth of their number for the columns in the first)
+SIZES = [384 * 32 + x for x in (-1, 0, 1, 32)] + [10559 + x for x in (-31, 0, 1)]
+SIZES += [4096 * 32 + x for x in (-31, 0, 1)]
 
 CASES = {
     "empty_columns": [0, 0, 3, 0, 31, 32, 33, 0, 1, 0, 0, 64, 65, 0, 0, 1] + [0, 1, 2] * 40,
@@ -115,6 +117,22 @@ def test_forms(ctx, nnz):
         cp, ri, av = (torch.from_numpy(x).cuda() for x in (c2, r2, a2))
         with pytest.raises(awpm.AwpmError):
             awpm.awpm_weights(ctx, n, cp, ri, av, 0, torch.empty_like(av))
+
+
+@pytest.mark.parametrize("n", [368 * 32 + 31, 369 * 32, 4096 * 32 + 31, 4097 * 32])
+def test_mostly_empty(ctx, n):
+    """500 entries (16 tiles) in so many columns that n decides the form."""
+    import torch
+    rng = np.random.default_rng(n)
+    key = np.unique(rng.integers(0, n * n, 500))
+    assert key.size == 500
+    colptr = np.concatenate([[0], np.cumsum(np.bincount(key // n, minlength=n))]).astype(np.int32)
+    rowidx, a = (key % n).astype(np.int32), rng.standard_normal(500)
+    want = reference(n, colptr, rowidx, a, 0)
+    cp, ri, av = (torch.from_numpy(x).cuda() for x in (colptr, rowidx, a))
+    out = torch.empty_like(av)
+    awpm.awpm_weights(ctx, n, cp, ri, av, 0, out)
+    assert np.array_equal(out.cpu().numpy(), want)
 
 
 @pytest.mark.parametrize("mode", [0, 1])

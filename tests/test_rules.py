@@ -54,3 +54,15 @@ def test_batches_by_work(rule):
     # empty matrices, and one class's largest n beside the next
     assert blocks((0, 0, 3)) and blocks((0, 0, 100), (20, 3, 1))
     assert not blocks((2048, 400, 4)) and blocks((2049, 400, 4)) and blocks((7169, 800, 4))
+
+
+def test_mostly_empty_matrices(rule):
+    """Columns count as well as entries where a form walks all of them: few
+    entries in millions of columns do not go to eight blocks."""
+    most = 2 ** 31 - 1
+    assert rule("mcm_cluster", 6000, 20000) and not rule("mcm_cluster", 6000, 32000)
+    assert rule("mcm_cluster", 32, 131072) and not rule("mcm_cluster", 32, 262144)
+    assert not rule("mcm_cluster", 1, most) and not rule("mcm_cluster", 67108862, most)
+    assert [rule("weights_form", 16, n) for n in (100, 11807, 11808, 131103, 131104, most)] == \
+        [0, 0, 1, 1, 2, 2]
+    assert [rule("weights_form", t, 1000) for t in (353, 354, 4096, 4097)] == [0, 1, 1, 2]
