@@ -173,13 +173,6 @@ int32_t inc_min_tiles()
     return least;
 }
 
-// Most entries of a single solve by the small-matrix kernel (one cluster of
-// eight blocks).  us per solve, by the kernel against the general path: random
-// n = 300 70 / 138, n = 2,000 with 18,000 entries 75 / 139, 72,000 entries 111
-// / 138, 180,000 entries 158 / 123; banded (19 passes) 4,400 entries 225 / 379,
-// 30,000 entries 423 / 491, 60,000 entries 581 / 500; 5-point 39,000 entries
-// 174 / 188; 27-point 22,000 entries 434 / 546, 51,000 entries 647 / 640.
-constexpr int32_t kSmallOneNnz = 40960;
 // Largest n tried without reading the number of entries first (a round trip
 // of about 10 us): above, an average column of 20 entries is too many.
 constexpr int32_t kSmallOneN = 2048;
@@ -1464,7 +1457,7 @@ int ctx_finish(awpm_ctx *c, awpm_stats *st, awpm_stats *per_matrix)
         // the general path names the error (or solves what was not for the
         // small-matrix kernel)
         Request again = pd.req;
-        if (again.count == 0 && pd.nnz < 0)
+        if (again.count == 0 && pd.nnz < 0 && small_too_many(h.small_nnz))
             c->small_dense |= 1u << ilog2(pd.n);
         const std::vector<int32_t> off = pd.n_off;
         if (again.off_host)

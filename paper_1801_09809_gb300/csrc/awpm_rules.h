@@ -76,6 +76,22 @@ inline int small_class(int32_t n)
     return n <= kSmallMaxN[2] ? 2 : n <= kSmallMaxN[1] ? 1 : 0;
 }
 
+// Most entries of a single solve by the small-matrix kernel (one cluster of
+// eight blocks).  us per solve, by the kernel against the general path: random
+// n = 300 70 / 138, n = 2,000 with 18,000 entries 75 / 139, 72,000 entries 111
+// / 138, 180,000 entries 158 / 123; banded (19 passes) 4,400 entries 225 / 379,
+// 30,000 entries 423 / 491, 60,000 entries 581 / 500; 5-point 39,000 entries
+// 174 / 188; 27-point 22,000 entries 434 / 546, 51,000 entries 647 / 640.
+constexpr int32_t kSmallOneNnz = 40960;
+
+// Whether a solve that came back undone from that kernel, which had read the
+// number of entries itself, had too many (and not an input to be refused): then
+// the next ones of its size have the number read first.
+inline bool small_too_many(int32_t nnz)
+{
+    return nnz > kSmallOneNnz;
+}
+
 // Whether a batch of small matrices is solved by a block per matrix, rather than
 // as a union over the whole GPU.  A block has one SM at most, so the call lasts
 // as long as its slowest matrix there, however idle the other SMs are; the union

@@ -755,14 +755,15 @@ __global__ void __cluster_dims__(kOneBlocks, 1, 1)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     const Work &w = *W;
-    if (gtid() == 0)
+    if (gtid() == 0) {
         small_reset(w);
+        w.ctl->small_nnz = w.small_nnz ? *w.small_nnz : w.nnz;
+    }
     // (the reset is ordered before every use by the solve's first barrier)
     solve_matrix<kSmallOne, kOneBlocks>(w, 0, s_raw);
     if (gtid() == 0 && !w.ctl->err) {
         w.ctl->weight_in = w.bw.mw_in[0];
         w.ctl->weight_out = w.bw.mw_out[0];
-        w.ctl->small_nnz = w.bw.mnnz[0];
     }
 }
 

@@ -22,7 +22,9 @@ int main(int argc, char **argv)
         for (int k = 2; k + 1 < argc; k += 2)
             load.add((int32_t)arg(k), arg(k + 1));
         std::printf("%d\n", load.blocks_pay() ? 1 : 0);
-    } else if (!std::strcmp(what, "mcm_cluster"))  // tiles, n
+    } else if (!std::strcmp(what, "small_too_many"))
+        std::printf("%d\n", small_too_many((int32_t)arg(2)) ? 1 : 0);
+    else if (!std::strcmp(what, "mcm_cluster"))  // tiles, n
         std::printf("%d\n", mcm_cluster((int32_t)arg(2), (int32_t)arg(3)) ? 1 : 0);
     else if (!std::strcmp(what, "weights_form"))  // tiles, n: 0 cluster, 1 thin, 2 full
         std::printf("%d\n", weights_cluster((int32_t)arg(2), (int32_t)arg(3)) ? 0

@@ -66,3 +66,9 @@ def test_mostly_empty_matrices(rule):
     assert [rule("weights_form", 16, n) for n in (100, 11807, 11808, 131103, 131104, most)] == \
         [0, 0, 1, 1, 2, 2]
     assert [rule("weights_form", t, 1000) for t in (353, 354, 4096, 4097)] == [0, 1, 1, 2]
+
+
+def test_small_solve_with_too_many_entries(rule):
+    """A solve of at most 40,960 entries that comes back undone was refused for
+    something else: its size class goes on without the number read first."""
+    assert [rule("small_too_many", z) for z in (0, 300, 40960, 40961, 2 ** 31 - 1)] == [0, 0, 0, 1, 1]
