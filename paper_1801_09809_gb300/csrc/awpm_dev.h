@@ -163,6 +163,28 @@ __device__ __forceinline__ bool rec_better(double g, int32_t p, double cg, int32
     return a > b || (a == b && p < cp);
 }
 
+// A 16-byte record read in one piece, from L2, as other threads' exchanges leave
+// it: two reads of eight bytes, or a vector load, which promises no more, may
+// see halves of two records.
+template <typename T>
+__device__ __forceinline__ T ld_record(const T *addr)
+{
+    static_assert(sizeof(T) == 16 && alignof(T) == 16, "one 128-bit access");
+    union {
+        unsigned long long h[2];
+        T rec;
+    } v;
+    asm volatile("{\n\t"
+                 ".reg .b128 t;\n\t"
+                 "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
+                 "mov.b128 {%0, %1}, t;\n\t"
+                 "}"
+                 : "=l"(v.h[0]), "=l"(v.h[1])
+                 : "l"(addr)
+                 : "memory");
+    return v.rec;
+}
+
 // Maximum of (g, lowest p) into a Step-C record.
 __device__ __forceinline__ void rec_combine(Rec *addr, Rec mine, Ctl *ctl)
 {
@@ -186,31 +208,11 @@ __device__ __forceinline__ bool sel_better(double g, int32_t j, double cg, int32
     return a > b || (a == b && j < cj);
 }
 
-// A Step-D selection read in one piece: its gain is only meaningful together
-// with its epoch.
-__device__ __forceinline__ Sel ld_sel(const Sel *addr)
-{
-    unsigned long long a, b;
-    asm volatile("{\n\t"
-                 ".reg .b128 t;\n\t"
-                 "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
-                 "mov.b128 {%0, %1}, t;\n\t"
-                 "}"
-                 : "=l"(a), "=l"(b)
-                 : "l"(addr)
-                 : "memory");
-    Sel s;
-    s.g = __longlong_as_double((long long)a);
-    s.j = (int32_t)(uint32_t)b;
-    s.epoch = (int32_t)(uint32_t)(b >> 32);
-    return s;
-}
-
 // Maximum of (g, lowest root j) into a Step-D selection (a record of another
 // epoch counts as empty).
 __device__ __forceinline__ void sel_combine(Sel *addr, Sel mine, Ctl *ctl)
 {
-    Sel cur = ld_sel(addr);
+    Sel cur = ld_record(addr);
     for (int it = 0; it < kCasRetryCap; ++it) {
         if (cur.epoch == mine.epoch && !sel_better(mine.g, mine.j, cur.g, cur.j))
             return;

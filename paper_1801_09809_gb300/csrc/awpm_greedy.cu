@@ -37,24 +37,6 @@ constexpr int32_t kMatched = -1;
 // of its tiles are dead (no free entry left; none ever comes back).
 constexpr int kGroup = 8;
 
-__device__ __forceinline__ Off ld_rec(const Off *addr)
-{
-    unsigned long long a, b;
-    asm volatile("{\n\t"
-                 ".reg .b128 t;\n\t"
-                 "ld.relaxed.gpu.global.b128 t, [%2];\n\t"
-                 "mov.b128 {%0, %1}, t;\n\t"
-                 "}"
-                 : "=l"(a), "=l"(b)
-                 : "l"(addr)
-                 : "memory");
-    Off o;
-    o.key = (long long)a;
-    o.who = (int32_t)(uint32_t)b;
-    o.pad = (int32_t)(uint32_t)(b >> 32);
-    return o;
-}
-
 // Fold (key, who) of this round into the record at addr, last seen as cur:
 // the larger key, then the lower index (128-bit compare-and-swap; a failed
 // exchange means another thread stored a better record, so the loop is short;
@@ -164,7 +146,7 @@ __device__ __forceinline__ void gm_best(const Work &w)
             for (int u = 0; u < kU; ++u) {
                 cur[u] = Off{0, 0, kMatched};
                 if (r[u] >= 0)
-                    cur[u] = ld_rec(w.grow + r[u]);
+                    cur[u] = ld_record(w.grow + r[u]);
             }
 #pragma unroll
             for (int u = 0; u < kU; ++u) {
@@ -208,7 +190,7 @@ __device__ __forceinline__ void gm_best(const Work &w)
                     if (segment_complete(mk[u], lane, base, nnz, w.starts, tg + h + u))
                         *c = Off{k, base + at, round};
                     else
-                        rec_fold(c, ld_rec(c), k, base + at, round, ctl);
+                        rec_fold(c, ld_record(c), k, base + at, round, ctl);
                 }
             }
         }

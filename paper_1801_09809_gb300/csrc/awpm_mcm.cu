@@ -297,18 +297,6 @@ __device__ __forceinline__ bool off_better(long long key, int32_t who, const Off
     return key > cur.key || (key == cur.key && who < cur.who);
 }
 
-// A record read from L2, where the other threads' exchanges land, so that
-// fewer exchanges start from a stale copy.
-__device__ __forceinline__ Off ld_off(const Off *addr)
-{
-    const int4 v = __ldcg(reinterpret_cast<const int4 *>(addr));
-    Off cur;
-    cur.key = (long long)(((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x);
-    cur.who = v.z;
-    cur.pad = v.w;
-    return cur;
-}
-
 // Fold (key, who) into the record at addr, last seen as cur (128-bit
 // compare-and-swap; a failed exchange means another thread stored a better
 // record, so the loop is short; its bound only turns a broken invariant into
@@ -405,7 +393,7 @@ __device__ __forceinline__ void mc_offer(const Work &w, int32_t *buf)
             cur[u] = Off{0, 0, 0};
             if (go[u]) {
                 key[u] = order_key(__ldg(w.w + (int64_t)t[u] * kTile + lane));
-                cur[u] = ld_off(w.mroff + r[u]);
+                cur[u] = ld_record(w.mroff + r[u]);
             }
             // the tile leaves the list (its next listing is by the advance)
             if (lane == 0 && t[u] >= 0)
@@ -444,7 +432,7 @@ __device__ __forceinline__ void mc_join(const Work &w)
     const int32_t touched = w.ctl->touched;
     for (int64_t x = first; x < touched; x += step) {
         const int32_t r = w.mtouch[x];
-        const Off o = ld_off(w.mroff + r);
+        const Off o = ld_record(w.mroff + r);
         const int32_t c = o.who;
         const int32_t c2 = w.mr[r];
         const int32_t t_root = w.mroot[c];
@@ -453,7 +441,7 @@ __device__ __forceinline__ void mc_join(const Work &w)
         atomicOr(w.mreach + (r >> 5), 1u << (r & 31));
         w.mtouch[x] = c2;
         if (c2 < 0)
-            off_combine(w.mtend + t_root, ld_off(w.mtend + t_root), o.key, r, w.ctl);
+            off_combine(w.mtend + t_root, ld_record(w.mtend + t_root), o.key, r, w.ctl);
         else
             w.mroot[c2] = t_root;
     }
@@ -479,7 +467,7 @@ __device__ __forceinline__ void mc_advance(const Work &w)
             root[u] = c[u] >= 0 ? w.mroot[c[u]] : -1;
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
-            if (root[u] >= 0 && ld_off(w.mtend + root[u]).who != 0x7fffffff)
+            if (root[u] >= 0 && ld_record(w.mtend + root[u]).who != 0x7fffffff)
                 c[u] = -1;
             if (c[u] >= 0)
                 atomicOr(w.mfront + (c[u] >> 5), 1u << (c[u] & 31));

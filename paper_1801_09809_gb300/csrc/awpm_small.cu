@@ -602,7 +602,7 @@ __device__ void solve_matrix(const Work &w, int32_t b, unsigned char *smem)
         solve_sync<kC>();
         // the flip (see flip_body for the records that stand)
         auto selected = [&](int32_t key, int32_t j) {
-            const Sel s = ld_sel(w.dsel + o + key);
+            const Sel s = ld_record(w.dsel + o + key);
             return s.epoch == epoch && s.j == j;
         };
         // in every block's copy
