@@ -1189,6 +1189,7 @@ int enqueue_once(awpm_ctx *c, const Request &r)
     wk.colsig = (unsigned long long *)c->colsig.p;
     wk.htab = lookup == AWPM_LOOKUP_HASH ? (unsigned long long *)c->htab.p : nullptr;
     wk.bloom = lookup == AWPM_LOOKUP_BSEARCH && bloom_enabled() ? (uint32_t *)c->bloom.p : nullptr;
+    wk.bloom_min = wk.bloom ? bloom_min(n, nnz) : kNoBloom;
     if (lookup == AWPM_LOOKUP_ROWMARK) {
         wk.rowsig = (unsigned long long *)c->rowsig.p;
         wk.trowptr = (int32_t *)c->trowptr.p;

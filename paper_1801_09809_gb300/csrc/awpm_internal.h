@@ -191,7 +191,7 @@ struct Work {
     int32_t inc;        // passes after the first search only what the last flips affect
     int32_t epoch0;     // Step-D records of this solve's passes: epochs epoch0 + 1, ...
     int32_t map_bits;   // bits of the large folded bitmap (0: none kept)
-    int32_t inc_pad;
+    int32_t bloom_min;  // columns with more rows than this have a Bloom filter
     const int32_t *colptr;
     const int32_t *rowidx;
     const double *w;
@@ -323,6 +323,11 @@ struct Shape {
 
 constexpr int kWsumBlocks = 1024;
 constexpr int kWsumThreads = 256;
+
+// Rows above which a column has a Bloom filter, by the matrix's size, and the
+// value that gives none to any.
+int32_t bloom_min(int32_t n, int32_t nnz);
+constexpr int32_t kNoBloom = 0x7fffffff;
 
 // Where launches go: a stream (launched at once, asynchronously) or a graph
 // (appended as kernel nodes, each depending on the previous one).  Graphs are

@@ -121,19 +121,28 @@ __device__ __forceinline__ int32_t slot_start(int32_t r, int32_t base, int32_t s
 }
 
 // ---- blocked Bloom filters of long columns (binary-search lookup) -------------
-// A column with more than kBloomMin rows, stored at positions [s, e), owns the
-// words [s/4, (e-1)/4] of the bloom array: one 32-bit word per 4 nonzeros (a
+// A column with more than Work::bloom_min rows, stored at positions [s, e), owns
+// the words [s/4, (e-1)/4] of the bloom array: one 32-bit word per 4 nonzeros (a
 // word at a boundary may be shared with the neighbouring column, which only
 // adds false positives).  Each row sets three bits of one word, word and bits
 // picked by a hash of the row; a row with a clear bit is not in the column.
 // Long columns are where the 64-bit signature fills up, so this filter keeps
 // most of their absent closing entries away from the search.
 
-// The line: a filter entry costs the entry pass an atomic (135 of 387 us on
-// the R-MAT graph of scale 22 from 32 rows up), and only the first pass's
-// lookups use many of them.  Whole solves of that graph: 1.447 ms from 32 rows
-// up, 1.435 from 64, 1.439 from 128, 1.53 from 512.
-constexpr int32_t kBloomMin = 64;
+// Rows above which a column has a Bloom filter (binary-search lookup).  A filter
+// entry costs the entry pass an atomic (135 of 387 us on the R-MAT graph of scale
+// 22 from 32 rows up), and only the first pass's lookups use many of them.
+// Whole solves of that graph: 1.447 ms from 32 rows up, 1.435 from 64, 1.439 from
+// 128, 1.53 from 512.  Where the average column is that long the lookups are the
+// larger part: from 64 and from 32 rows up, random with 55 entries a column, n =
+// 400,000: a search 453 / 411 us, a solve 607 / 557; with 41, n = 1 M, 724 / 660
+// and 854 / 793; with 37, n = 600,000, 395 / 376 and 484 / 469; against that,
+// banded with 41, n = 500,000, 639 / 669 and 7,183 / 7,333.
+constexpr int32_t kBloomMin = 64, kBloomMinLong = 32;
+int32_t bloom_min(int32_t n, int32_t nnz)
+{
+    return nnz / 40 >= n ? kBloomMinLong : kBloomMin;
+}
 
 __device__ __forceinline__ void bloom_key(int32_t r, int32_t s, int32_t e, uint32_t &word,
                                           uint32_t &bits)
@@ -493,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_entries(const Work *__restrict_
                     const bool head = !(inner & ((2u << u) - 1u));
                     const bool tail = !(inner >> (u + 1));
                     const int32_t s = head ? s0 : s3, e = head ? e0 : e3;
-                    if ((head || tail) && e - s > kBloomMin) {
+                    if ((head || tail) && e - s > w.bloom_min) {
                         uint32_t word_b, b;
                         bloom_key(r[u], s, e, word_b, b);
                         atomicOr(w.bloom + word_b, b);
@@ -1297,7 +1306,7 @@ __device__ __forceinline__ unsigned resolve_inline(const Work *__restrict__ W, c
                 q = v;
         }
     } else {
-        if (w.bloom && len > kBloomMin) {
+        if (len > w.bloom_min) {
             // long column: its Bloom filter rules most absent rows out first
             uint32_t word, b;
             bloom_key(mj, lo, lo + len, word, b);

@@ -151,6 +151,7 @@ extern "C" int awpm_search_noalloc(int32_t n, const int32_t *colptr, const int32
     wk.max_passes = 1;
     wk.lookup = AWPM_LOOKUP_BSEARCH;
     wk.htab = nullptr;
+    wk.bloom_min = kNoBloom;
     wk.colptr = colptr;
     wk.rowidx = rowidx;
     wk.w = weight;

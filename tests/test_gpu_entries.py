@@ -127,3 +127,27 @@ def test_errors_anywhere(ctx, torch):
             r[p] = r[p - 1]
             assert code(r, g.weight) == "UNSORTED_OR_DUP", p
     assert code(g.rowidx, g.weight) == "OK"
+
+
+@pytest.mark.parametrize("mean", [39, 40])
+def test_filters_of_ordinary_columns(torch, mean):
+    """Columns of 31 to 66 rows (and one of 1,000) on both sides of the average from which columns
+    of more than 32 rows have a Bloom filter, a search and a whole solve."""
+    rng = np.random.default_rng(mean)
+    d = rng.choice([31, 32, 33, 34, 45, 64, 65, 66], 1400, p=[.3, .2, .2, .1, .05, .05, .05, .05])
+    d[:1300] += (mean * 1400 - d.sum()) // 1300
+    d[-1] += mean * 1400 - d.sum()
+    g = shaped(list(d), 9991)
+    assert g.nnz == mean * g.n and g.nnz > 40960
+    ref, rst, _ = oracle.get().improve(g)
+    c = awpm.awpm_create(device=0, lookup=awpm.LOOKUP_BSEARCH)
+    try:
+        out = np.empty(g.n, np.int32)
+        st = awpm.awpm_improve_ctx(c, g.n, g.colptr, g.rowidx, g.weight, g.mate, out)
+        assert_same_as_oracle(g, out, st, ref, rst)
+        gain, row = np.empty(g.n), np.empty(g.n, np.int32)
+        awpm.awpm_search(c, g.n, g.colptr, g.rowidx, g.weight, g.mate, gain, row)
+        want_gain, want_row, _ = oracle.get().step_c(g)
+        assert np.array_equal(gain, want_gain) and np.array_equal(row, want_row)
+    finally:
+        awpm.awpm_destroy(c)
