@@ -1028,8 +1028,8 @@ int enqueue_once(awpm_ctx *c, const Request &r)
         l_row < 0 || l_off < 0)
         return AWPM_ERR_INVALID_ARG;
 
-    // Small matrices: a block each, in one kernel.  A single one does not even
-    // have its nnz read back first.
+    // Small matrices: a block each of a batch, where that pays, or one cluster
+    // for a single one, which does not even have its nnz read back first.
     const bool small = c->small_mode && !c->general_only && !c->least_memory && !r.search_only &&
                        !(c->opt.flags & AWPM_FLAG_TIME_SEARCH) &&
                        c->opt.select == AWPM_SELECT_STEP_D &&
