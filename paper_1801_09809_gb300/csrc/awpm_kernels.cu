@@ -2202,11 +2202,14 @@ __device__ __forceinline__ void mark_column(const Work &w, int set, int32_t j, i
 // when k is flipped: as the key of the winner selected there (j lost to it),
 // or as the root of the winner that dropped j, if that one was selected.
 // (The greedy selection drops a winner only for sharing a column with a kept
-// cycle, so all its winners' records go.)  Without incremental passes (kInc
-// false) none of that code is there: a flip is short, and fetching its code is
-// part of it (R-MAT, 20,000 columns, 8 passes: 276 us per solve with one kernel
-// for both, 271 so).
-template <bool kInc>
+// cycle, so all its winners' records go.)  In the graph form of a single
+// problem's pass kInc says which passes these are, and a flip without
+// incremental passes holds none of their code: with few winners it is short, and
+// fetching its code is part of it (R-MAT, 20,000 columns, 8 passes: 276 us per
+// solve with one kernel for both, 271 so).  -1 asks the descriptor: a batch's
+// union, with many winners, takes 6.4 ms so and 7.0 without that code (1,024
+// matrices of 200 to 20,000 columns).
+template <int kInc>
 __device__ __forceinline__ unsigned long long flip_body(const Work &w)
 {
     unsigned long long flips = 0;
@@ -2216,7 +2219,8 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
         const int64_t nwarps = gstride() >> 5;
         const int per = few_winners(w, nwarps) ? 32 : words_per_warp(words, nwarps);
         const int32_t epoch = pass_epoch(w);
-        const int set = kInc ? w.ctl->iterations & 1 : 0;
+        const bool inc = kInc < 0 ? w.inc != 0 : kInc != 0;
+        const int set = inc ? w.ctl->iterations & 1 : 0;
         auto selected = [&](int32_t key, int32_t j) {
             const Sel sl = w.dsel[key];
             return sl.epoch == epoch && sl.j == j;
@@ -2232,7 +2236,7 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
                     if (k >= 0 && AWPM_IN(w.ctl, k, w.n) && AWPM_IN(w.ctl, r.p, w.nnz) &&
                         AWPM_IN(w.ctl, r.q, w.nnz)) {
                         sel = selected(k, j);
-                    } else if (kInc && !w.psel && key < 0 && AWPM_IN(w.ctl, ~key, w.n)) {
+                    } else if (inc && !w.psel && key < 0 && AWPM_IN(w.ctl, ~key, w.n)) {
                         const int32_t k2 = w.wkey[~key];
                         stands = k2 < 0 || !AWPM_IN(w.ctl, k2, w.n) || !selected(k2, ~key);
                     }
@@ -2240,7 +2244,7 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
                         atomicOr(w.winbits + (j >> 5), 1u << (j & 31));
                     } else {
                         w.best[j] = Rec{0.0, 0, 0};
-                        if (kInc && !sel) {
+                        if (inc && !sel) {
                             atomicOr(w.colpos[set] + (j >> 5), 1u << (j & 31));
                             mark_tiles(w, set, w.colptr[j], w.colptr[j + 1]);
                         }
@@ -2264,7 +2268,7 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
                             ++flips;
                             if (w.bw.count > 0)
                                 mat = w.bw.colmat[k];
-                            if (kInc) {
+                            if (inc) {
                                 mark_row(w, set, i);
                                 mark_row(w, set, mj);
                                 mark_column(w, set, j, mj, js, je);
@@ -2282,17 +2286,16 @@ __device__ __forceinline__ unsigned long long flip_body(const Work &w)
             });
         }
         // the set of bitmaps that this pass's search read, for the next flips
-        if (kInc && w.ctl->iterations > 0)
+        if (inc && w.ctl->iterations > 0)
             inc_clear(w, set ^ 1);
     }
     return flips;
 }
 
-template <bool kInc>
 __global__ void k_flip(const Work *__restrict__ W)
 {
     const Work &w = *W;
-    block_add_u64(flip_body<kInc>(w), &w.ctl->pass_flips);
+    block_add_u64(flip_body<-1>(w), &w.ctl->pass_flips);
 }
 
 __global__ void k_control(const Work *__restrict__ W)
@@ -2308,7 +2311,7 @@ __global__ void k_control_graph(const Work *__restrict__ W, cudaGraphConditional
 // The flip in the graph form of a single problem's pass: the block that
 // finishes last (its count of finished blocks orders it after every other
 // block's flip count) ends the pass and sets the WHILE condition.
-template <bool kInc>
+template <int kInc>
 __global__ void k_flip_graph(const Work *__restrict__ W, cudaGraphConditionalHandle h)
 {
     const Work &w = *W;
@@ -2319,7 +2322,7 @@ __global__ void k_flip_graph(const Work *__restrict__ W, cudaGraphConditionalHan
         if (prev == gridDim.x - 1) {
             __threadfence();
             w.ctl->flip_done = 0u;
-            cudaGraphSetConditional(h, control_step(w.ctl, kInc) ? 1u : 0u);
+            cudaGraphSetConditional(h, control_step(w.ctl, kInc != 0) ? 1u : 0u);
         }
     }
 }
@@ -2915,16 +2918,11 @@ void launch_greedy_select_round(const Work *d, const Shape &sh, bool graph,
         k.launch((const void *)k_ps_cond, 1, 1, ah);
 }
 
-static inline const void *flip_fn(const Shape &sh)
-{
-    return sh.inc ? (const void *)k_flip<true> : (const void *)k_flip<false>;
-}
-
 void launch_greedy_select_end_and_flip(const Work *d, const Shape &sh, Sink &k)
 {
     void *a[] = {(void *)&d};
     k.launch((const void *)k_ps_end, tile_grid(sh), kThreads, a);
-    k.launch(flip_fn(sh), tile_grid(sh), kThreads, a);
+    k.launch((const void *)k_flip, tile_grid(sh), kThreads, a);
 }
 
 // Step D's kernels take 32 words of the winner bitmap per warp; a single
@@ -2944,7 +2942,7 @@ void launch_select_flip_control_graph(const Work *d, const Shape &sh,
     void *a[] = {(void *)&d};
     void *ah[] = {(void *)&d, (void *)&h};
     k.launch((const void *)k_select, winner_grid(sh), kThreads, a);
-    k.launch(sh.inc ? (const void *)k_flip_graph<true> : (const void *)k_flip_graph<false>,
+    k.launch(sh.inc ? (const void *)k_flip_graph<1> : (const void *)k_flip_graph<0>,
              winner_grid(sh), kThreads, ah);
 }
 
@@ -2952,7 +2950,7 @@ void launch_select_and_flip(const Work *d, const Shape &sh, Sink &k)
 {
     void *a[] = {(void *)&d};
     k.launch((const void *)k_select, winner_grid(sh), kThreads, a);
-    k.launch(flip_fn(sh), winner_grid(sh), kThreads, a);
+    k.launch((const void *)k_flip, winner_grid(sh), kThreads, a);
 }
 
 void launch_control(const Work *d, const Shape &sh, bool graph, cudaGraphConditionalHandle h,
