@@ -983,6 +983,7 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
 {
     NvtxRange nvtx_range("enqueue");
     c->spares_used = false;
+    c->union_tiles = 0;
     int rc = enqueue_once(c, r);
     const bool no_room = rc == AWPM_ERR_BUDGET || (rc == AWPM_ERR_OOM && !c->injected);
     if (no_room && c->spares_used) {
@@ -994,6 +995,15 @@ int ctx_enqueue(awpm_ctx *c, const Request &r)
         c->least_memory = true;
         rc = enqueue_once(c, r);
         c->least_memory = false;
+    } else if (no_room && c->union_tiles > 0) {
+        // a batch that would be the faster as a union: the blocks need less
+        const int64_t tiles = c->union_tiles;
+        ctx_trim(c);
+        if (rc == AWPM_ERR_BUDGET && (c->union_full == 0 || tiles < c->union_full))
+            c->union_full = tiles;
+        c->force_blocks = true;
+        rc = enqueue_once(c, r);
+        c->force_blocks = false;
     }
     return rc;
 }
@@ -1051,7 +1061,9 @@ int enqueue_once(awpm_ctx *c, const Request &r)
     if (small_batch) {
         BatchLoad load;
         AWPM_TRY(read_batch(c, r, l_colptr, l_off, &nnz, &load));
-        blocks = c->small_mode == 2 || load.blocks_pay();
+        blocks = c->small_mode == 2 || c->force_blocks || load.blocks_pay() ||
+                 (c->union_full > 0 && load.all >= c->union_full);
+        c->union_tiles = blocks ? 0 : load.all;
     }
     if (nnz < 0 && !small_batch) {
         if (l_colptr == 1) {
@@ -1675,7 +1687,7 @@ static int solve_sync(awpm_ctx *c, const Request &r, awpm_stats *st, awpm_stats 
         if (rc == AWPM_OK)
             return ctx_finish(c, st, per_matrix);
     } catch (const std::bad_alloc &) {  // (host memory: offsets and order of a batch)
-        c->general_only = false;
+        c->general_only = c->force_blocks = c->least_memory = false;
         rc = AWPM_ERR_OOM;
     }
     if (c->stream)

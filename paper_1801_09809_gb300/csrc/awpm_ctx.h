@@ -138,6 +138,11 @@ struct awpm_ctx {
     uint32_t small_dense = 0;        // log2(n) classes whose single solves had too many entries
     int small_mode = 1;              // see small_mode()
     bool clusters = true;            // see cluster_enabled()
+    // a batch that the rule makes a union, while it is enqueued: its tiles; the
+    // fewest of one that the budget had no room for; set while such a batch is
+    // enqueued again as blocks
+    int64_t union_tiles = 0, union_full = 0;
+    bool force_blocks = false;
     bool general_only = false;       // set while a small solve is repeated by the general path
     awpm::DevBuf incbuf;  // incremental passes: entry bits, row and column bitmaps
     // The buffers that only a faster path needs (incbuf, smallbuf, b_order) are

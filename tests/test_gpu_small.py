@@ -130,6 +130,33 @@ def test_pass_cap(torch):
         awpm.awpm_destroy(c)
 
 
+def test_budget_for_blocks_only(torch, monkeypatch):
+    """A batch that the rule makes a union, under a budget with room for the blocks
+    only, is solved by them, within the budget."""
+    graphs = [gen.banded(7000 + k, 9, 9980 + k) for k in range(4)]
+
+    def context(small, budget):
+        monkeypatch.setenv("AWPM_SMALL", small)
+        return awpm.awpm_create(device=0, mem_budget_bytes=budget)
+
+    c = context("1", 0)
+    batch_check(c, torch, graphs)
+    budget = awpm.awpm_memory_held(c)[1]
+    awpm.awpm_destroy(c)
+    c = context("0", budget)
+    with pytest.raises(awpm.AwpmError) as e:
+        batch_check(c, torch, graphs)
+    assert e.value.name == "BUDGET"
+    awpm.awpm_destroy(c)
+    c = context("", budget)
+    try:
+        used = batch_check(c, torch, graphs, times=4)
+        assert used == [awpm.LOOKUP_BSEARCH] * 4
+        assert awpm.awpm_memory_held(c)[1] <= budget
+    finally:
+        awpm.awpm_destroy(c)
+
+
 @pytest.mark.parametrize("make", [
     lambda: gen.random_small(1, 1.0, 1), lambda: gen.random_small(33, 0.5, 2, integer_weights=True),
     lambda: gen.banded(2048, 15, 3), lambda: gen.banded(2049, 15, 4), lambda: gen.stencil_2d(90, 5),
